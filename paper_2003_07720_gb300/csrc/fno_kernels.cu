@@ -60,6 +60,8 @@ constexpr int kOffQ = kNeP;
 constexpr int kNeA = W * W + W;                  // (A, a)
 constexpr int kNeQ = NH * W + NH;                // (Q, q): 612
 constexpr int kNeHead = kNeQ + 1;                // + squared-error sum
+// floats of a partial row: the largest of the gradient kernels' rows
+constexpr int kPartRow = std::max(kNeHead, std::max(kNeA, kNeP));
 static_assert(kOffQ + kNeQ <= kHeader, "head parameters overflow the header");
 
 size_t r_floats(int m) { return (size_t)2 * (2 * m * m) * (2 * m) * W * W; }
@@ -1685,7 +1687,7 @@ rpm_status rpm_fno_create(const rpm_fno_config* cfg, void* cuda_stream, rpm_fno*
   const size_t act = f->act_floats() * sizeof(float);
   const size_t colb = (size_t)B * N * f->ncol * W * sizeof(float2);
   const size_t vsb = (size_t)L * f->ncol * B * 2 * m * W * sizeof(float2);
-  const size_t partb = (size_t)kPwBlocksMax * kNeA * sizeof(float);   // largest row
+  const size_t partb = (size_t)kPwBlocksMax * kPartRow * sizeof(float);
   const bool ok =
       alloc((void**)&f->params, P) && alloc((void**)&f->grads, P) &&
       alloc((void**)&f->adam1, P) && alloc((void**)&f->adam2, P) &&

@@ -100,6 +100,32 @@ def test_loss_and_every_gradient_match_oracle(fno):
         assert rel < GRAD_TOL, (k, rel)
 
 
+def test_gradients_with_a_full_grid_of_partial_rows(fno):
+    """Enough voxels that the head kernel runs its largest grid: every block's
+    partial row (613 floats, the widest of the gradient kernels) has its own
+    place in the workspace, so nothing behind it is overwritten."""
+    N, m, L, B = 40, 3, 1, 4
+    p = _round32(_params(m, L, 8))
+    feat, E = _inputs(N, B, 6)
+    rng = np.random.Generator(np.random.PCG64(9))
+    target = rng.standard_normal((B, 6, N, N, N)).astype(np.float32).astype(np.float64)
+    E = E.astype(np.float32).astype(np.float64)
+    loss_ref, g_ref = fo.backward(p, feat, E, target, m, L)
+    with fno.Fno(N, m, L, max_batch=B, precision="fp32") as net:
+        act = 4 * N ** 3 * 16 * B
+        col = 8 * 2 * m * m * 16 * B
+        other = (4 * 4 * net.nparam + (2 * L + 3) * act + (2 * N + 2 * m * L) * col + 8 * N + 64 +
+                 24 * B + 4 * N ** 3 * (2 + 6 + 6) + 8 * 256)
+        assert net.device_bytes() - other >= 4 * 152 * 613 * 4
+        net.set_params(p)
+        loss = net.loss_grad(_dev(feat), E, _dev(target))
+        g = fno.unpack_params(net.get_grads(), m, L)
+    assert abs(loss - loss_ref) <= 1e-5 * loss_ref
+    for k in g_ref:
+        rel = np.linalg.norm(g[k] - g_ref[k]) / np.linalg.norm(g_ref[k])
+        assert rel < GRAD_TOL, (k, rel)
+
+
 def test_adam_step_matches_definition(fno):
     N, m, L, B = 24, 3, 1, 1
     p = _params(m, L, 11)
