@@ -88,7 +88,7 @@ def recorded_traffic(key: str):
     if not rec:
         return None
     h = hashlib.sha256()
-    for f in ("gamma_kernels.cu", "fft_smem.cuh"):
+    for f in ("gamma_kernels.cu", "fft_smem.cuh", "gamma_pair.cu", "pair_fft.cuh"):
         with open(os.path.join(ROOT, "paper_2003_07720_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return rec["dram_bytes_per_launch"] if h.hexdigest()[:16] == rec["source_sha256_16"] else None

@@ -94,13 +94,14 @@ typedef struct {
                             z-pass variants below on the context's grid and keeps the
                             fastest (rpm_set_options then keeps that choice while
                             autotune stays 1); 0 (default): the variants below */
-  int plane_variant;     /* x/y passes: 0 (default) the fused plane kernels where the
+  int plane_variant;     /* x/y passes: 0 (default) the paired plane kernels where the
                             grid has them (square planes 48-128), else as 1; 1 the
                             whole-plane kernels where the plane fits (nx = ny <= 128),
                             else as 2; 2 the five-pass row and y-pencil kernels */
-  int pencil_variant;    /* z pass: 0 (default) the fused register-resident kernel where
-                            the grid has it (nz 32, 48, 96, 128), else the default tile; 1 half,
-                            2 twice the default pencils per block; 3 the default tile */
+  int pencil_variant;    /* z pass: 0 (default) the default tile (with the paired plane
+                            kernels their own z pass; otherwise the register-resident kernel
+                            where the grid has it, nz 32, 48, 96, 128); 1 half, 2 twice the
+                            default pencils per block; 3 the default tile */
   int share_basis;       /* 1: a solve starts from the unstable basis (Z, W = F_u Z, H)
                             that an earlier solve of the same map left in the context --
                             F_u does not depend on the load E, so the six loads of
@@ -301,7 +302,7 @@ const char* rpm_status_string(rpm_status s);
  * options.autotune was set at creation); 0 for a null context. */
 int rpm_pencil_tile(const rpm_ctx* ctx);
 
-/* Plane-pass kernels in use: 0 fused, 1 whole-plane, 2 five-pass (the
+/* Plane-pass kernels in use: 0 paired, 1 whole-plane, 2 five-pass (the
  * autotuner's choice when options.autotune was set at creation); -1 for a
  * null context. */
 int rpm_plane_variant(const rpm_ctx* ctx);

@@ -118,7 +118,7 @@ __device__ __forceinline__ void allow_dependent_launch() {
 // cluster arrives (release) and waits (acquire), so shared-memory writes
 // before it are visible to the other blocks after it; all threads of a block
 // must execute it.  cluster_map: the address of `p` in the shared memory of
-// the cluster's block `rank`; ld_cluster_f2 reads through such an address.
+// the cluster's block `rank`; ld_cluster_f2 / _f4 read through such an address.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
@@ -134,6 +134,14 @@ __device__ __forceinline__ uint32_t cluster_map(const void* p, uint32_t rank) {
 __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
   float2 v;
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+  return v;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr));
   return v;
 }
 

@@ -12,15 +12,11 @@
 //   pass C (one block per z-plane and component): inverse FFT along y,
 //       complex-to-real tangling, inverse FFT along x of length nx/2, scale.
 //
-// Two generations of kernels implement the passes.  The fused ones
-// (k_plane_fwd, k_pencil_green, k_plane_inv) serve the common sizes: their
-// first and last register FFT steps read and write global memory directly
-// (pass C takes its plane in one bulk asynchronous copy), the (un)tangling
-// of the half-length x transform is fused into an x step, the real DC and
-// Nyquist x columns travel as one complex column so that the y transforms
-// run on exactly nx/2 columns, and in pass B the forward z step 2, the
-// Green operator and the inverse z step 1 run in registers.  The original
-// kernels (k_pass_a/b/c and the five-pass variant) serve the other sizes.
+// Square planes nx = ny in {48, 64, 96, 128} run the paired kernels of
+// gamma_pair.cu.  The kernels here serve the other sizes (and the forced
+// variants): k_pass_a/b/c, the z pass k_pencil_green, in which the forward z
+// step 2, the Green operator and the inverse z step 1 run in registers, and
+// the five-pass variant for planes that do not fit in shared memory.
 //
 // The Green operator of the isotropic reference medium is evaluated on the
 // fly from the unit wave vector n = xi/|xi|:
@@ -211,12 +207,6 @@ __global__ void __launch_bounds__(kPlaneThreads, kPlaneMinBlocks)
     out2[idx] = cscale(P[h * C::NYP + y], scale);
   }
 }
-
-struct GammaArgs {
-  float En[6];       // E * n_vox (zero frequency of the strain in GM_FULL_MAP)
-  float a;           // (lam0 + mu0) / (lam0 + 2 mu0)
-  float inv_mu0;
-};
 
 // T consecutive (ky, kx) pencils per pass-B block: TT = 0 takes the default
 // for the length (8 pencils = 64-byte rows at nz = 64 and 128; 16 at
@@ -421,11 +411,6 @@ __global__ void __launch_bounds__(2 * kThreads, 2) k_pass_b_wide(GridDev g,
 }
 
 
-// ---------------------------------------------------------------------------
-// Fused-step kernels (square planes nx = ny in {48, 64, 96, 128}; pencils of
-// length nz with 128 / split_n1(nz) pencils per block, nz in {32, 48, 96, 128}).
-// ---------------------------------------------------------------------------
-
 // Row task q of an x step over NY rows: (y, n2).  With N2 = 8 the two
 // half-warps take rows y and y + 8, so that the 8-byte accesses of one
 // instruction fall in distinct banks (row stride nx/2 + 1 float2).
@@ -439,488 +424,6 @@ __device__ __forceinline__ void row_task(int q, int& y, int& n2) {
     n2 = q % N2;
     y = q / N2;
   }
-}
-
-// Pass A, one block per (z, component).  x step 1 reads the strain rows from
-// global memory and forms tau on the way in; x step 2 is fused with the
-// real-to-complex untangling; the (real) DC and Nyquist x columns are stored
-// together as X_0 + i X_nx/2 in column 0, so the y transform runs on nx/2
-// columns; y step 2 writes the spectrum plane to global memory, and the
-// packed column is separated last (A_k = (C_k + conj C_-k) / 2,
-// B_k = (C_k - conj C_-k) / 2i).
-// 16-point x steps (nx = 96) need more registers than three blocks per SM allow
-template <int NX, int NY>
-__global__ void __launch_bounds__(kPlaneThreads, Split<NX / 2>::N1 >= 16 ? 2 : kPlaneMinBlocks)
-    k_plane_fwd(GridDev g, const float* __restrict__ in, float2* __restrict__ spec, int mode) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  constexpr int X1 = Split<NXH>::N1, X2 = Split<NXH>::N2;
-  constexpr int Y1 = Split<NY>::N1, Y2 = Split<NY>::N2;
-  static_assert(X2 > 1 && X1 % 2 == 0, "x split must have two steps and an even first factor");
-  extern __shared__ __align__(128) float2 sm[];
-  float2* P = sm;                      // [NY][SX]: the spectrum plane's own layout
-  float2* twx = P + NY * SX;           // transposed: W^(n2 k1) at k1 * X2 + n2
-  float2* twy = twx + NXH;
-  float2* r2c = twy + NY;
-  float2* dm = r2c + SX;
-  const int c = blockIdx.x, z = blockIdx.y;
-  allow_dependent_launch();
-  for (int i = threadIdx.x; i < NXH; i += blockDim.x)
-    twx[(i % X1) * X2 + i / X1] = g.tw_x[i];
-  for (int i = threadIdx.x; i < NY; i += blockDim.x) twy[i] = g.tw_y[i];
-  for (int i = threadIdx.x; i < SX; i += blockDim.x) r2c[i] = g.r2c_w[i];
-  grid_dependency_wait();   // the FFT tables are fixed; everything below may be in flight
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) dm[i] = g.dmat[i];
-  __syncthreads();
-  const size_t nf2 = (size_t)g.n / 2;
-  const float2* in2 = reinterpret_cast<const float2*>(in) + (size_t)z * NY * NXH;
-  const uchar2* ph2 = reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * NY * NXH;
-  const bool three = mode != GM_RAW_TAU && c < 3;
-  // With at most two phases the material table is two register pairs and a
-  // select (phase ids are < n_phases), which takes the table lookups off the
-  // shared-memory pipe.
-  const bool two = g.n_phases <= 2;
-  const float2 dm0 = dm[0], dm1 = dm[1];
-  auto dmat = [&](unsigned char id) { return two ? (id ? dm1 : dm0) : dm[id]; };
-  for (int q = threadIdx.x; q < NY * X2; q += blockDim.x) {
-    int y, n2;
-    row_task<X2, NY>(q, y, n2);
-    const int rb = y * NXH + n2;
-    float2 v[X1];
-    if (!three) {
-      float2 a[X1];
-      uchar2 ph[X1];
-#pragma unroll
-      for (int i = 0; i < X1; ++i) {
-        a[i] = in2[c * nf2 + rb + X2 * i];
-        if (mode != GM_RAW_TAU) ph[i] = ph2[rb + X2 * i];
-      }
-#pragma unroll
-      for (int i = 0; i < X1; ++i) {
-        if (mode == GM_RAW_TAU) {
-          v[i] = a[i];
-        } else {
-          const float2 d0 = dmat(ph[i].x), d1 = dmat(ph[i].y);
-          v[i] = make_float2(2.f * d0.y * a[i].x, 2.f * d1.y * a[i].y);
-        }
-      }
-    } else {
-      constexpr int H = X1 >= 4 ? 4 : X1;   // voxel pairs loaded per batch
-#pragma unroll
-      for (int i0 = 0; i0 < X1; i0 += H) {
-        float2 a[H], b[H], d[H];
-        uchar2 ph[H];
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-          const int i = i0 + j;
-          a[j] = in2[rb + X2 * i];
-          b[j] = in2[nf2 + rb + X2 * i];
-          d[j] = in2[2 * nf2 + rb + X2 * i];
-          ph[j] = ph2[rb + X2 * i];
-        }
-#pragma unroll
-        for (int j = 0; j < H; ++j) {
-          const float2 d0 = dmat(ph[j].x), d1 = dmat(ph[j].y);
-          const float2 e = c == 0 ? a[j] : (c == 1 ? b[j] : d[j]);
-          v[i0 + j] = make_float2(fmaf(d0.x, a[j].x + b[j].x + d[j].x, 2.f * d0.y * e.x),
-                                  fmaf(d1.x, a[j].y + b[j].y + d[j].y, 2.f * d1.y * e.y));
-        }
-      }
-    }
-    RegDft<X1, false>::run(v);
-#pragma unroll
-    for (int k1 = 1; k1 < X1; ++k1) v[k1] = cmul(v[k1], twx[k1 * X2 + n2]);
-    float2* p = P + y * SX + n2;
-#pragma unroll
-    for (int i = 0; i < X1; ++i) p[i * X2] = v[i];
-  }
-  __syncthreads();
-  // x step 2 fused with the untangling.  Slot group k1 holds the
-  // frequencies k1 + X1 i; the partner nx/2 - k of k lies in group X1 - k1
-  // (groups 0 and X1/2 pair with themselves).
-  constexpr int NU = X1 / 2 + 1;
-  for (int t = threadIdx.x; t < NY * NU; t += blockDim.x) {
-    const int b = t % NY, u = t / NY;
-    float2* p = P + b * SX;
-    if (u == 0 || u == X1 / 2) {
-      const int k1 = u;
-      float2 v[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) v[i] = p[k1 * X2 + i];
-      RegDft<X2, false>::run(v);
-      float2 o[X2];
-      if (k1 == 0) {
-        const float2 z0 = v[0];
-        o[0] = make_float2(z0.x + z0.y, z0.x - z0.y);   // (X_0, X_nx/2), both real
-#pragma unroll
-        for (int i = 1; i < X2; ++i) {
-          const int ip = X2 - i;
-          if (i < ip) {
-            o[i] = r2c_post(v[i], v[ip], r2c[X1 * i]);
-            o[ip] = r2c_post(v[ip], v[i], r2c[X1 * ip]);
-          } else if (i == ip) {
-            o[i] = r2c_post(v[i], v[i], r2c[X1 * i]);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < X2; ++i) {
-          const int ip = X2 - 1 - i;
-          if (i < ip) {
-            o[i] = r2c_post(v[i], v[ip], r2c[X1 / 2 + X1 * i]);
-            o[ip] = r2c_post(v[ip], v[i], r2c[X1 / 2 + X1 * ip]);
-          } else if (i == ip) {
-            o[i] = r2c_post(v[i], v[i], r2c[X1 / 2 + X1 * i]);
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < X2; ++i) p[k1 * X2 + i] = o[i];
-    } else {
-      const int k1 = u, k1p = X1 - u;
-      float2 va[X2], vb[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        va[i] = p[k1 * X2 + i];
-        vb[i] = p[k1p * X2 + i];
-      }
-      RegDft<X2, false>::run(va);
-      RegDft<X2, false>::run(vb);
-      float2 oa[X2], ob[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        const int ip = X2 - 1 - i;
-        oa[i] = r2c_post(va[i], vb[ip], r2c[k1 + X1 * i]);
-        ob[ip] = r2c_post(vb[ip], va[i], r2c[k1p + X1 * ip]);
-      }
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        p[k1 * X2 + i] = oa[i];
-        p[k1p * X2 + i] = ob[i];
-      }
-    }
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < NXH * Y2; t += blockDim.x) {   // y step 1
-    const int b = t % NXH, n2 = t / NXH;
-    float2* p = P + b + n2 * SX;
-    float2 v[Y1];
-#pragma unroll
-    for (int i = 0; i < Y1; ++i) v[i] = p[i * Y2 * SX];
-    RegDft<Y1, false>::run(v);
-#pragma unroll
-    for (int k1 = 1; k1 < Y1; ++k1) v[k1] = cmul(v[k1], twy[n2 * Y1 + k1]);
-#pragma unroll
-    for (int i = 0; i < Y1; ++i) p[i * Y2 * SX] = v[i];
-  }
-  __syncthreads();
-  float2* out = spec + ((size_t)c * g.nz + z) * g.plane;
-  for (int t = threadIdx.x; t < NXH * Y1; t += blockDim.x) {   // y step 2 -> global
-    const int b = t % NXH, k1 = t / NXH;
-    float2* p = P + b + k1 * Y2 * SX;
-    float2 v[Y2];
-#pragma unroll
-    for (int i = 0; i < Y2; ++i) v[i] = p[i * SX];
-    RegDft<Y2, false>::run(v);
-    if (b == 0) {
-#pragma unroll
-      for (int i = 0; i < Y2; ++i) p[i * SX] = v[i];
-    } else {
-#pragma unroll
-      for (int i = 0; i < Y2; ++i) out[(size_t)(k1 * Y2 + i) * SX + b] = v[i];
-    }
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s < NY; s += blockDim.x) {   // separate the packed column
-    const int k = freq_of<NY>(s);
-    const int sn = slot_of<NY>((NY - k) % NY);
-    const float2 a = P[s * SX], b = P[sn * SX];
-    out[(size_t)s * SX] = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-    out[(size_t)s * SX + NXH] = make_float2(0.5f * (a.y + b.y), -0.5f * (a.x - b.x));
-  }
-}
-
-// Algorithm 3's last step at one voxel: out = (C + C0)^-1 : (s_a + C0 : eps_b)
-// with s_a = lam_a tr(eps) I + 2 mu_a eps and (C + C0) = (lam_s, mu_s); the
-// inverse of an isotropic stiffness maps t to (t - k_s tr(t) I) h_s with
-// k_s = lam_s / (3 lam_s + 2 mu_s), h_s = 1 / (2 mu_s).  pm = (lam_a, mu_a,
-// k_s, h_s) of the voxel's phase.
-__device__ __forceinline__ void post_normal(const float e[3], const float b[3], float4 pm,
-                                            float lam0, float mu0, float o[3]) {
-  const float tre = e[0] + e[1] + e[2];
-  const float trb = b[0] + b[1] + b[2];
-  float t[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    t[k] = 2.f * pm.y * e[k] + 2.f * mu0 * b[k];
-    t[k] += pm.x * tre + lam0 * trb;
-  }
-  const float sh = pm.z * (t[0] + t[1] + t[2]);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) o[k] = (t[k] - sh) * pm.w;
-}
-
-__device__ __forceinline__ float post_shear(float e, float b, float4 pm, float mu0) {
-  return (2.f * pm.y * e + 2.f * mu0 * b) * pm.w;
-}
-
-// Pass C, one block per (component, z).  The spectrum plane arrives by one
-// bulk asynchronous copy; y step 1 packs the DC and Nyquist x columns as
-// X_0 + i X_nx/2 (their inverse y transforms are real, so the result holds
-// both in its real and imaginary parts); the tangling is fused into x step
-// 1; x step 2 writes the real rows to global memory, scaled.  Without POST
-// a non-null `eps` is a field added to the output on the way out (the
-// defect of a re-centred iterate).
-//
-// POST: the pass ends with Algorithm 3's post-step instead (Section 5.5),
-// the transformed planes being eps_b and `eps` the map's input.  Blocks are
-// numbered z * 6 + c and run in clusters of three: the shear blocks apply
-// the post-step to their own component on the way out; the three normal
-// blocks of a plane, which need tr(eps_b), keep their real planes in shared
-// memory and each finishes all three normal components on a third of the
-// plane, reading the other two planes from the cluster's shared memory.
-template <int NX, int NY, bool POST>
-__global__ void __launch_bounds__(kPlaneThreads, kPlaneMinBlocks)
-    k_plane_inv(GridDev g, const float2* __restrict__ spec, float* __restrict__ outp,
-                float scale, const float* __restrict__ eps, const float4* __restrict__ post) {
-  constexpr int NXH = NX / 2, SX = NXH + 1, PL = NY * SX;
-  constexpr int X1 = Split<NXH>::N1, X2 = Split<NXH>::N2;
-  constexpr int Y1 = Split<NY>::N1, Y2 = Split<NY>::N2;
-  static_assert(X2 > 1 && X1 % 2 == 0, "x split must have two steps and an even first factor");
-  static_assert((PL * 8) % 16 == 0, "bulk copy size");
-  extern __shared__ __align__(128) float2 sm[];
-  float2* P = sm;
-  float2* twx = P + PL;
-  float2* twy = twx + NXH;
-  float2* r2c = twy + NY;
-  float4* pt = reinterpret_cast<float4*>(r2c + SX + ((PL + NXH + NY + SX) & 1));   // POST
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ int fail;
-  const int c = POST ? (int)blockIdx.x % 6 : (int)blockIdx.x / g.nz;
-  const int z = POST ? (int)blockIdx.x / 6 : (int)blockIdx.x - c * g.nz;
-  const int item = c * g.nz + z;
-  const bool gather = POST && c < 3;   // a normal block of a post-step cluster
-  allow_dependent_launch();
-  if (threadIdx.x == 0) {
-    fail = 0;
-    mbar_init(&bar, 1);
-    mbar_init_fence();
-  }
-  for (int i = threadIdx.x; i < NXH; i += blockDim.x) twx[i] = g.tw_x[i];
-  for (int i = threadIdx.x; i < NY; i += blockDim.x) twy[i] = g.tw_y[i];
-  for (int i = threadIdx.x; i < SX; i += blockDim.x) r2c[i] = g.r2c_w[i];
-  if (POST)
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) pt[i] = post[i];
-  grid_dependency_wait();
-  if (threadIdx.x == 0) {
-    mbar_arrive_expect_tx(&bar, PL * 8);
-    bulk_load(P, spec + (size_t)item * g.plane, PL * 8, &bar);
-  }
-  __syncthreads();
-  if (!mbar_wait(&bar, 0)) fail = 1;
-  __syncthreads();
-  if (fail) {   // the copy never completed: record it and leave the plane alone
-    if (threadIdx.x == 0) {
-      atomicExch(g.err, 1);
-      mbar_wait(&bar, 0);
-    }
-    if (gather) {   // the cluster's two barriers are still met
-      cluster_sync();
-      cluster_sync();
-    }
-    return;
-  }
-  for (int t = threadIdx.x; t < NXH * Y1; t += blockDim.x) {   // y step 1 (inverse)
-    const int b = t % NXH, k1 = t / NXH;
-    float2* p = P + k1 * Y2 * SX + b;
-    float2 v[Y2];
-#pragma unroll
-    for (int i = 0; i < Y2; ++i) v[i] = p[i * SX];
-    if (b == 0) {
-#pragma unroll
-      for (int i = 0; i < Y2; ++i) {
-        const float2 w = p[i * SX + NXH];
-        v[i] = make_float2(v[i].x - w.y, v[i].y + w.x);
-      }
-    }
-    RegDft<Y2, true>::run(v);
-#pragma unroll
-    for (int n2 = 1; n2 < Y2; ++n2) v[n2] = cmulc(v[n2], twy[n2 * Y1 + k1]);
-#pragma unroll
-    for (int i = 0; i < Y2; ++i) p[i * SX] = v[i];
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < NXH * Y2; t += blockDim.x) {   // y step 2 (inverse)
-    const int b = t % NXH, n2 = t / NXH;
-    float2* p = P + b + n2 * SX;
-    float2 v[Y1];
-#pragma unroll
-    for (int i = 0; i < Y1; ++i) v[i] = p[i * Y2 * SX];
-    RegDft<Y1, true>::run(v);
-#pragma unroll
-    for (int i = 0; i < Y1; ++i) p[i * Y2 * SX] = v[i];
-  }
-  __syncthreads();
-  constexpr int NU = X1 / 2 + 1;   // tangling fused into x step 1 (inverse)
-  for (int t = threadIdx.x; t < NY * NU; t += blockDim.x) {
-    const int b = t % NY, u = t / NY;
-    float2* p = P + b * SX;
-    if (u == 0 || u == X1 / 2) {
-      const int k1 = u;
-      float2 v[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) v[i] = p[k1 * X2 + i];
-      float2 o[X2];
-      if (k1 == 0) {
-        o[0] = make_float2(v[0].x + v[0].y, v[0].x - v[0].y);   // from (x_DC, x_Nyquist)
-#pragma unroll
-        for (int i = 1; i < X2; ++i) {
-          const int ip = X2 - i;
-          if (i < ip) {
-            o[i] = c2r_pre(v[i], v[ip], r2c[X1 * i]);
-            o[ip] = c2r_pre(v[ip], v[i], r2c[X1 * ip]);
-          } else if (i == ip) {
-            o[i] = c2r_pre(v[i], v[i], r2c[X1 * i]);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < X2; ++i) {
-          const int ip = X2 - 1 - i;
-          if (i < ip) {
-            o[i] = c2r_pre(v[i], v[ip], r2c[X1 / 2 + X1 * i]);
-            o[ip] = c2r_pre(v[ip], v[i], r2c[X1 / 2 + X1 * ip]);
-          } else if (i == ip) {
-            o[i] = c2r_pre(v[i], v[i], r2c[X1 / 2 + X1 * i]);
-          }
-        }
-      }
-      RegDft<X2, true>::run(o);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2) o[n2] = cmulc(o[n2], twx[n2 * X1 + k1]);
-#pragma unroll
-      for (int i = 0; i < X2; ++i) p[k1 * X2 + i] = o[i];
-    } else {
-      const int k1 = u, k1p = X1 - u;
-      float2 va[X2], vb[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        va[i] = p[k1 * X2 + i];
-        vb[i] = p[k1p * X2 + i];
-      }
-      float2 oa[X2], ob[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        const int ip = X2 - 1 - i;
-        oa[i] = c2r_pre(va[i], vb[ip], r2c[k1 + X1 * i]);
-        ob[ip] = c2r_pre(vb[ip], va[i], r2c[k1p + X1 * ip]);
-      }
-      RegDft<X2, true>::run(oa);
-      RegDft<X2, true>::run(ob);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2) {
-        oa[n2] = cmulc(oa[n2], twx[n2 * X1 + k1]);
-        ob[n2] = cmulc(ob[n2], twx[n2 * X1 + k1p]);
-      }
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        p[k1 * X2 + i] = oa[i];
-        p[k1p * X2 + i] = ob[i];
-      }
-    }
-  }
-  __syncthreads();
-  const size_t nf2 = (size_t)g.n / 2, zoff = (size_t)z * NY * NXH;
-  float2* out2 = reinterpret_cast<float2*>(outp) + zoff;
-  const float2* e2 = reinterpret_cast<const float2*>(eps) + zoff;
-  const uchar2* ph2 = reinterpret_cast<const uchar2*>(g.phase) + zoff;
-  for (int q = threadIdx.x; q < NY * X2; q += blockDim.x) {   // x step 2 (inverse)
-    int y, n2;
-    row_task<X2, NY>(q, y, n2);
-    float2* p = P + y * SX + n2;
-    const int r = y * NXH + n2;
-    float2 ev[X1];   // shear post-step: the map's input and phases, loaded ahead
-    uchar2 pv[X1];   // of the transform where the registers allow
-    constexpr bool AHEAD = X1 <= 8;
-    const bool addend = !POST && eps != nullptr;
-    if ((POST || addend) && AHEAD && !gather) {
-#pragma unroll
-      for (int i = 0; i < X1; ++i) {
-        ev[i] = e2[c * nf2 + r + i * X2];
-        if (POST) pv[i] = ph2[r + i * X2];
-      }
-    }
-    float2 v[X1];
-#pragma unroll
-    for (int i = 0; i < X1; ++i) v[i] = p[i * X2];
-    RegDft<X1, true>::run(v);
-    if (!POST && addend) {   // -> global, with the added field
-#pragma unroll
-      for (int i = 0; i < X1; ++i) {
-        if (!AHEAD) ev[i] = e2[c * nf2 + r + i * X2];
-        const float2 b = cscale(v[i], scale);
-        out2[c * nf2 + r + i * X2] = make_float2(b.x + ev[i].x, b.y + ev[i].y);
-      }
-    } else if (!POST) {   // -> global
-#pragma unroll
-      for (int i = 0; i < X1; ++i) out2[c * nf2 + r + i * X2] = cscale(v[i], scale);
-    } else if (gather) {   // -> the block's own slots, for the cluster's post-step
-#pragma unroll
-      for (int i = 0; i < X1; ++i) p[i * X2] = cscale(v[i], scale);
-    } else {   // shear component: post-step on the way out
-#pragma unroll
-      for (int i = 0; i < X1; ++i) {
-        if (!AHEAD) {
-          ev[i] = e2[c * nf2 + r + i * X2];
-          pv[i] = ph2[r + i * X2];
-        }
-        const float2 b = cscale(v[i], scale);
-        out2[c * nf2 + r + i * X2] = make_float2(post_shear(ev[i].x, b.x, pt[pv[i].x], g.mu0),
-                                                 post_shear(ev[i].y, b.y, pt[pv[i].y], g.mu0));
-      }
-    }
-  }
-  if (!gather) return;
-  // eps_b of the three normal components sits in the cluster's blocks 0, 1, 2
-  // (rank = c), at slot y * SX + h for the float2 pair h of row y.  Each
-  // thread takes U float2 pairs at a time, all loads issued before any use.
-  cluster_sync();
-  uint32_t rb[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) rb[k] = cluster_map(P, (uint32_t)k);
-  constexpr int U = 4, STRIDE = 3 * kPlaneThreads, TOT = NY * NXH;
-  for (int f0 = threadIdx.x + c * kPlaneThreads; f0 < TOT; f0 += U * STRIDE) {
-    float2 b[U][3], e[U][3];
-    uchar2 ph[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int f = f0 + u * STRIDE;
-      if (f < TOT) {
-        const int s = f + f / NXH;   // y * SX + h
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          b[u][k] = ld_cluster_f2(rb[k] + 8u * (uint32_t)s);
-          e[u][k] = e2[k * nf2 + f];
-        }
-        ph[u] = ph2[f];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int f = f0 + u * STRIDE;
-      if (f < TOT) {
-        const float ex[3] = {e[u][0].x, e[u][1].x, e[u][2].x};
-        const float ey[3] = {e[u][0].y, e[u][1].y, e[u][2].y};
-        const float bx[3] = {b[u][0].x, b[u][1].x, b[u][2].x};
-        const float by[3] = {b[u][0].y, b[u][1].y, b[u][2].y};
-        float ox[3], oy[3];
-        post_normal(ex, bx, pt[ph[u].x], g.lam0, g.mu0, ox);
-        post_normal(ey, by, pt[ph[u].y], g.lam0, g.mu0, oy);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) out2[k * nf2 + f] = make_float2(ox[k], oy[k]);
-      }
-    }
-  }
-  cluster_sync();   // no block leaves while another still reads its planes
 }
 
 // Pass B with T = 128 / split_n1(nz) pencils per block and 256 threads.
@@ -1570,43 +1073,8 @@ static cudaError_t launch_ypencil(const GridDev& g, float2* spec, bool inv, cuda
 }
 
 
-// the fused plane passes: nx = ny with a two-step x split of nx/2 and an even
-// first factor; the fused pencil pass: 128 / split_n1(nz) pencils per block
-#define RPM_FUSED_PLANE_SIZES(X) X(48) X(64) X(96) X(128)
-// (nz = 64 takes the 8-pencil tile of the original z pass: 0.0293 vs
-// 0.0314 ms per 64^3 apply)
+// nz = 64 takes the 8-pencil tile of the original z pass
 #define RPM_FUSED_Z_SIZES(X) X(32) X(48) X(96) X(128)
-
-template <int NX>
-static cudaError_t launch_fused_plane(const GridDev& g, const float* in, float* out, float2* spec,
-                                      int mode, int which, cudaStream_t st,
-                                      const float* add = nullptr) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  const size_t tab = (size_t)(NXH + NX + SX) * sizeof(float2);
-  const size_t smem = (size_t)NX * SX * sizeof(float2) + tab;
-  cudaError_t e;
-  if (which == 0) {
-    if ((e = set_smem(k_plane_fwd<NX, NX>, smem + 256 * sizeof(float2))) != cudaSuccess) return e;
-    return launch_pdl(k_plane_fwd<NX, NX>, dim3(6, g.nz), kPlaneThreads,
-                      smem + 256 * sizeof(float2), st, g, in, spec, mode);
-  }
-  if ((e = set_smem(k_plane_inv<NX, NX, false>, smem)) != cudaSuccess) return e;
-  return launch_pdl(k_plane_inv<NX, NX, false>, dim3(6 * g.nz), kPlaneThreads, smem, st, g,
-                    (const float2*)spec, out, 1.0f / (float)g.n, add, (const float4*)nullptr);
-}
-
-// pass C with Algorithm 3's post-step (clusters of three blocks)
-template <int NX>
-static cudaError_t launch_fused_inv_post(const GridDev& g, float* out, float2* spec,
-                                         const float* eps, const float4* post, cudaStream_t st) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  constexpr int F2 = NX * SX + NXH + NX + SX;
-  const size_t smem = (size_t)(F2 + (F2 & 1)) * sizeof(float2) + 256 * sizeof(float4);
-  cudaError_t e;
-  if ((e = set_smem(k_plane_inv<NX, NX, true>, smem)) != cudaSuccess) return e;
-  return launch_pdl_cluster(k_plane_inv<NX, NX, true>, dim3(6 * g.nz), kPlaneThreads, smem, st,
-                            3u, g, (const float2*)spec, out, 1.0f / (float)g.n, eps, post);
-}
 
 template <int NZ>
 static cudaError_t launch_fused_pencil(const GridDev& g, float2* spec, int mode,
@@ -1619,17 +1087,6 @@ static cudaError_t launch_fused_pencil(const GridDev& g, float2* spec, int mode,
                     spec, mode, ga);
 }
 
-static bool fused_plane_ok(const GridDev& g, const float2* spec) {
-  if (g.nx != g.ny || ((uintptr_t)spec & 15) != 0) return false;   // pass C's bulk copy
-  switch (g.nx) {
-#define RPM_CASE(N) case N:
-    RPM_FUSED_PLANE_SIZES(RPM_CASE)
-#undef RPM_CASE
-    return true;
-    default: return false;
-  }
-}
-
 static bool fused_pencil_ok(int nz) {
   switch (nz) {
 #define RPM_CASE(N) case N:
@@ -1637,29 +1094,6 @@ static bool fused_pencil_ok(int nz) {
 #undef RPM_CASE
     return true;
     default: return false;
-  }
-}
-
-static cudaError_t dispatch_fused_plane(const GridDev& g, const float* in, float* out,
-                                        float2* spec, int mode, int which, cudaStream_t st,
-                                        const float* add = nullptr) {
-  switch (g.nx) {
-#define RPM_CASE(N) \
-  case N: return launch_fused_plane<N>(g, in, out, spec, mode, which, st, add);
-    RPM_FUSED_PLANE_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-static cudaError_t dispatch_fused_inv_post(const GridDev& g, float* out, float2* spec,
-                                           const float* eps, const float4* post, cudaStream_t st) {
-  switch (g.nx) {
-#define RPM_CASE(N) \
-  case N: return launch_fused_inv_post<N>(g, out, spec, eps, post, st);
-    RPM_FUSED_PLANE_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
   }
 }
 
@@ -1746,16 +1180,17 @@ static cudaError_t dispatch_pencil(const GridDev& g, float2* spec, int mode, con
   }
 }
 
-// The plane kernels g.plane_v resolves to on this grid: 0 fused, 1 whole-plane, 2 five-pass.
+// The plane kernels g.plane_v resolves to on this grid: 0 paired (gamma_pair.cu),
+// 1 whole-plane, 2 five-pass.
 static int plane_path(const GridDev& g, const float2* spec) {
-  if (g.plane_v == 0 && fused_plane_ok(g, spec)) return 0;
+  if (g.plane_v == 0 && pair_plane_ok(g, spec)) return 0;
   if (g.plane_v <= 1 && plane_fits(g.nx, g.ny)) return 1;
   return 2;
 }
 
 static bool fused_z(const GridDev& g) { return g.pencil_t == 0 && fused_pencil_ok(g.nz); }
 
-bool fused_z_pass(const GridDev& g) { return fused_z(g); }
+bool fused_z_pass(const GridDev& g) { return plane_variant(g) != 0 && fused_z(g); }
 
 // (for a spectrum buffer from cudaMalloc, whose alignment is 256 bytes)
 int plane_variant(const GridDev& g) { return plane_path(g, nullptr); }
@@ -1763,6 +1198,7 @@ int plane_variant(const GridDev& g) { return plane_path(g, nullptr); }
 int gamma_launches(const GridDev& g) { return plane_variant(g) == 2 ? 5 : 3; }
 
 int pencil_tile(const GridDev& g) {
+  if (plane_variant(g) == 0) return 2 * pair_z_tile(g);
   if (fused_z(g)) return 128 / split_n1(g.nz);
   int t0;
   switch (g.nz) {
@@ -1780,7 +1216,7 @@ bool grid_supported(int nx, int ny, int nz) {
   return xy_size_ok(nx) && xy_size_ok(ny) && z_size_ok(nz);
 }
 
-static GammaArgs gamma_args(const GridDev& g, const double E[6]) {
+GammaArgs gamma_args(const GridDev& g, const double E[6]) {
   GammaArgs ga;
   for (int c = 0; c < 6; ++c) ga.En[c] = (float)(E ? E[c] * (double)g.n : 0.0);
   const double l0 = g.lam0, m0 = g.mu0;
@@ -1795,52 +1231,38 @@ static cudaError_t z_pass(const GridDev& g, float2* spec, int mode, const GammaA
                     : dispatch_pencil(g, spec, mode, ga, st);
 }
 
-// the post-step rides on the fused plane passes; fields are read as float2
-static bool fused_post_ok(const GridDev& g, const float* in, const float* out,
-                          const float2* spec) {
+// the post-step and an added field ride on the paired last pass; fields are read as float2
+static bool pair_map_ok(const GridDev& g, const float* in, const float* out, const float2* spec) {
   return plane_path(g, spec) == 0 && ((uintptr_t)in & 7) == 0 && ((uintptr_t)out & 7) == 0;
 }
 
 int polarization_launches(const GridDev& g, const float* in, const float* out,
                           const float2* spec) {
-  return fused_post_ok(g, in, out, spec) ? 3 : gamma_launches(g) + 1;
+  return pair_map_ok(g, in, out, spec) ? 3 : gamma_launches(g) + 1;
 }
 
 cudaError_t launch_polarization_map(const GridDev& g, const float4* post, const float* in,
                                     float* eb, float* out, float2* spec, const double Eb[6],
                                     int mode, cudaStream_t st) {
-  cudaError_t e;
-  if (fused_post_ok(g, in, out, spec)) {
-    const GammaArgs ga = gamma_args(g, Eb);
-    if ((e = dispatch_fused_plane(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
-    if ((e = z_pass(g, spec, mode, ga, st)) != cudaSuccess) return e;
-    return dispatch_fused_inv_post(g, out, spec, in, post, st);
-  }
-  if ((e = launch_apply_gamma(g, in, eb, spec, Eb, mode, st)) != cudaSuccess) return e;
+  if (pair_map_ok(g, in, out, spec))
+    return launch_pair_polarization(g, post, in, out, spec, Eb, mode, st);
+  const cudaError_t e = launch_apply_gamma(g, in, eb, spec, Eb, mode, st);
+  if (e != cudaSuccess) return e;
   return launch_polarization_post(g, post, in, eb, out, st);
 }
 
-// the added field rides on the fused last pass (float2 accesses)
-static bool fused_add_ok(const GridDev& g, const float* out, const float* add,
-                         const float2* spec) {
-  return plane_path(g, spec) == 0 && ((uintptr_t)out & 7) == 0 && ((uintptr_t)add & 7) == 0;
-}
-
 int gamma_add_launches(const GridDev& g, const float* out, const float* add, const float2* spec) {
-  return gamma_launches(g) + (add && !fused_add_ok(g, out, add, spec) ? 1 : 0);
+  return gamma_launches(g) + (add && !pair_map_ok(g, add, out, spec) ? 1 : 0);
 }
 
 cudaError_t launch_apply_gamma(const GridDev& g, const float* in, float* out, float2* spec,
                                const double E[6], int mode, cudaStream_t st, const float* add) {
+  const int path = plane_path(g, spec);
+  if (path == 0 && (!add || pair_map_ok(g, add, out, spec)))
+    return launch_pair_map(g, in, out, spec, E, mode, st, add);
   const GammaArgs ga = gamma_args(g, E);
   cudaError_t e;
   auto zpass = [&]() { return z_pass(g, spec, mode, ga, st); };
-  const int path = plane_path(g, spec);
-  if (path == 0 && (!add || fused_add_ok(g, out, add, spec))) {
-    if ((e = dispatch_fused_plane(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
-    if ((e = zpass()) != cudaSuccess) return e;
-    return dispatch_fused_plane(g, in, out, spec, mode, 1, st, add);
-  }
   if (path <= 1 && plane_fits(g.nx, g.ny)) {
     if ((e = dispatch_plane(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
     if ((e = zpass()) != cudaSuccess) return e;

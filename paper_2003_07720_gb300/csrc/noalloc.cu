@@ -9,6 +9,7 @@
 // -- lives in file-scope __device__ arrays of fixed size, which every GPU that
 // loads the library keeps until the process exits.  The caller passes the
 // phase map, the input field and the output field.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -29,6 +30,10 @@ static __device__ __align__(256) float2 g_na_spec[kNaSpec];
 static __device__ __align__(256) float2 g_na_tw[3 * kNaMax];        // x (nx/2), y, z twiddles
 static __device__ __align__(256) float2 g_na_r2c[kNaMax / 2 + 1];
 static __device__ __align__(256) int2 g_na_f[kNaMax / 2 + 1 + kNaMax];  // x slots, then y slots
+// the paired kernels' tables: x (nx/2), y (ny/2), z twiddles, W_ny^j; x and y slots
+static __device__ __align__(256) float2 g_na_ptw[5 * kNaMax / 2];
+static __device__ __align__(256) int2 g_na_pfx[kNaMax / 2 + 1];
+static __device__ __align__(256) int4 g_na_pfy[kNaMax / 2];
 static __device__ __align__(256) float2 g_na_mat[2 * 256];           // (dlam, dmu), (lam, mu)
 static __device__ __align__(256) int g_na_err[4];                    // bounded-wait flag
 
@@ -42,6 +47,9 @@ struct NaDevice {
   float2* tw = nullptr;
   float2* r2c = nullptr;
   int2* f = nullptr;
+  float2* ptw = nullptr;
+  int2* pfx = nullptr;
+  int4* pfy = nullptr;
   float2* mat = nullptr;
   int* err = nullptr;
   std::mutex mu;            // guards the key below
@@ -63,6 +71,9 @@ cudaError_t na_setup(int dev, NaDevice** out) {
         (e = cudaGetSymbolAddress((void**)&d.tw, g_na_tw)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.r2c, g_na_r2c)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.f, g_na_f)) != cudaSuccess ||
+        (e = cudaGetSymbolAddress((void**)&d.ptw, g_na_ptw)) != cudaSuccess ||
+        (e = cudaGetSymbolAddress((void**)&d.pfx, g_na_pfx)) != cudaSuccess ||
+        (e = cudaGetSymbolAddress((void**)&d.pfy, g_na_pfy)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.mat, g_na_mat)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.err, g_na_err)) != cudaSuccess)
       d.setup = e;
@@ -149,8 +160,25 @@ extern "C" rpm_status rpm_apply_gamma_noalloc(const rpm_grid* grid, const uint8_
         f[nxh + 1 + s] =
             make_int2((2 * k < ny) ? k : k - ny, (ny % 2 == 0 && 2 * k == ny) ? 1 : 0);
       }
+      PairTables pt;
+      pair_tables(nx, ny, nz, &pt);
+      float2 ptw[5 * kNaMax / 2];
+      int2 pfx[kNaMax / 2 + 1];
+      int4 pfy[kNaMax / 2];
+      std::memset(ptw, 0, sizeof(ptw));
+      std::memset(pfx, 0, sizeof(pfx));
+      std::memset(pfy, 0, sizeof(pfy));
+      std::copy(pt.twx.begin(), pt.twx.end(), ptw);
+      std::copy(pt.twy.begin(), pt.twy.end(), ptw + kNaMax / 2);
+      std::copy(pt.twz.begin(), pt.twz.end(), ptw + kNaMax);
+      std::copy(pt.hw.begin(), pt.hw.end(), ptw + 2 * kNaMax);
+      std::copy(pt.fx.begin(), pt.fx.end(), pfx);
+      std::copy(pt.fy.begin(), pt.fy.end(), pfy);
       a->have_key = false;
-      if (cudaMemcpyAsync(a->tw, tw, sizeof(tw), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      if (cudaMemcpyAsync(a->ptw, ptw, sizeof(ptw), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+          cudaMemcpyAsync(a->pfx, pfx, sizeof(pfx), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+          cudaMemcpyAsync(a->pfy, pfy, sizeof(pfy), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+          cudaMemcpyAsync(a->tw, tw, sizeof(tw), cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(a->r2c, r2c, sizeof(r2c), cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(a->f, f, sizeof(f), cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(a->mat, mat, sizeof(mat), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -176,6 +204,12 @@ extern "C" rpm_status rpm_apply_gamma_noalloc(const rpm_grid* grid, const uint8_
   g.r2c_w = a->r2c;
   g.fx = a->f;
   g.fy = a->f + nxh + 1;
+  g.p_twx = a->ptw;
+  g.p_twy = a->ptw + kNaMax / 2;
+  g.p_twz = a->ptw + kNaMax;
+  g.p_hw = a->ptw + 2 * kNaMax;
+  g.p_fx = a->pfx;
+  g.p_fy = a->pfy;
   g.phase = phase;
   g.dmat = a->mat;
   g.cmat = a->mat + 256;

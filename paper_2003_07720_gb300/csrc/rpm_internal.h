@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "rpm.h"
 
 namespace rpm {
@@ -29,6 +31,13 @@ struct GridDev {
   const float2* r2c_w;   // W_{nx}^k, k = 0..nxh
   const int2* fx;        // per x slot: (signed frequency m, nyquist flag)
   const int2* fy;        // per y slot
+  // the same for the paired kernels (gamma_pair.cu), built by pair_tables
+  const float2* p_twx;   // W_{nx/2}^(n2*k1)
+  const float2* p_twy;   // W_{ny/2}^(n2*k1)
+  const float2* p_twz;   // W_{nz}^(n2*k1)
+  const float2* p_hw;    // W_{ny}^j, j < ny/2
+  const int2* p_fx;      // per x slot: (signed frequency, nyquist flag)
+  const int4* p_fy;      // per y slot: the same of the even and the odd line
   const uint8_t* phase;  // [nz][ny][nx]
   const float2* dmat;    // per phase: (lam - lam0, mu - mu0)
   const float2* cmat;    // per phase: (lam, mu)
@@ -36,11 +45,35 @@ struct GridDev {
   float lam0, mu0;
   float inv_lx, inv_ly, inv_lz;   // 1 / L_j (frequency scaling)
   int nyquist;           // 0: zero mixed Nyquist frequencies, 1: signed
-  int plane_v;           // x/y passes: 0 fused where available, 1 whole-plane, 2 five-pass
+  int plane_v;           // x/y passes: 0 paired where available, 1 whole-plane, 2 five-pass
   int pencil_t;          // z pass: 0 fused where available, else the default tile;
                          // 1 half, 2 twice the default pencils; 3 the default tile
   int* err;              // device flag set to 1 when a bounded wait of a kernel gave up
 };
+
+struct GammaArgs {
+  float En[6];       // E * n_vox (zero frequency of the strain in GM_FULL_MAP)
+  float a;           // (lam0 + mu0) / (lam0 + 2 mu0)
+  float inv_mu0;
+};
+GammaArgs gamma_args(const GridDev& g, const double E[6]);
+
+// ---- paired kernels (gamma_pair.cu) ----------------------------------------
+// Host tables of a grid; the vectors go to the p_* pointers of GridDev.
+struct PairTables {
+  std::vector<float2> twx, twy, twz, hw;
+  std::vector<int2> fx;
+  std::vector<int4> fy;
+};
+void pair_tables(int nx, int ny, int nz, PairTables* t);
+bool pair_plane_ok(const GridDev& g, const float2* spec);   // grid and buffer take them
+int pair_z_tile(const GridDev& g);                          // pencil pairs per z block
+// launch_apply_gamma / launch_polarization_map on such a grid (float2-aligned fields)
+cudaError_t launch_pair_map(const GridDev& g, const float* in, float* out, float2* spec,
+                            const double E[6], int mode, cudaStream_t st, const float* add);
+cudaError_t launch_pair_polarization(const GridDev& g, const float4* post, const float* in,
+                                     float* out, float2* spec, const double Eb[6], int mode,
+                                     cudaStream_t st);
 
 // One Gamma0 application: in [6][n] -> out [6][n] through the spectrum
 // scratch spec [6][nz][plane] (float2).  E (6 tensor components) is only

@@ -1,0 +1,43 @@
+"""The paired kernels (square planes of side 48-128) against the FP64 oracle
+over the z lengths and options their z pass distinguishes: single-step and
+two-step lengths, each number of pencils per block, a ragged last block,
+non-unit cell lengths, a material table of more than two phases."""
+import numpy as np
+import pytest
+
+import microstructure as ms
+from oracle import rpm_oracle as o
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5      # single Gamma0-apply, relative L2 (float32 fields)
+
+
+def _cell(shape, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    lam, mu = zip(*(ms.lame(e, 0.3) for e in (1.0, 10.0, 0.1)))
+    l0, m0 = ms.lame(5.0, 0.3)
+    return ms.Cell(phase=rng.integers(0, 3, shape).astype(np.uint8), lam=np.array(lam),
+                   mu=np.array(mu), lam0=l0, mu0=m0)
+
+
+@pytest.mark.parametrize("nz,n", [(1, 128), (2, 64), (3, 96), (4, 48), (6, 64), (8, 48), (12, 96),
+                                  (16, 64), (24, 48), (32, 48), (48, 96), (64, 48), (96, 48),
+                                  (128, 96), (256, 64)])
+@pytest.mark.parametrize("pencil", [0, 1, 2])
+def test_paired_map_matches_oracle(nz, n, pencil):
+    from paper_2003_07720_gb300 import rpm
+    cell = _cell((nz, n, n), 100 * nz + n)
+    lengths = (0.7, 1.0, 1.3)
+    E = np.array([0.3, -0.2, 0.1, 0.05, -0.04, 0.07])
+    x = np.random.Generator(np.random.PCG64(nz)).standard_normal((6, nz, n, n)).astype(np.float32)
+    out = torch.full((6, nz, n, n), float("nan"), device="cuda")
+    opts = rpm.rpm_default_options(p_max=0, pencil_variant=pencil)
+    with rpm.Context(cell, opts, lengths=lengths) as ctx:
+        assert rpm.rpm_plane_variant(ctx.handle) == 0
+        ctx.apply_gamma(torch.from_numpy(x).cuda(), E, out)
+    got = out.cpu().numpy().astype(np.float64)
+    prob = o.Problem(cell.phase, cell.lam, cell.mu, cell.lam0, cell.mu0, lengths=lengths)
+    ref = o.apply_F(prob, x.astype(np.float64), E)
+    assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < TOL
