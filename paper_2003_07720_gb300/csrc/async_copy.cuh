@@ -94,6 +94,20 @@ __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// 16-byte asynchronous copies global -> shared by ordinary threads (both
+// addresses 16-byte aligned), past the L1 cache; wait: all of the calling
+// thread's copies have arrived.
+__device__ __forceinline__ void async_copy16(void* dst_smem, const void* src_gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem)
+               : "memory");
+}
+__device__ __forceinline__ void async_copy_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void async_copy_wait() {
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 // Orders this thread's ordinary shared-memory accesses before later accesses
 // of the asynchronous copy engine (and the reverse).
 __device__ __forceinline__ void fence_async_smem() {

@@ -13,10 +13,10 @@
 //       complex-to-real tangling, inverse FFT along x of length nx/2, scale.
 //
 // Square planes nx = ny in {48, 64, 96, 128} run the paired kernels of
-// gamma_pair.cu.  The kernels here serve the other sizes (and the forced
-// variants): k_pass_a/b/c, the z pass k_pencil_green, in which the forward z
-// step 2, the Green operator and the inverse z step 1 run in registers, and
-// the five-pass variant for planes that do not fit in shared memory.
+// gamma_pair.cu, which also serves 256^2 planes and nx != ny in five passes.
+// The kernels here serve the small square planes (and the forced whole-plane
+// variant): k_pass_a/b/c, and the z pass k_pencil_green, in which the forward
+// z step 2, the Green operator and the inverse z step 1 run in registers.
 //
 // The Green operator of the isotropic reference medium is evaluated on the
 // fly from the unit wave vector n = xi/|xi|:
@@ -411,21 +411,6 @@ __global__ void __launch_bounds__(2 * kThreads, 2) k_pass_b_wide(GridDev g,
 }
 
 
-// Row task q of an x step over NY rows: (y, n2).  With N2 = 8 the two
-// half-warps take rows y and y + 8, so that the 8-byte accesses of one
-// instruction fall in distinct banks (row stride nx/2 + 1 float2).
-template <int N2, int NY>
-__device__ __forceinline__ void row_task(int q, int& y, int& n2) {
-  if (N2 == 8 && NY % 16 == 0) {
-    n2 = q & 7;
-    const int h = (q >> 3) & 1, g = q >> 4;
-    y = (g & 7) + ((g >> 3) << 4) + (h << 3);
-  } else {
-    n2 = q % N2;
-    y = q / N2;
-  }
-}
-
 // Pass B with T = 128 / split_n1(nz) pencils per block and 256 threads.
 // Forward z step 1 reads the spectrum from global memory; forward step 2, the
 // Green operator and inverse step 1 run in registers on one (pencil, k1)
@@ -592,376 +577,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_pencil_green(GridDev g, float2*
 }
 
 // ---------------------------------------------------------------------------
-// Five-pass variant for planes that do not fit in shared memory (nx = 256)
-// and for nx != ny: rows along x, pencils along y, the z pass above, pencils
-// along y (inverse), rows along x (inverse).  The spectrum layout and slot
-// orders are those of the three-pass path, so pass B is shared.
-// ---------------------------------------------------------------------------
-constexpr int kRows = 32;             // rows per block in the inverse x pass
-constexpr int kRowsP = kRows + 1;     // odd stride
-
-// Forward x pass of the five-pass variant, one block per (component group,
-// group of kRowsG rows, z): group 0 holds the three normal components, group 1
-// the three shear components, as 3 kRowsG lines.  Each strain component is
-// loaded once and the trace once per voxel (Eq. 2.3), then the packed
-// half-length x-FFT and the real-to-complex untangling run on all lines.
-constexpr int kRowsG = 16;              // rows of one component per block
-constexpr int kLinesG = 3 * kRowsG;     // lines per block (three components)
-constexpr int kLinesGP = kLinesG + 1;   // odd stride
-
-template <int NX>
-__global__ void __launch_bounds__(kThreads) k_rows_fwd(GridDev g, const float* __restrict__ in,
-                                                       float2* __restrict__ spec, int mode) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  extern __shared__ float2 sm[];
-  float2* P = sm;                                  // [SX][kLinesGP], line = j kRowsG + row
-  float2* twx = P + SX * kLinesGP;
-  float2* r2c = twx + NXH;
-  float2* dm = r2c + SX;
-  const int grp = blockIdx.x, y0 = blockIdx.y * kRowsG, z = blockIdx.z;
-  const int ny = g.ny;
-  for (int i = threadIdx.x; i < NXH; i += blockDim.x) twx[i] = g.tw_x[i];
-  for (int i = threadIdx.x; i < SX; i += blockDim.x) r2c[i] = g.r2c_w[i];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) dm[i] = g.dmat[i];
-  __syncthreads();
-  const size_t n2 = (size_t)g.n / 2;
-  const size_t row2 = ((size_t)z * ny + y0) * NXH;         // float2 offset of row y0
-  const float2* in2 = reinterpret_cast<const float2*>(in) + 3 * grp * n2 + row2;
-  const uchar2* ph2 = reinterpret_cast<const uchar2*>(g.phase) + row2;
-  // Loads are issued in groups of U voxel pairs per thread before any use.
-  constexpr int TOT = kRowsG * NXH, U = 2;
-  for (int base = threadIdx.x; base < TOT; base += U * kThreads) {
-    float2 e[U][3];
-    uchar2 ph[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int idx = base + u * kThreads;
-      if (idx < TOT && y0 + idx / NXH < ny) {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) e[u][j] = in2[j * n2 + idx];
-        if (mode != GM_RAW_TAU) ph[u] = ph2[idx];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int idx = base + u * kThreads;
-      if (idx < TOT) {
-        const int r = idx / NXH, h = idx - r * NXH;
-        float2 t[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) t[j] = make_float2(0.f, 0.f);
-        if (y0 + r < ny) {
-          if (mode == GM_RAW_TAU) {
-#pragma unroll
-            for (int j = 0; j < 3; ++j) t[j] = e[u][j];
-          } else {
-            const float2 d0 = dm[ph[u].x], d1 = dm[ph[u].y];
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-              t[j] = make_float2(2.f * d0.y * e[u][j].x, 2.f * d1.y * e[u][j].y);
-            if (grp == 0) {
-              const float trx = e[u][0].x + e[u][1].x + e[u][2].x;
-              const float try_ = e[u][0].y + e[u][1].y + e[u][2].y;
-#pragma unroll
-              for (int j = 0; j < 3; ++j) {
-                t[j].x = fmaf(d0.x, trx, t[j].x);
-                t[j].y = fmaf(d1.x, try_, t[j].y);
-              }
-            }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 3; ++j) P[h * kLinesGP + j * kRowsG + r] = t[j];
-      }
-    }
-  }
-  __syncthreads();
-  smem_fft<NXH, false, kLinesG, 1, kLinesGP>(P, twx);
-  for (int t = threadIdx.x; t < kLinesG * (NXH / 2 + 1); t += blockDim.x) {
-    const int r = t % kLinesG, k = t / kLinesG;
-    if (k == 0) {
-      const float2 z0 = P[r];
-      P[r] = make_float2(z0.x + z0.y, 0.f);
-      P[NXH * kLinesGP + r] = make_float2(z0.x - z0.y, 0.f);
-    } else {
-      const int kk = NXH - k;
-      const int sk = slot_of<NXH>(k), skk = slot_of<NXH>(kk);
-      const float2 a = P[sk * kLinesGP + r], b = P[skk * kLinesGP + r];
-      P[sk * kLinesGP + r] = r2c_post(a, b, r2c[k]);
-      if (kk != k) P[skk * kLinesGP + r] = r2c_post(b, a, r2c[kk]);
-    }
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < kLinesG * SX; idx += blockDim.x) {
-    const int l = idx / SX, sx = idx - l * SX;
-    const int j = l / kRowsG, r = l - j * kRowsG;
-    if (y0 + r < ny)
-      spec[((size_t)(3 * grp + j) * g.nz + z) * g.plane + (size_t)(y0 + r) * SX + sx] =
-          P[sx * kLinesGP + l];
-  }
-}
-
-template <int NX>
-__global__ void __launch_bounds__(kThreads) k_rows_inv(GridDev g, const float2* __restrict__ spec,
-                                                       float* __restrict__ outp, float scale) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  extern __shared__ float2 sm[];
-  float2* P = sm;
-  float2* twx = P + SX * kRowsP;
-  float2* r2c = twx + NXH;
-  const int c = blockIdx.x, y0 = blockIdx.y * kRows, z = blockIdx.z;
-  const int ny = g.ny;
-  for (int i = threadIdx.x; i < NXH; i += blockDim.x) twx[i] = g.tw_x[i];
-  for (int i = threadIdx.x; i < SX; i += blockDim.x) r2c[i] = g.r2c_w[i];
-  const float2* src = spec + ((size_t)c * g.nz + z) * g.plane + (size_t)y0 * SX;
-  for (int idx = threadIdx.x; idx < kRows * SX; idx += blockDim.x) {
-    const int r = idx / SX, sx = idx - r * SX;
-    P[sx * kRowsP + r] = (y0 + r < ny) ? src[idx] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < kRows * (NXH / 2 + 1); t += blockDim.x) {
-    const int r = t % kRows, k = t / kRows;
-    if (k == 0) {
-      P[r] = c2r_pre(P[r], P[NXH * kRowsP + r], make_float2(1.f, 0.f));
-    } else {
-      const int kk = NXH - k;
-      const int sk = slot_of<NXH>(k), skk = slot_of<NXH>(kk);
-      const float2 a = P[sk * kRowsP + r], b = P[skk * kRowsP + r];
-      P[sk * kRowsP + r] = c2r_pre(a, b, r2c[k]);
-      if (kk != k) P[skk * kRowsP + r] = c2r_pre(b, a, r2c[kk]);
-    }
-  }
-  __syncthreads();
-  smem_fft<NXH, true, kRows, 1, kRowsP>(P, twx);
-  const size_t n2 = (size_t)g.n / 2;
-  float2* out2 = reinterpret_cast<float2*>(outp) + c * n2 + ((size_t)z * ny + y0) * NXH;
-  for (int idx = threadIdx.x; idx < kRows * NXH; idx += blockDim.x) {
-    const int r = idx / NXH, h = idx - r * NXH;
-    if (y0 + r < ny) out2[idx] = cscale(P[h * kRowsP + r], scale);
-  }
-}
-
-// The inverse x-row pass of the five-pass variant with the tangling fused
-// into x step 1 and x step 2 writing the real rows straight to global memory
-// (nx/2 with a two-step split and an even first factor).  Rows past ny are
-// skipped.  (A forward counterpart -- strain rows read in x step 1, untangling
-// fused into x step 2 -- measured slower than k_rows_fwd at 256^3: 280 against
-// 248 us.)
-template <int NX>
-__global__ void __launch_bounds__(kThreads) k_rows_inv_direct(GridDev g, const float2* __restrict__ spec,
-                                                              float* __restrict__ outp, float scale) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  constexpr int X1 = Split<NXH>::N1, X2 = Split<NXH>::N2;
-  static_assert(X2 > 1 && X1 % 2 == 0, "x split must have two steps and an even first factor");
-  extern __shared__ float2 sm[];
-  float2* P = sm;                                  // [SX][kRowsP]
-  float2* twx = P + SX * kRowsP;
-  float2* r2c = twx + NXH;
-  const int c = blockIdx.x, y0 = blockIdx.y * kRows, z = blockIdx.z;
-  const int ny = g.ny;
-  allow_dependent_launch();
-  for (int i = threadIdx.x; i < NXH; i += blockDim.x) twx[i] = g.tw_x[i];
-  for (int i = threadIdx.x; i < SX; i += blockDim.x) r2c[i] = g.r2c_w[i];
-  grid_dependency_wait();
-  const float2* src = spec + ((size_t)c * g.nz + z) * g.plane + (size_t)y0 * SX;
-  for (int idx = threadIdx.x; idx < kRows * SX; idx += blockDim.x) {
-    const int r = idx / SX, sx = idx - r * SX;
-    P[sx * kRowsP + r] = (y0 + r < ny) ? src[idx] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  constexpr int NU = X1 / 2 + 1;   // tangling fused into x step 1 (inverse)
-  constexpr int LS = kRowsP;
-  for (int t = threadIdx.x; t < kRows * NU; t += blockDim.x) {
-    const int b = t % kRows, u = t / kRows;
-    float2* p = P + b;
-    if (u == 0 || u == X1 / 2) {
-      const int k1 = u;
-      float2 v[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) v[i] = p[(k1 * X2 + i) * LS];
-      float2 o[X2];
-      if (k1 == 0) {
-        o[0] = c2r_pre(v[0], p[NXH * LS], make_float2(1.f, 0.f));
-#pragma unroll
-        for (int i = 1; i < X2; ++i) {
-          const int ip = X2 - i;
-          if (i < ip) {
-            o[i] = c2r_pre(v[i], v[ip], r2c[X1 * i]);
-            o[ip] = c2r_pre(v[ip], v[i], r2c[X1 * ip]);
-          } else if (i == ip) {
-            o[i] = c2r_pre(v[i], v[i], r2c[X1 * i]);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < X2; ++i) {
-          const int ip = X2 - 1 - i;
-          if (i < ip) {
-            o[i] = c2r_pre(v[i], v[ip], r2c[X1 / 2 + X1 * i]);
-            o[ip] = c2r_pre(v[ip], v[i], r2c[X1 / 2 + X1 * ip]);
-          } else if (i == ip) {
-            o[i] = c2r_pre(v[i], v[i], r2c[X1 / 2 + X1 * i]);
-          }
-        }
-      }
-      RegDft<X2, true>::run(o);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2) o[n2] = cmulc(o[n2], twx[n2 * X1 + k1]);
-#pragma unroll
-      for (int i = 0; i < X2; ++i) p[(k1 * X2 + i) * LS] = o[i];
-    } else {
-      const int k1 = u, k1p = X1 - u;
-      float2 va[X2], vb[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        va[i] = p[(k1 * X2 + i) * LS];
-        vb[i] = p[(k1p * X2 + i) * LS];
-      }
-      float2 oa[X2], ob[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        const int ip = X2 - 1 - i;
-        oa[i] = c2r_pre(va[i], vb[ip], r2c[k1 + X1 * i]);
-        ob[ip] = c2r_pre(vb[ip], va[i], r2c[k1p + X1 * ip]);
-      }
-      RegDft<X2, true>::run(oa);
-      RegDft<X2, true>::run(ob);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2) {
-        oa[n2] = cmulc(oa[n2], twx[n2 * X1 + k1]);
-        ob[n2] = cmulc(ob[n2], twx[n2 * X1 + k1p]);
-      }
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        p[(k1 * X2 + i) * LS] = oa[i];
-        p[(k1p * X2 + i) * LS] = ob[i];
-      }
-    }
-  }
-  __syncthreads();
-  const size_t nf2 = (size_t)g.n / 2;
-  float2* out2 = reinterpret_cast<float2*>(outp) + c * nf2 + ((size_t)z * ny + y0) * NXH;
-  for (int q = threadIdx.x; q < kRows * X2; q += blockDim.x) {   // x step 2 -> global
-    int r, n2;
-    row_task<X2, kRows>(q, r, n2);
-    float2 v[X1];
-#pragma unroll
-    for (int i = 0; i < X1; ++i) v[i] = P[(n2 + X2 * i) * kRowsP + r];
-    RegDft<X1, true>::run(v);
-    if (y0 + r < ny) {
-      float2* o = out2 + (size_t)r * NXH + n2;
-#pragma unroll
-      for (int i = 0; i < X1; ++i) o[i * X2] = cscale(v[i], scale);
-    }
-  }
-}
-
-// In-place FFT along y of TY consecutive x slots of one (component, z) plane.
-template <int NY>
-struct YPencilCfg {
-  static constexpr int TY = NY >= 256 ? 16 : (NY >= 128 ? 32 : 64);
-  static constexpr int NYP = NY + 1;
-};
-
-template <int NY, bool INV>
-__global__ void __launch_bounds__(kThreads) k_ypencil(GridDev g, float2* __restrict__ spec) {
-  using C = YPencilCfg<NY>;
-  constexpr int TY = C::TY, NYP = C::NYP;
-  extern __shared__ float2 sm[];
-  float2* B = sm;                  // [TY][NYP]
-  float2* twy = B + TY * NYP;
-  for (int i = threadIdx.x; i < NY; i += blockDim.x) twy[i] = g.tw_y[i];
-  const int sx0 = blockIdx.x * TY;
-  const int SX = g.nxh + 1;
-  float2* pl = spec + (size_t)blockIdx.y * g.plane;     // blockIdx.y = c * nz + z
-  for (int idx = threadIdx.x; idx < TY * NY; idx += blockDim.x) {
-    const int t = idx % TY, y = idx / TY;
-    B[t * NYP + y] = (sx0 + t < SX) ? pl[(size_t)y * SX + sx0 + t] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  smem_fft<NY, INV, TY, NYP, 1>(B, twy);
-  for (int idx = threadIdx.x; idx < TY * NY; idx += blockDim.x) {
-    const int t = idx % TY, y = idx / TY;
-    if (sx0 + t < SX) pl[(size_t)y * SX + sx0 + t] = B[t * NYP + y];
-  }
-}
-
-// The y pass of the five-pass variant with its outer FFT steps on global
-// memory: the first register step reads the TY columns straight from the
-// spectrum, the second writes them straight back, and shared memory holds the
-// exchange between the two steps only (column stride NY + 1: conflict-free).
-template <int NY, bool INV>
-__global__ void __launch_bounds__(kThreads) k_ypencil_direct(GridDev g, float2* __restrict__ spec) {
-  using C = YPencilCfg<NY>;
-  constexpr int TY = C::TY, NYP = C::NYP;
-  constexpr int Y1 = Split<NY>::N1, Y2 = Split<NY>::N2;
-  static_assert(Y2 > 1, "two register steps");
-  extern __shared__ __align__(16) float2 sm[];
-  float2* B = sm;                  // [TY][NYP]
-  float2* twy = B + TY * NYP;
-  allow_dependent_launch();
-  for (int i = threadIdx.x; i < NY; i += blockDim.x) twy[i] = g.tw_y[i];
-  grid_dependency_wait();
-  __syncthreads();
-  const int sx0 = blockIdx.x * TY;
-  const int SX = g.nxh + 1;
-  float2* pl = spec + (size_t)blockIdx.y * g.plane;     // blockIdx.y = c * nz + z
-  if (!INV) {
-    for (int q = threadIdx.x; q < TY * Y2; q += blockDim.x) {   // step 1: Y1-point, stride Y2
-      const int t = q % TY, n2 = q / TY;
-      const bool ok = sx0 + t < SX;
-      float2 v[Y1];
-#pragma unroll
-      for (int i = 0; i < Y1; ++i)
-        v[i] = ok ? pl[(size_t)(n2 + Y2 * i) * SX + sx0 + t] : make_float2(0.f, 0.f);
-      RegDft<Y1, false>::run(v);
-#pragma unroll
-      for (int k1 = 1; k1 < Y1; ++k1) v[k1] = cmul(v[k1], twy[n2 * Y1 + k1]);
-#pragma unroll
-      for (int i = 0; i < Y1; ++i) B[t * NYP + n2 + Y2 * i] = v[i];
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < TY * Y1; q += blockDim.x) {   // step 2: Y2-point, contiguous
-      const int t = q % TY, k1 = q / TY;
-      float2 v[Y2];
-#pragma unroll
-      for (int i = 0; i < Y2; ++i) v[i] = B[t * NYP + k1 * Y2 + i];
-      RegDft<Y2, false>::run(v);
-      if (sx0 + t < SX) {
-#pragma unroll
-        for (int i = 0; i < Y2; ++i) pl[(size_t)(k1 * Y2 + i) * SX + sx0 + t] = v[i];
-      }
-    }
-  } else {
-    for (int q = threadIdx.x; q < TY * Y1; q += blockDim.x) {   // inverse step 1
-      const int t = q % TY, k1 = q / TY;
-      const bool ok = sx0 + t < SX;
-      float2 v[Y2];
-#pragma unroll
-      for (int i = 0; i < Y2; ++i)
-        v[i] = ok ? pl[(size_t)(k1 * Y2 + i) * SX + sx0 + t] : make_float2(0.f, 0.f);
-      RegDft<Y2, true>::run(v);
-#pragma unroll
-      for (int n2 = 1; n2 < Y2; ++n2) v[n2] = cmulc(v[n2], twy[n2 * Y1 + k1]);
-#pragma unroll
-      for (int i = 0; i < Y2; ++i) B[t * NYP + k1 * Y2 + i] = v[i];
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < TY * Y2; q += blockDim.x) {   // inverse step 2
-      const int t = q % TY, n2 = q / TY;
-      float2 v[Y1];
-#pragma unroll
-      for (int i = 0; i < Y1; ++i) v[i] = B[t * NYP + n2 + Y2 * i];
-      RegDft<Y1, true>::run(v);
-      if (sx0 + t < SX) {
-#pragma unroll
-        for (int i = 0; i < Y1; ++i) pl[(size_t)(n2 + Y2 * i) * SX + sx0 + t] = v[i];
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 template <typename K>
@@ -1019,60 +634,6 @@ static cudaError_t launch_pencil_pass(const GridDev& g, float2* spec, int mode, 
 }
 
 
-template <int NX>
-static cudaError_t launch_rows(const GridDev& g, const float* in, float* out, float2* spec,
-                               int mode, int which, cudaStream_t st) {
-  constexpr int NXH = NX / 2, SX = NXH + 1;
-  const dim3 grid(6, (g.ny + kRows - 1) / kRows, g.nz);
-  if constexpr (Split<NXH>::N2 > 1 && Split<NXH>::N1 % 2 == 0) {
-    if (which == 1) {
-      const size_t smem = (size_t)(SX * kRowsP + NXH + SX) * sizeof(float2);
-      cudaError_t e;
-      if ((e = set_smem(k_rows_inv_direct<NX>, smem)) != cudaSuccess) return e;
-      return launch_pdl(k_rows_inv_direct<NX>, grid, kThreads, smem, st, g, (const float2*)spec,
-                        out, 1.0f / (float)g.n);
-    }
-  }
-  if (which == 0) {
-    const dim3 grid_f(2, (g.ny + kRowsG - 1) / kRowsG, g.nz);
-    const size_t smem = (size_t)(SX * kLinesGP + NXH + SX + 256) * sizeof(float2);
-    cudaError_t e = set_smem(k_rows_fwd<NX>, smem);
-    if (e != cudaSuccess) return e;
-    k_rows_fwd<NX><<<grid_f, kThreads, smem, st>>>(g, in, spec, mode);
-  } else {
-    const size_t smem = (size_t)(SX * kRowsP + NXH + SX) * sizeof(float2);
-    cudaError_t e = set_smem(k_rows_inv<NX>, smem);
-    if (e != cudaSuccess) return e;
-    k_rows_inv<NX><<<grid, kThreads, smem, st>>>(g, spec, out, 1.0f / (float)g.n);
-  }
-  return cudaGetLastError();
-}
-
-template <int NY>
-static cudaError_t launch_ypencil(const GridDev& g, float2* spec, bool inv, cudaStream_t st) {
-  using C = YPencilCfg<NY>;
-  const size_t smem = (size_t)(C::TY * C::NYP + NY) * sizeof(float2);
-  const dim3 grid((g.nxh + 1 + C::TY - 1) / C::TY, 6 * g.nz);
-  cudaError_t e;
-  if constexpr (Split<NY>::N2 > 1) {
-    if (inv) {
-      if ((e = set_smem(k_ypencil_direct<NY, true>, smem)) != cudaSuccess) return e;
-      return launch_pdl(k_ypencil_direct<NY, true>, grid, kThreads, smem, st, g, spec);
-    }
-    if ((e = set_smem(k_ypencil_direct<NY, false>, smem)) != cudaSuccess) return e;
-    return launch_pdl(k_ypencil_direct<NY, false>, grid, kThreads, smem, st, g, spec);
-  }
-  if (inv) {
-    if ((e = set_smem(k_ypencil<NY, true>, smem)) != cudaSuccess) return e;
-    k_ypencil<NY, true><<<grid, kThreads, smem, st>>>(g, spec);
-  } else {
-    if ((e = set_smem(k_ypencil<NY, false>, smem)) != cudaSuccess) return e;
-    k_ypencil<NY, false><<<grid, kThreads, smem, st>>>(g, spec);
-  }
-  return cudaGetLastError();
-}
-
-
 // nz = 64 takes the 8-pencil tile of the original z pass
 #define RPM_FUSED_Z_SIZES(X) X(32) X(48) X(96) X(128)
 
@@ -1111,27 +672,6 @@ static cudaError_t dispatch_fused_pencil(const GridDev& g, float2* spec, int mod
 #define RPM_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
 #define RPM_Z_SIZES(X) \
   X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
-
-static cudaError_t dispatch_rows(const GridDev& g, const float* in, float* out, float2* spec,
-                                 int mode, int which, cudaStream_t st) {
-  switch (g.nx) {
-#define RPM_CASE(N) \
-  case N: return launch_rows<N>(g, in, out, spec, mode, which, st);
-    RPM_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-static cudaError_t dispatch_ypencil(const GridDev& g, float2* spec, bool inv, cudaStream_t st) {
-  switch (g.ny) {
-#define RPM_CASE(N) \
-  case N: return launch_ypencil<N>(g, spec, inv, st);
-    RPM_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
-  }
-}
 
 // three-pass (whole xy planes in shared memory) when the plane fits
 static bool plane_fits(int nx, int ny) { return nx == ny && nx <= 128; }
@@ -1190,7 +730,7 @@ static int plane_path(const GridDev& g, const float2* spec) {
 
 static bool fused_z(const GridDev& g) { return g.pencil_t == 0 && fused_pencil_ok(g.nz); }
 
-bool fused_z_pass(const GridDev& g) { return plane_variant(g) != 0 && fused_z(g); }
+bool fused_z_pass(const GridDev& g) { return plane_variant(g) == 1 && fused_z(g); }
 
 // (for a spectrum buffer from cudaMalloc, whose alignment is 256 bytes)
 int plane_variant(const GridDev& g) { return plane_path(g, nullptr); }
@@ -1198,7 +738,7 @@ int plane_variant(const GridDev& g) { return plane_path(g, nullptr); }
 int gamma_launches(const GridDev& g) { return plane_variant(g) == 2 ? 5 : 3; }
 
 int pencil_tile(const GridDev& g) {
-  if (plane_variant(g) == 0) return 2 * pair_z_tile(g);
+  if (plane_variant(g) != 1) return g.nz <= 4 ? 128 : 2 * pair_z_tile(g);
   if (fused_z(g)) return 128 / split_n1(g.nz);
   int t0;
   switch (g.nz) {
@@ -1231,50 +771,51 @@ static cudaError_t z_pass(const GridDev& g, float2* spec, int mode, const GammaA
                     : dispatch_pencil(g, spec, mode, ga, st);
 }
 
-// the post-step and an added field ride on the paired last pass; fields are read as float2
-static bool pair_map_ok(const GridDev& g, const float* in, const float* out, const float2* spec) {
-  return plane_path(g, spec) == 0 && ((uintptr_t)in & 7) == 0 && ((uintptr_t)out & 7) == 0;
+// the post-step (paired planes) and an added field (paired planes and five
+// passes) ride on the last pass, which accesses fields as float2
+static bool float2_ok(const float* a, const float* b) {
+  return (((uintptr_t)a | (uintptr_t)b) & 7) == 0;
 }
 
 int polarization_launches(const GridDev& g, const float* in, const float* out,
                           const float2* spec) {
-  return pair_map_ok(g, in, out, spec) ? 3 : gamma_launches(g) + 1;
+  return plane_path(g, spec) == 0 && float2_ok(in, out) ? 3 : gamma_launches(g) + 1;
 }
 
 cudaError_t launch_polarization_map(const GridDev& g, const float4* post, const float* in,
                                     float* eb, float* out, float2* spec, const double Eb[6],
                                     int mode, cudaStream_t st) {
-  if (pair_map_ok(g, in, out, spec))
+  if (plane_path(g, spec) == 0 && float2_ok(in, out))
     return launch_pair_polarization(g, post, in, out, spec, Eb, mode, st);
   const cudaError_t e = launch_apply_gamma(g, in, eb, spec, Eb, mode, st);
   if (e != cudaSuccess) return e;
   return launch_polarization_post(g, post, in, eb, out, st);
 }
 
+static bool add_rides(const GridDev& g, const float* out, const float* add, const float2* spec) {
+  return plane_path(g, spec) != 1 && float2_ok(out, add);
+}
+
 int gamma_add_launches(const GridDev& g, const float* out, const float* add, const float2* spec) {
-  return gamma_launches(g) + (add && !pair_map_ok(g, add, out, spec) ? 1 : 0);
+  return gamma_launches(g) + (add && !add_rides(g, out, add, spec) ? 1 : 0);
 }
 
 cudaError_t launch_apply_gamma(const GridDev& g, const float* in, float* out, float2* spec,
                                const double E[6], int mode, cudaStream_t st, const float* add) {
   const int path = plane_path(g, spec);
-  if (path == 0 && (!add || pair_map_ok(g, add, out, spec)))
-    return launch_pair_map(g, in, out, spec, E, mode, st, add);
-  const GammaArgs ga = gamma_args(g, E);
+  const float* riding = add && add_rides(g, out, add, spec) ? add : nullptr;
   cudaError_t e;
-  auto zpass = [&]() { return z_pass(g, spec, mode, ga, st); };
-  if (path <= 1 && plane_fits(g.nx, g.ny)) {
-    if ((e = dispatch_plane(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
-    if ((e = zpass()) != cudaSuccess) return e;
-    e = dispatch_plane(g, in, out, spec, mode, 1, st);
+  if (path == 0) {
+    e = launch_pair_map(g, in, out, spec, E, mode, st, riding);
+  } else if (path == 2) {
+    e = launch_pair_rows_map(g, in, out, spec, E, mode, st, riding);
   } else {
-    if ((e = dispatch_rows(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
-    if ((e = dispatch_ypencil(g, spec, false, st)) != cudaSuccess) return e;
-    if ((e = zpass()) != cudaSuccess) return e;
-    if ((e = dispatch_ypencil(g, spec, true, st)) != cudaSuccess) return e;
-    e = dispatch_rows(g, in, out, spec, mode, 1, st);
+    const GammaArgs ga = gamma_args(g, E);
+    if ((e = dispatch_plane(g, in, out, spec, mode, 0, st)) != cudaSuccess) return e;
+    if ((e = z_pass(g, spec, mode, ga, st)) != cudaSuccess) return e;
+    e = dispatch_plane(g, in, out, spec, mode, 1, st);
   }
-  if (e != cudaSuccess || !add) return e;
+  if (e != cudaSuccess || !add || riding) return e;
   return launch_axpby(out, 1.f, out, 1.f, add, g.n, st);
 }
 

@@ -24,6 +24,7 @@
 // two or three resident blocks bound them.  One map of 128^3: 96 -> 87 us, of
 // 64^3 20.5 -> 16.1 us, of 48^3 15.3 -> 12.8 us; 96^3 passes A + B + C
 // 71 -> 40 us (single-kernel times).
+#include <algorithm>
 #include <cmath>
 
 #include "async_copy.cuh"
@@ -43,16 +44,24 @@ namespace {
 constexpr int pair_threads(int n) { return n == 96 ? 128 : 256; }
 constexpr int pair_blocks(int n) { return n == 96 ? 4 : 2; }
 
+// The x transform of a block's row pairs: rows nx long, ROWS pairs in shared
+// memory as [ROWS][nx/2 + 1], TPB threads.
+template <int NX, int ROWS_, int TPB_>
+struct PairX {
+  static constexpr int NXH = NX / 2, SX = NXH + 1, ROWS = ROWS_, TPB = TPB_;
+  static constexpr int X1 = pair_n1(NXH), X2 = NXH / X1;
+  static constexpr int NU = X1 / 2 + 1;
+  static_assert(X2 == 1 || X1 % 2 == 0, "two-step x splits need an even first factor");
+  static_assert(SX % 2 == 1 || X2 == 1, "odd row stride: rows fall in distinct 16-byte banks");
+};
+
 template <int N>
 struct PairPlane {
   static constexpr int NXH = N / 2, SX = NXH + 1, H = N / 2, PL = H * SX;
   static constexpr int X1 = pair_n1(NXH), X2 = NXH / X1;
   static constexpr int Y1 = pair_n1(H), Y2 = H / Y1;
-  static constexpr int NU = X1 / 2 + 1;
   static constexpr int TPB = pair_threads(N), MINB = pair_blocks(N);
-  static_assert(X2 > 1 && X1 % 2 == 0, "x split must have two steps and an even first factor");
-  static_assert(SX % 2 == 1, "odd row stride: rows fall in distinct 16-byte banks");
-  static_assert((PL * 16) % 16 == 0, "bulk copy size");
+  using X = PairX<N, H, TPB>;
 };
 
 // Task q of an x step that walks rows: (row, n2), n2 fastest.  With X2 = 4
@@ -105,19 +114,36 @@ __device__ __forceinline__ float4 splat_twiddle(float2 w) {
   return make_float4(w.x, w.x, w.y, w.y);
 }
 
+// Untangling of a row pair held whole in registers (Z_k in v), with the
+// radix-2 step along y; X_0 and X_M in slots 0 and M.
+template <int M>
+__device__ __forceinline__ void pair_untangle_row(const C2* v, const float4* r2c, float2 w,
+                                                  float4* p) {
+  const float2 zero = f2splat(0.f), x0 = f2add(v[0].re, v[0].im), xm = f2sub(v[0].re, v[0].im);
+  c2_store(p, pair_split_rows(C2{f2add(x0, x0), zero}, w));
+  c2_store(p + M, pair_split_rows(C2{f2add(xm, xm), zero}, w));
+#pragma unroll
+  for (int k = 1; k <= M / 2; ++k) {
+    C2 xk, xmk;
+    pair_r2c(v[k], v[M - k], r2c + k, xk, xmk);
+    c2_store(p + k, pair_split_rows(xk, w));
+    if (k < M - k) c2_store(p + M - k, pair_split_rows(xmk, w));
+  }
+}
+
 // x step 1 of pass A: the strain rows j and j + ny/2 are read from global
 // memory, the polarization formed on the way in (KIND: one component's rows as
 // they are, a shear component, or a normal one, which needs the trace and so
-// the other two normal components e1, e2).
+// the other two normal components e1, e2).  Row j + ny/2 lies `low` float2
+// after row j; rows past `rows` are skipped.
 enum { kRaw, kShear, kNormal };
-template <int N, int KIND, bool TWO>
+template <class C, int KIND, bool TWO, bool PACK>
 __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const float2* __restrict__ e1,
                                         const float2* __restrict__ e2,
-                                        const uchar2* __restrict__ phase, const float2* dm,
-                                        float4* P, const float4* twx) {
-  using C = PairPlane<N>;
-  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, X1 = C::X1, X2 = C::X2;
-  constexpr int LOW = H * NXH;         // row j + ny/2 lies LOW float2 after row j
+                                        const uchar2* __restrict__ phase, int low, int rows,
+                                        const float2* dm, float4* P, const float4* twx,
+                                        const float4* r2c, const float2* hw) {
+  constexpr int NXH = C::NXH, SX = C::SX, X1 = C::X1, X2 = C::X2;
   constexpr int B = KIND == kNormal && X1 > 4 ? 4 : X1;   // voxel pairs loaded per batch
   const float2 dm0 = dm[0], dm1 = dm[1];
   auto material = [&](unsigned char id) {
@@ -127,16 +153,17 @@ __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const flo
   // twiddles then stay in registers
   constexpr bool KEEP = C::TPB % X2 == 0;
   float2 tw[X1];
-  if (KEEP) {
+  if (KEEP && X2 > 1) {
 #pragma unroll
     for (int k1 = 1; k1 < X1; ++k1) {
       const float4 w = twx[k1 * X2 + threadIdx.x % X2];
       tw[k1] = make_float2(w.x, w.z);
     }
   }
-  for (int q = threadIdx.x; q < H * X2; q += C::TPB) {
+  for (int q = threadIdx.x; q < C::ROWS * X2; q += C::TPB) {
     int j, n2;
-    pair_row_task<X2, H>(q, j, n2);
+    pair_row_task<X2, C::ROWS>(q, j, n2);
+    if (j >= rows) continue;
     const int rb = j * NXH + n2;
     C2 v[X1];
 #pragma unroll
@@ -147,7 +174,7 @@ __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const flo
       for (int k = 0; k < B; ++k)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          const int at = rb + r * LOW + X2 * (i0 + k);
+          const int at = rb + r * low + X2 * (i0 + k);
           e[k][r] = __ldcs(e0 + at);
           if (KIND == kNormal) {
             f[k][r] = __ldcs(e1 + at);
@@ -175,6 +202,11 @@ __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const flo
     }
     PairDft<X1, false>::run(v);
     float4* p = P + j * SX + n2;
+    if constexpr (X2 == 1) {   // the whole row is here: untangle it in registers
+      const float2 w = hw[j];
+      pair_untangle_row<NXH>(v, r2c, w, p);
+      continue;
+    }
     c2_store(p, v[0]);
 #pragma unroll
     for (int k1 = 1; k1 < X1; ++k1)
@@ -183,62 +215,46 @@ __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const flo
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
-    k_pair_fwd(GridDev g, const float* __restrict__ in, float4* __restrict__ spec, int mode) {
-  using C = PairPlane<N>;
-  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, TPB = C::TPB;
-  constexpr int X1 = C::X1, X2 = C::X2, Y1 = C::Y1, Y2 = C::Y2;
-  extern __shared__ __align__(128) float4 sm4[];
-  float4* P = sm4;                     // [H][SX]
-  float4* twx = P + C::PL;             // [X1][X2]
-  float4* twy = twx + NXH;             // [Y1][Y2]
-  float4* r2c = twy + H;               // W_nx^k, k < nx/2
-  float2* hw = reinterpret_cast<float2*>(r2c + NXH);   // W_ny^j, j < ny/2
-  float2* dm = hw + H;
-  const int c = blockIdx.x, z = blockIdx.y;
-  allow_dependent_launch();
-  for (int i = threadIdx.x; i < NXH; i += TPB) {
-    twx[i] = splat_twiddle(g.p_twx[i]);
-    r2c[i] = splat_twiddle(g.r2c_w[i]);
-  }
-  for (int i = threadIdx.x; i < H; i += TPB) {
-    twy[i] = splat_twiddle(g.p_twy[i]);
-    hw[i] = g.p_hw[i];
-  }
-  grid_dependency_wait();   // the FFT tables are fixed; everything below may be in flight
-  for (int i = threadIdx.x; i < 256; i += TPB) {   // (lam, 2 mu) of C - C0 per phase
-    const float2 m = g.dmat[i];
-    dm[i] = make_float2(m.x, 2.f * m.y);
-  }
-  __syncthreads();
+// x step 1 of component c of a block's rows (`in`, `phase`: the first row).
+template <class C, bool PACK>
+__device__ __forceinline__ void pair_x1_component(const GridDev& g, const float2* in, int c,
+                                                  const uchar2* phase, int low, int rows, int mode,
+                                                  const float2* dm, float4* P, const float4* twx,
+                                                  const float4* r2c, const float2* hw) {
   const size_t nf2 = (size_t)g.n / 2;
-  const float2* in2 = reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH;
-  const uchar2* ph2 = reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH;
+  const float2* own = in + c * nf2;
   // With at most two phases the material table is two register pairs and a
   // select (phase ids are < n_phases), which takes the table lookups off the
   // shared-memory pipe.
-  if (mode == GM_RAW_TAU)
-    pair_x1<N, kRaw, true>(in2 + c * nf2, in2, in2, ph2, dm, P, twx);
-  else if (c >= 3 && g.n_phases <= 2)
-    pair_x1<N, kShear, true>(in2 + c * nf2, in2, in2, ph2, dm, P, twx);
-  else if (c >= 3)
-    pair_x1<N, kShear, false>(in2 + c * nf2, in2, in2, ph2, dm, P, twx);
-  else {
-    const float2* other = in2 + (c == 0 ? 1 : 0) * nf2;
-    const float2* last = in2 + (c == 2 ? 1 : 2) * nf2;
+  if (mode == GM_RAW_TAU) {
+    pair_x1<C, kRaw, true, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
+  } else if (c >= 3) {
     if (g.n_phases <= 2)
-      pair_x1<N, kNormal, true>(in2 + c * nf2, other, last, ph2, dm, P, twx);
+      pair_x1<C, kShear, true, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
     else
-      pair_x1<N, kNormal, false>(in2 + c * nf2, other, last, ph2, dm, P, twx);
+      pair_x1<C, kShear, false, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
+  } else {
+    const float2* other = in + (c == 0 ? 1 : 0) * nf2;
+    const float2* last = in + (c == 2 ? 1 : 2) * nf2;
+    if (g.n_phases <= 2)
+      pair_x1<C, kNormal, true, PACK>(own, other, last, phase, low, rows, dm, P, twx, r2c, hw);
+    else
+      pair_x1<C, kNormal, false, PACK>(own, other, last, phase, low, rows, dm, P, twx, r2c, hw);
   }
-  __syncthreads();
-  // x step 2 fused with the untangling and the radix-2 step along y.  Slot
-  // group k1 holds the frequencies k1 + X1 i; the partner nx/2 - k of k lies
-  // in group X1 - k1 (groups 0 and X1/2 pair with themselves).  X_0 and
-  // X_nx/2, both real, travel as X_0 + i X_nx/2 in column 0.
-  for (int t = threadIdx.x; t < H * C::NU; t += TPB) {
+}
+
+// x step 2 (two-step lengths) fused with the untangling and the radix-2 step
+// along y.  Slot group k1 holds the frequencies k1 + X1 i; the partner nx/2 - k
+// of k lies in group X1 - k1 (groups 0 and X1/2 pair with themselves).  X_0
+// and X_nx/2 are both real: with PACK they travel as X_0 + i X_nx/2 in column
+// 0, otherwise in columns 0 and nx/2.
+template <class C, bool PACK>
+__device__ __forceinline__ void pair_x2(float4* P, int rows, const float4* r2c, const float2* hw) {
+  constexpr int NXH = C::NXH, SX = C::SX, X1 = C::X1, X2 = C::X2, H = C::ROWS;
+  if constexpr (X2 > 1) {
+  for (int t = threadIdx.x; t < H * C::NU; t += C::TPB) {
     const int j = t % H, u = t / H;
+    if (j >= rows) continue;
     float4* p = P + j * SX;
     const float2 w = hw[j];
     if (u == 0 || u == X1 / 2) {
@@ -247,8 +263,13 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
       for (int i = 0; i < X2; ++i) v[i] = c2_load(p + u * X2 + i);
       PairDft<X2, false>::run(v);
       if (u == 0) {
-        const C2 o = {f2add(v[0].re, v[0].im), f2sub(v[0].re, v[0].im)};
-        c2_store(p, pair_split_rows(o, w));
+        const float2 x0 = f2add(v[0].re, v[0].im), xm = f2sub(v[0].re, v[0].im);
+        if (PACK) {
+          c2_store(p, pair_split_rows(C2{x0, xm}, w));
+        } else {
+          c2_store(p, pair_split_rows(C2{f2add(x0, x0), f2splat(0.f)}, w));
+          c2_store(p + NXH, pair_split_rows(C2{f2add(xm, xm), f2splat(0.f)}, w));
+        }
       }
 #pragma unroll
       for (int i = 0; i < X2; ++i) {
@@ -291,6 +312,44 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
       }
     }
   }
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
+    k_pair_fwd(GridDev g, const float* __restrict__ in, float4* __restrict__ spec, int mode) {
+  using C = PairPlane<N>;
+  using X = typename C::X;
+  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, TPB = C::TPB;
+  constexpr int Y1 = C::Y1, Y2 = C::Y2;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* P = sm4;                     // [H][SX]
+  float4* twx = P + C::PL;             // [X1][X2]
+  float4* twy = twx + NXH;             // [Y1][Y2]
+  float4* r2c = twy + H;               // W_nx^k, k < nx/2
+  float2* hw = reinterpret_cast<float2*>(r2c + NXH);   // W_ny^j, j < ny/2
+  float2* dm = hw + H;
+  const int c = blockIdx.x, z = blockIdx.y;
+  allow_dependent_launch();
+  for (int i = threadIdx.x; i < NXH; i += TPB) {
+    twx[i] = splat_twiddle(g.p_twx[i]);
+    r2c[i] = splat_twiddle(g.r2c_w[i]);
+  }
+  for (int i = threadIdx.x; i < H; i += TPB) {
+    twy[i] = splat_twiddle(g.p_twy[i]);
+    hw[i] = g.p_hw[i];
+  }
+  grid_dependency_wait();   // the FFT tables are fixed; everything below may be in flight
+  for (int i = threadIdx.x; i < 256; i += TPB) {   // (lam, 2 mu) of C - C0 per phase
+    const float2 m = g.dmat[i];
+    dm[i] = make_float2(m.x, 2.f * m.y);
+  }
+  __syncthreads();
+  pair_x1_component<X, true>(g, reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH, c,
+                             reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH,
+                             H * NXH, H, mode, dm, P, twx, r2c, hw);
+  __syncthreads();
+  pair_x2<X, true>(P, H, r2c, hw);
   __syncthreads();
   for (int t = threadIdx.x; t < NXH * Y2; t += TPB) {   // y step 1
     const int b = t % NXH, n2 = t / NXH;
@@ -328,6 +387,98 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
     const C2 b = {make_float2(be.re.x, bo.re.y), make_float2(be.im.x, bo.im.y)};
     c2_store(out + (size_t)s * SX, C2{f2add(a.re, b.re), f2sub(a.im, b.im)});
     c2_store(out + (size_t)s * SX + NXH, C2{f2add(a.im, b.im), f2sub(b.re, a.re)});
+  }
+}
+
+// The reverse of pair_untangle_row: 2 Z_k of a row pair from its M + 1 slots.
+template <int M>
+__device__ __forceinline__ void pair_tangle_row(const float4* p, const float4* r2c, float2 w,
+                                                C2* v) {
+  const float2 x0 = pair_join_rows(c2_load(p), w).re, xm = pair_join_rows(c2_load(p + M), w).re;
+  v[0] = {f2add(x0, xm), f2sub(x0, xm)};
+#pragma unroll
+  for (int k = 1; k <= M / 2; ++k) {
+    C2 zk, zm;
+    const C2 a = pair_join_rows(c2_load(p + k), w), b = pair_join_rows(c2_load(p + M - k), w);
+    pair_c2r(a, b, r2c + k, zk, zm);
+    v[k] = zk;
+    if (k < M - k) v[M - k] = zm;
+  }
+}
+
+// The last radix-2 step along y and the tangling, fused into x step 1 of the
+// inverse (two-step lengths); the reverse of pair_x2.
+template <class C, bool PACK>
+__device__ __forceinline__ void pair_x1_inv(float4* P, int rows, const float4* twx,
+                                            const float4* r2c, const float2* hw) {
+  constexpr int NXH = C::NXH, SX = C::SX, X1 = C::X1, X2 = C::X2, H = C::ROWS;
+  if constexpr (X2 > 1) {
+  for (int t = threadIdx.x; t < H * C::NU; t += C::TPB) {
+    const int j = t % H, u = t / H;
+    if (j >= rows) continue;
+    float4* p = P + j * SX;
+    const float2 w = hw[j];
+    if (u == 0 || u == X1 / 2) {
+      C2 v[X2], o[X2];
+#pragma unroll
+      for (int i = 0; i < X2; ++i) v[i] = pair_join_rows(c2_load(p + u * X2 + i), w);
+      if (u == 0) {
+        const float2 xm = PACK ? v[0].im : pair_join_rows(c2_load(p + NXH), w).re;
+        o[0] = {f2add(v[0].re, xm), f2sub(v[0].re, xm)};   // from X_0 and X_nx/2, both real
+#pragma unroll
+        for (int i = 1; i < X2; ++i) {
+          const int ip = X2 - i;
+          if (i <= ip) {
+            C2 zk, zm;
+            pair_c2r(v[i], v[ip], r2c + X1 * i, zk, zm);
+            o[i] = zk;
+            if (i < ip) o[ip] = zm;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < X2; ++i) {
+          const int ip = X2 - 1 - i;
+          if (i <= ip) {
+            C2 zk, zm;
+            pair_c2r(v[i], v[ip], r2c + X1 / 2 + X1 * i, zk, zm);
+            o[i] = zk;
+            if (i < ip) o[ip] = zm;
+          }
+        }
+      }
+      PairDft<X2, true>::run(o);
+      c2_store(p + u * X2, o[0]);
+#pragma unroll
+      for (int n2 = 1; n2 < X2; ++n2)
+        c2_store(p + u * X2 + n2, c2_mul<true>(o[n2], twx + u * X2 + n2));
+    } else {
+      const int up = X1 - u;
+      C2 va[X2], vb[X2];
+#pragma unroll
+      for (int i = 0; i < X2; ++i) {
+        va[i] = pair_join_rows(c2_load(p + u * X2 + i), w);
+        vb[i] = pair_join_rows(c2_load(p + up * X2 + i), w);
+      }
+#pragma unroll
+      for (int i = 0; i < X2; ++i) {
+        const int ip = X2 - 1 - i;
+        C2 zk, zm;
+        pair_c2r(va[i], vb[ip], r2c + u + X1 * i, zk, zm);
+        va[i] = zk;
+        vb[ip] = zm;
+      }
+      PairDft<X2, true>::run(va);
+      PairDft<X2, true>::run(vb);
+      c2_store(p + u * X2, va[0]);
+      c2_store(p + up * X2, vb[0]);
+#pragma unroll
+      for (int n2 = 1; n2 < X2; ++n2) {
+        c2_store(p + u * X2 + n2, c2_mul<true>(va[n2], twx + u * X2 + n2));
+        c2_store(p + up * X2 + n2, c2_mul<true>(vb[n2], twx + up * X2 + n2));
+      }
+    }
+  }
   }
 }
 
@@ -372,6 +523,7 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
     k_pair_inv(GridDev g, const float4* __restrict__ spec, float* __restrict__ outp, float scale,
                const float* __restrict__ eps, const float4* __restrict__ post) {
   using C = PairPlane<N>;
+  using X = typename C::X;
   constexpr int NXH = C::NXH, SX = C::SX, H = C::H, PL = C::PL, TPB = C::TPB;
   constexpr int X1 = C::X1, X2 = C::X2, Y1 = C::Y1, Y2 = C::Y2;
   extern __shared__ __align__(128) float4 sm4[];
@@ -448,71 +600,7 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
     for (int i = 0; i < Y1; ++i) c2_store(p + i * Y2 * SX, v[i]);
   }
   __syncthreads();
-  // last radix-2 step along y and the tangling, fused into x step 1 (inverse)
-  for (int t = threadIdx.x; t < H * C::NU; t += TPB) {
-    const int j = t % H, u = t / H;
-    float4* p = P + j * SX;
-    const float2 w = hw[j];
-    if (u == 0 || u == X1 / 2) {
-      C2 v[X2], o[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) v[i] = pair_join_rows(c2_load(p + u * X2 + i), w);
-      if (u == 0) {
-        o[0] = {f2add(v[0].re, v[0].im), f2sub(v[0].re, v[0].im)};   // from (x_DC, x_Nyquist)
-#pragma unroll
-        for (int i = 1; i < X2; ++i) {
-          const int ip = X2 - i;
-          if (i <= ip) {
-            C2 zk, zm;
-            pair_c2r(v[i], v[ip], r2c + X1 * i, zk, zm);
-            o[i] = zk;
-            if (i < ip) o[ip] = zm;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < X2; ++i) {
-          const int ip = X2 - 1 - i;
-          if (i <= ip) {
-            C2 zk, zm;
-            pair_c2r(v[i], v[ip], r2c + X1 / 2 + X1 * i, zk, zm);
-            o[i] = zk;
-            if (i < ip) o[ip] = zm;
-          }
-        }
-      }
-      PairDft<X2, true>::run(o);
-      c2_store(p + u * X2, o[0]);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2)
-        c2_store(p + u * X2 + n2, c2_mul<true>(o[n2], twx + u * X2 + n2));
-    } else {
-      const int up = X1 - u;
-      C2 va[X2], vb[X2];
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        va[i] = pair_join_rows(c2_load(p + u * X2 + i), w);
-        vb[i] = pair_join_rows(c2_load(p + up * X2 + i), w);
-      }
-#pragma unroll
-      for (int i = 0; i < X2; ++i) {
-        const int ip = X2 - 1 - i;
-        C2 zk, zm;
-        pair_c2r(va[i], vb[ip], r2c + u + X1 * i, zk, zm);
-        va[i] = zk;
-        vb[ip] = zm;
-      }
-      PairDft<X2, true>::run(va);
-      PairDft<X2, true>::run(vb);
-      c2_store(p + u * X2, va[0]);
-      c2_store(p + up * X2, vb[0]);
-#pragma unroll
-      for (int n2 = 1; n2 < X2; ++n2) {
-        c2_store(p + u * X2 + n2, c2_mul<true>(va[n2], twx + u * X2 + n2));
-        c2_store(p + up * X2 + n2, c2_mul<true>(vb[n2], twx + up * X2 + n2));
-      }
-    }
-  }
+  pair_x1_inv<X, true>(P, H, twx, r2c, hw);
   __syncthreads();
   constexpr int LOW = H * NXH;         // row j + ny/2 lies LOW float2 after row j
   const size_t nf2 = (size_t)g.n / 2, zoff = (size_t)z * N * NXH;
@@ -641,6 +729,227 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
 // l + 16 holding the normal and the shear components of the same frequencies
 // and exchanging their partial sums of tau_hat n by shuffles; inverse step 2
 // writes back to global memory.
+// ---------------------------------------------------------------------------
+// The same map in five passes, for planes that do not fit in shared memory
+// (256^2) and for nx != ny: x rows, y lines, the z pass, y lines and x rows
+// back.  Same spectrum; the columns 0 and nx/2 are not packed.
+// ---------------------------------------------------------------------------
+
+// x rows, one block per (component, R row pairs, z): both x steps, the rows
+// j and j + ny/2 of a pair side by side; the finished rows leave in one bulk
+// copy.  Inverse: one bulk copy in, both steps, the rows straight to global
+// memory.  Bound by DRAM back (256^3: 182 -> 122 us, one pass over the field
+// and one over the spectrum take 119 us at the copy rate) and by the L1 pipe
+// forward (246 -> 183 us: a normal component reads three strain fields).
+// 160 threads, one round for both x steps, leave room for three blocks an SM
+// instead of four: 200 and 132 us.
+template <int NX, int R>
+struct PairRows {
+    static constexpr int TPB = PairX<NX, R, 1>::X2 == 1 ? (R < 32 ? 32 : R) : 8 * R;
+  static constexpr int MINB = 512 / TPB;
+  using X = PairX<NX, R, TPB>;
+  static size_t smem(bool table) {
+    return (size_t)(R * X::SX + 2 * X::NXH) * sizeof(float4) + R * sizeof(float2) +
+           (table ? 256 * sizeof(float2) : 0);
+  }
+};
+
+template <int NX, int R>
+__global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
+    k_pair_rows_fwd(GridDev g, const float* __restrict__ in, float4* __restrict__ spec, int mode) {
+  using X = typename PairRows<NX, R>::X;
+  constexpr int NXH = X::NXH, SX = X::SX, TPB = X::TPB;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* P = sm4;                     // [R][SX]
+  float4* twx = P + R * SX;
+  float4* r2c = twx + NXH;
+  float2* hw = reinterpret_cast<float2*>(r2c + NXH);
+  float2* dm = hw + R;
+  const int c = blockIdx.x, j0 = blockIdx.y * R, z = blockIdx.z;
+  const int h = g.ny / 2, rows = min(R, h - j0);
+  allow_dependent_launch();
+  for (int i = threadIdx.x; i < NXH; i += TPB) {
+    twx[i] = splat_twiddle(g.p_twx[i]);
+    r2c[i] = splat_twiddle(g.r2c_w[i]);
+  }
+  for (int i = threadIdx.x; i < rows; i += TPB) hw[i] = g.p_hw[j0 + i];
+  grid_dependency_wait();
+  for (int i = threadIdx.x; i < 256; i += TPB) {   // (lam, 2 mu) of C - C0 per phase
+    const float2 m = g.dmat[i];
+    dm[i] = make_float2(m.x, 2.f * m.y);
+  }
+  __syncthreads();
+  const size_t row0 = ((size_t)z * g.ny + j0) * NXH;
+  pair_x1_component<X, false>(g, reinterpret_cast<const float2*>(in) + row0, c,
+                              reinterpret_cast<const uchar2*>(g.phase) + row0, h * NXH, rows,
+                              mode, dm, P, twx, r2c, hw);
+  __syncthreads();
+  pair_x2<X, false>(P, rows, r2c, hw);
+  fence_async_smem();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    bulk_store(spec + (((size_t)c * g.nz + z) * h + j0) * SX, P, (uint32_t)rows * SX * 16);
+    bulk_commit();
+    bulk_wait_all();
+  }
+}
+
+template <int NX, int R>
+__global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
+    k_pair_rows_inv(GridDev g, const float4* __restrict__ spec, float* __restrict__ outp,
+                    float scale, const float* __restrict__ add) {
+  using X = typename PairRows<NX, R>::X;
+  constexpr int NXH = X::NXH, SX = X::SX, TPB = X::TPB, X1 = X::X1, X2 = X::X2;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* P = sm4;
+  float4* twx = P + R * SX;
+  float4* r2c = twx + NXH;
+  float2* hw = reinterpret_cast<float2*>(r2c + NXH);
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ int fail;
+  const int c = blockIdx.x, j0 = blockIdx.y * R, z = blockIdx.z;
+  const int h = g.ny / 2, rows = min(R, h - j0);
+  allow_dependent_launch();
+  if (threadIdx.x == 0) {
+    fail = 0;
+    mbar_init(&bar, 1);
+    mbar_init_fence();
+  }
+  for (int i = threadIdx.x; i < NXH; i += TPB) {
+    twx[i] = splat_twiddle(g.p_twx[i]);
+    r2c[i] = splat_twiddle(g.r2c_w[i]);
+  }
+  for (int i = threadIdx.x; i < rows; i += TPB) hw[i] = g.p_hw[j0 + i];
+  grid_dependency_wait();
+  if (threadIdx.x == 0) {
+    mbar_arrive_expect_tx(&bar, (uint32_t)rows * SX * 16);
+    bulk_load(P, spec + (((size_t)c * g.nz + z) * h + j0) * SX, (uint32_t)rows * SX * 16, &bar);
+  }
+  __syncthreads();
+  if (!mbar_wait(&bar, 0)) fail = 1;
+  __syncthreads();
+  if (fail) {   // the copy never completed: record it and leave the rows alone
+    if (threadIdx.x == 0) {
+      atomicExch(g.err, 1);
+      mbar_wait(&bar, 0);
+    }
+    return;
+  }
+  pair_x1_inv<X, false>(P, rows, twx, r2c, hw);
+  if (X2 > 1) __syncthreads();
+  const size_t nf2 = (size_t)g.n / 2;
+  const int low = h * NXH;
+  const size_t at0 = c * nf2 + ((size_t)z * g.ny + j0) * NXH;
+  float2* out2 = reinterpret_cast<float2*>(outp) + at0;
+  const float2* a2 = reinterpret_cast<const float2*>(add) + at0;
+  for (int q = threadIdx.x; q < R * X2; q += TPB) {   // x step 2 (inverse)
+    int j, n2;
+    pair_row_task<X2, R>(q, j, n2);
+    if (j >= rows) continue;
+    const float4* p = P + j * SX + n2;
+    const int r = j * NXH + n2;
+    C2 v[X1];
+    if constexpr (X2 == 1) {
+      pair_tangle_row<NXH>(p, r2c, hw[j], v);
+    } else {
+#pragma unroll
+      for (int i = 0; i < X1; ++i) v[i] = c2_load(p + i * X2);
+    }
+    PairDft<X1, true>::run(v);
+#pragma unroll
+    for (int i = 0; i < X1; ++i) {
+      float2 a = make_float2(v[i].re.x * scale, v[i].im.x * scale);
+      float2 b = make_float2(v[i].re.y * scale, v[i].im.y * scale);
+      if (add) {
+        const float2 ea = a2[r + i * X2], eb = a2[r + low + i * X2];
+        a = make_float2(a.x + ea.x, a.y + ea.y);
+        b = make_float2(b.x + eb.x, b.y + eb.y);
+      }
+      __stcs(out2 + r + i * X2, a);
+      __stcs(out2 + r + low + i * X2, b);
+    }
+  }
+}
+
+// (Splitting the map into slabs of z planes so that the spectrum of a slab
+// stays in L2 between the x and the y pass loses more at the kernel boundaries
+// than it saves: 256^3 826 us whole, 862 / 929 / 1086 us in slabs of 64 / 32 / 16.)
+
+// y lines of H = ny/2 pairs: T columns of the spectrum per block, numbered
+// over all planes (column = (component, z) plane * (nx/2 + 1) + x slot), so
+// that only the last block is ragged.  The first register step reads global
+// memory, the second writes it; shared memory holds the exchange between the
+// two (none for single-step lengths).
+// T: 256-byte rows forward, 128-byte rows back (256^3: 126 and 122 us a pass;
+// the other way round 139 and 139 us).
+template <int H, bool INV>
+struct PairLines {
+  static constexpr int Y1 = pair_n1(H), Y2 = H / Y1;
+  static constexpr int TPB = 128, T = Y2 == 1 ? TPB : (INV ? 8 : 16), HP = H | 1;
+  static constexpr size_t SMEM = Y2 == 1 ? 0 : (size_t)(T * HP + H) * sizeof(float4);
+};
+
+template <int H, bool INV>
+__global__ void __launch_bounds__(PairLines<H, INV>::TPB, 4)
+    k_pair_lines(GridDev g, float4* __restrict__ spec) {
+  using C = PairLines<H, INV>;
+  constexpr int Y1 = C::Y1, Y2 = C::Y2, T = C::T, TPB = C::TPB, HP = C::HP;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* B = sm4;                     // [T][HP]
+  float4* twy = B + T * HP;
+  const int SX = g.nxh + 1, cols = 6 * g.nz * SX;
+  const int m0 = blockIdx.x * T;
+  allow_dependent_launch();
+  if (Y2 > 1)
+    for (int i = threadIdx.x; i < H; i += TPB) twy[i] = splat_twiddle(g.p_twy[i]);
+  grid_dependency_wait();
+  if (Y2 > 1) __syncthreads();
+  auto column = [&](int t) {   // first element of column m0 + t (rows SX apart)
+    const int m = m0 + t, pl = m / SX;
+    return spec + (size_t)pl * H * SX + (m - pl * SX);
+  };
+  if constexpr (Y2 == 1) {
+    if (m0 + (int)threadIdx.x < cols) {
+      float4* p = column(threadIdx.x);
+      C2 v[Y1];
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) v[i] = c2_load(p + (size_t)i * SX);
+      PairDft<Y1, INV>::run(v);
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) c2_store(p + (size_t)i * SX, v[i]);
+    }
+    return;
+  }
+  constexpr int A1 = INV ? Y2 : Y1, A2 = INV ? Y1 : Y2;   // points of the first, second step
+  for (int q = threadIdx.x; q < T * A2; q += TPB) {   // A2 tasks a column
+    const int t = q % T, k = q / T;   // k: n2 forward, k1 inverse
+    if (m0 + t >= cols) continue;
+    const float4* p = column(t) + (size_t)(INV ? k * Y2 : k) * SX;
+    C2 v[A1];
+#pragma unroll
+    for (int i = 0; i < A1; ++i) v[i] = c2_load(p + (size_t)(INV ? i : i * Y2) * SX);
+    PairDft<A1, INV>::run(v);
+    float4* b = B + t * HP + (INV ? k * Y2 : k);
+    c2_store(b, v[0]);
+#pragma unroll
+    for (int i = 1; i < A1; ++i)
+      c2_store(b + (INV ? i : i * Y2), c2_mul<INV>(v[i], twy + (INV ? k * Y2 + i : i * Y2 + k)));
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < T * A1; q += TPB) {
+    const int t = q % T, k = q / T;   // k: k1 forward, n2 inverse
+    if (m0 + t >= cols) continue;
+    const float4* b = B + t * HP + (INV ? k : k * Y2);
+    C2 v[A2];
+#pragma unroll
+    for (int i = 0; i < A2; ++i) v[i] = c2_load(b + (INV ? i * Y2 : i));
+    PairDft<A2, INV>::run(v);
+    float4* p = column(t) + (size_t)(INV ? k : k * Y2) * SX;
+#pragma unroll
+    for (int i = 0; i < A2; ++i) c2_store(p + (size_t)(INV ? i * Y2 : i) * SX, v[i]);
+  }
+}
+
 // Threads per z block and blocks per SM: with few pencils a block, 192 threads
 // take the first and last z steps in one round (nz = 64, T = 4: 5.6 us, 128
 // threads 7.0 us; nz = 48, T = 2: 4.2 against 4.9 us).
@@ -739,57 +1048,47 @@ __device__ __forceinline__ void pair_green_special(const PairFreq& f, bool full,
   }
 }
 
-template <int NZ, int T>
-__global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
-    k_pair_green(GridDev g, float4* __restrict__ spec, int mode, GammaArgs ga) {
+// All six components at one frequency: o = -Gamma0_hat : a.
+__device__ __forceinline__ void pair_green_all(const PairFreq& f, const C2* a, bool full,
+                                               const GammaArgs& ga, C2* o) {
+  const C2 p1 = pair_dot3(a[0], f.n1, a[5], f.n2, a[4], f.n3);
+  const C2 p2 = pair_dot3(a[5], f.n1, a[1], f.n2, a[3], f.n3);
+  const C2 p3 = pair_dot3(a[4], f.n1, a[3], f.n2, a[2], f.n3);
+  pair_green_w<0>(f, p1, p2, p3, ga, o);
+  pair_green_w<1>(f, p1, p2, p3, ga, o + 3);
+  if (f.special) {
+    pair_green_special(f, full, ga.En, o);
+    pair_green_special(f, full, ga.En + 3, o + 3);
+  }
+}
+
+// Wave vector of pencil pair m: *pen = (xi_x, xi_y even, xi_y odd, 0); *flag:
+// bits 0-1, 2-3 count the non-zero (x, y) components of the even and the odd
+// line, bits 4, 5 are their x or y Nyquist flags.
+__device__ __forceinline__ void pair_pencil(const GridDev& g, int m, int plane, float4* pen,
+                                            int* flag) {
+  float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+  int f = 0;
+  if (m < plane) {
+    const int sxn = g.nxh + 1, j = m / sxn, sx = m - j * sxn;
+    const int2 fx = g.p_fx[sx];
+    const int4 fy = g.p_fy[j];
+    q = make_float4(fx.x * g.inv_lx, fy.x * g.inv_ly, fy.z * g.inv_ly, 0.f);
+    f = ((fx.x != 0) + (fy.x != 0)) | (((fx.x != 0) + (fy.z != 0)) << 2) |
+        ((fx.y | fy.y) << 4) | ((fx.y | fy.w) << 5);
+  }
+  *pen = q;
+  *flag = f;
+}
+
+// Forward z step 2, the Green operator and inverse step 1 on the T pencil
+// pairs of a block (layout of PairZ), in place.
+template <int NZ, int T, int TPB>
+__device__ __forceinline__ void pair_z_middle(const GridDev& g, float4* B, const float4* twz,
+                                              const float4* pen, const int* flag, int mode,
+                                              const GammaArgs& ga) {
   using C = PairZ<NZ, T>;
-  constexpr int Z1 = C::Z1, Z2 = C::Z2, Z2P = C::Z2P, TS = C::TS, CS = C::CS, TPB = C::TPB;
-  extern __shared__ __align__(128) float4 sm4[];
-  float4* B = sm4;
-  float4* twz = B + 6 * CS;            // [Z1][Z2]
-  __shared__ float4 pen[T];            // (xi_x, xi_y even, xi_y odd, 0)
-  __shared__ int flag[T];              // non-zero components and Nyquist bits, see below
-  const int m0 = blockIdx.x * T;
-  const int sxn = g.nxh + 1, plane = (g.ny / 2) * sxn;   // pencil pairs
-  allow_dependent_launch();
-  for (int i = threadIdx.x; i < NZ; i += TPB) twz[i] = splat_twiddle(g.p_twz[i]);
-  if (threadIdx.x < T) {
-    const int m = m0 + threadIdx.x;
-    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-    int f = 0;
-    if (m < plane) {
-      const int j = m / sxn, sx = m - j * sxn;
-      const int2 fx = g.p_fx[sx];
-      const int4 fy = g.p_fy[j];
-      q = make_float4(fx.x * g.inv_lx, fy.x * g.inv_ly, fy.z * g.inv_ly, 0.f);
-      // bits 0-1, 2-3: count of non-zero (x, y) components of the even, odd
-      // line; bits 4, 5: their x or y Nyquist flags
-      f = ((fx.x != 0) + (fy.x != 0)) | (((fx.x != 0) + (fy.z != 0)) << 2) |
-          ((fx.y | fy.y) << 4) | ((fx.y | fy.w) << 5);
-    }
-    pen[threadIdx.x] = q;
-    flag[threadIdx.x] = f;
-  }
-  grid_dependency_wait();
-  __syncthreads();
-  // forward step 1; task q -> (pencil t fastest, then component, then n2)
-  for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {
-    const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
-    const int m = m0 + t;
-    const float4* src = spec + ((size_t)c * NZ + n2) * plane + m;
-    const size_t zs = (size_t)Z2 * plane;
-    C2 v[Z1];
-#pragma unroll
-    for (int i = 0; i < Z1; ++i)
-      v[i] = m < plane ? c2_load(src + i * zs) : C2{f2splat(0.f), f2splat(0.f)};
-    PairDft<Z1, false>::run(v);
-    float4* p = B + c * CS + t * TS + n2;
-    c2_store(p, v[0]);
-#pragma unroll
-    for (int k1 = 1; k1 < Z1; ++k1)
-      c2_store(p + k1 * Z2P, Z2 > 1 ? c2_mul<false>(v[k1], twz + k1 * Z2 + n2) : v[k1]);
-  }
-  __syncthreads();
+  constexpr int Z1 = C::Z1, Z2 = C::Z2, Z2P = C::Z2P, TS = C::TS, CS = C::CS;
   if constexpr (Z2 > 8) {
     // three components of a 16-point middle step do not fit a thread's
     // registers: forward step 2, Green operator and inverse step 1 separately
@@ -811,16 +1110,8 @@ __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
       C2 a[6];
 #pragma unroll
       for (int c = 0; c < 6; ++c) a[c] = c2_load(p + c * CS);
-      const C2 p1 = pair_dot3(a[0], f.n1, a[5], f.n2, a[4], f.n3);
-      const C2 p2 = pair_dot3(a[5], f.n1, a[1], f.n2, a[3], f.n3);
-      const C2 p3 = pair_dot3(a[4], f.n1, a[3], f.n2, a[2], f.n3);
       C2 o[6];
-      pair_green_w<0>(f, p1, p2, p3, ga, o);
-      pair_green_w<1>(f, p1, p2, p3, ga, o + 3);
-      if (f.special) {
-        pair_green_special(f, mode == GM_FULL_MAP, ga.En, o);
-        pair_green_special(f, mode == GM_FULL_MAP, ga.En + 3, o + 3);
-      }
+      pair_green_all(f, a, mode == GM_FULL_MAP, ga, o);
 #pragma unroll
       for (int c = 0; c < 6; ++c) c2_store(p + c * CS, o[c]);
     }
@@ -890,6 +1181,44 @@ __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
     }
   }
   }
+}
+
+template <int NZ, int T>
+__global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
+    k_pair_green(GridDev g, float4* __restrict__ spec, int mode, GammaArgs ga) {
+  using C = PairZ<NZ, T>;
+  constexpr int Z1 = C::Z1, Z2 = C::Z2, Z2P = C::Z2P, TS = C::TS, CS = C::CS, TPB = C::TPB;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* B = sm4;
+  float4* twz = B + 6 * CS;            // [Z1][Z2]
+  __shared__ float4 pen[T];            // see pair_pencil
+  __shared__ int flag[T];
+  const int m0 = blockIdx.x * T;
+  const int plane = (g.ny / 2) * (g.nxh + 1);   // pencil pairs
+  allow_dependent_launch();
+  for (int i = threadIdx.x; i < NZ; i += TPB) twz[i] = splat_twiddle(g.p_twz[i]);
+  if (threadIdx.x < T) pair_pencil(g, m0 + threadIdx.x, plane, pen + threadIdx.x, flag + threadIdx.x);
+  grid_dependency_wait();
+  __syncthreads();
+  // forward step 1; task q -> (pencil t fastest, then component, then n2)
+  for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {
+    const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
+    const int m = m0 + t;
+    const float4* src = spec + ((size_t)c * NZ + n2) * plane + m;
+    const size_t zs = (size_t)Z2 * plane;
+    C2 v[Z1];
+#pragma unroll
+    for (int i = 0; i < Z1; ++i)
+      v[i] = m < plane ? c2_load(src + i * zs) : C2{f2splat(0.f), f2splat(0.f)};
+    PairDft<Z1, false>::run(v);
+    float4* p = B + c * CS + t * TS + n2;
+    c2_store(p, v[0]);
+#pragma unroll
+    for (int k1 = 1; k1 < Z1; ++k1)
+      c2_store(p + k1 * Z2P, Z2 > 1 ? c2_mul<false>(v[k1], twz + k1 * Z2 + n2) : v[k1]);
+  }
+  __syncthreads();
+  pair_z_middle<NZ, T, TPB>(g, B, twz, pen, flag, mode, ga);
   __syncthreads();
   for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {   // inverse step 2 -> global
     const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
@@ -908,9 +1237,135 @@ __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
   }
 }
 
+// The z pass of up to four planes (a 2D cell: one): a thread holds its pencil
+// pair's six lines; no shared memory (256 x 256 x 1: 4.7 -> 2.6 us a pass).
+constexpr int kShortTPB = 64;
+template <int NZ>
+__global__ void __launch_bounds__(kShortTPB) k_pair_green_short(GridDev g,
+                                                                float4* __restrict__ spec, int mode,
+                                                                GammaArgs ga) {
+  const int plane = (g.ny / 2) * (g.nxh + 1), m = blockIdx.x * kShortTPB + threadIdx.x;
+  allow_dependent_launch();
+  float4 q;
+  int fl;
+  pair_pencil(g, m, plane, &q, &fl);
+  grid_dependency_wait();
+  if (m >= plane) return;
+  C2 v[6][NZ];
+#pragma unroll
+  for (int c = 0; c < 6; ++c)
+#pragma unroll
+    for (int i = 0; i < NZ; ++i) v[c][i] = c2_load(spec + ((size_t)c * NZ + i) * plane + m);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) PairDft<NZ, false>::run(v[c]);
+#pragma unroll
+  for (int k = 0; k < NZ; ++k) {
+    const PairFreq f = pair_freq_vector<NZ>(g, q, fl, k);
+    C2 a[6], o[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) a[c] = v[c][k];
+    pair_green_all(f, a, mode == GM_FULL_MAP, ga, o);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) v[c][k] = o[c];
+  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    PairDft<NZ, true>::run(v[c]);
+#pragma unroll
+    for (int i = 0; i < NZ; ++i) c2_store(spec + ((size_t)c * NZ + i) * plane + m, v[c][i]);
+  }
+}
+
+// The z pass for lines whose tile fills an SM (nz = 256): one persistent block
+// per SM; the next tile travels into a raw buffer [6][nz][T] by 16-byte
+// asynchronous copies while the present one is transformed in the work buffer
+// (the layout of PairZ).  Two resident blocks of k_pair_green hide less of the
+// loads (256^3: 298 us a pass, this one 238 us; T = 2 with two blocks 296 us).
+// At nz = 128, where three blocks fit, k_pair_green is the faster one (28.5
+// against 33.8 us).  The last and first steps have 6 T 16 tasks, the threads.
+template <int NZ, int T>
+struct PairZStream {
+  using Z = PairZ<NZ, T>;
+  static constexpr int TPB = 6 * T * Z::Z2, RAW = 6 * NZ * T;
+  static constexpr size_t SMEM = (size_t)(RAW + 6 * Z::CS + NZ) * sizeof(float4);
+};
+
+template <int NZ, int T>
+__global__ void __launch_bounds__(PairZStream<NZ, T>::TPB, 1)
+    k_pair_green_stream(GridDev g, float4* __restrict__ spec, int mode, GammaArgs ga) {
+  using C = PairZ<NZ, T>;
+  constexpr int Z1 = C::Z1, Z2 = C::Z2, Z2P = C::Z2P, TS = C::TS, CS = C::CS;
+  constexpr int TPB = PairZStream<NZ, T>::TPB, RAW = PairZStream<NZ, T>::RAW;
+  extern __shared__ __align__(128) float4 sm4[];
+  float4* raw = sm4;                   // [6][NZ][T]
+  float4* B = raw + RAW;
+  float4* twz = B + 6 * CS;            // [Z1][Z2]
+  __shared__ float4 pen[T];
+  __shared__ int flag[T];
+  const int plane = (g.ny / 2) * (g.nxh + 1), tiles = (plane + T - 1) / T;
+  allow_dependent_launch();
+  for (int i = threadIdx.x; i < NZ; i += TPB) twz[i] = splat_twiddle(g.p_twz[i]);
+  grid_dependency_wait();
+  auto prefetch = [&](int tile) {
+    for (int q = threadIdx.x; q < RAW; q += TPB) {
+      const int t = q % T, cz = q / T;
+      if (tile * T + t < plane) async_copy16(raw + q, spec + (size_t)cz * plane + tile * T + t);
+    }
+    async_copy_commit();
+  };
+  prefetch(blockIdx.x);
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int m0 = tile * T;
+    if (threadIdx.x < T) pair_pencil(g, m0 + threadIdx.x, plane, pen + threadIdx.x, flag + threadIdx.x);
+    async_copy_wait();
+    __syncthreads();
+    for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {   // forward step 1
+      const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
+      const float4* src = raw + (c * NZ + n2) * T + t;
+      C2 v[Z1];
+#pragma unroll
+      for (int i = 0; i < Z1; ++i) v[i] = c2_load(src + i * Z2 * T);
+      PairDft<Z1, false>::run(v);
+      float4* p = B + c * CS + t * TS + n2;
+      c2_store(p, v[0]);
+#pragma unroll
+      for (int k1 = 1; k1 < Z1; ++k1) c2_store(p + k1 * Z2P, c2_mul<false>(v[k1], twz + k1 * Z2 + n2));
+    }
+    __syncthreads();
+    if (tile + (int)gridDim.x < tiles) prefetch(tile + gridDim.x);
+    pair_z_middle<NZ, T, TPB>(g, B, twz, pen, flag, mode, ga);
+    __syncthreads();
+    for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {   // inverse step 2 -> global
+      const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
+      const float4* p = B + c * CS + t * TS + n2;
+      C2 v[Z1];
+#pragma unroll
+      for (int i = 0; i < Z1; ++i) v[i] = c2_load(p + i * Z2P);
+      PairDft<Z1, true>::run(v);
+      if (m0 + t < plane) {
+        float4* dst = spec + ((size_t)c * NZ + n2) * plane + m0 + t;
+        const size_t zs = (size_t)Z2 * plane;
+#pragma unroll
+        for (int i = 0; i < Z1; ++i) c2_store(dst + i * zs, v[i]);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 148;
+    return v;
+  }();
+  return n;
+}
+
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   if (bytes <= 48 * 1024) return cudaSuccess;
@@ -953,11 +1408,72 @@ cudaError_t launch_inv_post(const GridDev& g, float* out, const float4* spec, co
                             g, spec, out, 0.5f / (float)g.n, eps, post);
 }
 
+// Row pairs per block: enough for four blocks an SM, or few where the grid is small.
+template <int NX>
+struct RowsTile {
+  static constexpr bool ONE = PairX<NX, 1, 1>::X2 == 1;
+  static constexpr int BIG = ONE ? 64 : 16, SMALL = ONE ? 16 : 4;
+};
+
+template <int NX, int R>
+cudaError_t launch_rows_r(const GridDev& g, const float* in, float* out, float4* spec, int mode,
+                          bool inv, const float* add, cudaStream_t st) {
+  using C = PairRows<NX, R>;
+  const dim3 grid(6, (g.ny / 2 + R - 1) / R, g.nz);
+  const size_t smem = C::smem(!inv);
+  cudaError_t e;
+  if (inv) {
+    if ((e = set_smem(k_pair_rows_inv<NX, R>, smem)) != cudaSuccess) return e;
+    return launch_pdl(k_pair_rows_inv<NX, R>, grid, C::TPB, smem, st, g, (const float4*)spec, out,
+                      0.5f / (float)g.n, add);
+  }
+  if ((e = set_smem(k_pair_rows_fwd<NX, R>, smem)) != cudaSuccess) return e;
+  return launch_pdl(k_pair_rows_fwd<NX, R>, grid, C::TPB, smem, st, g, in, spec, mode);
+}
+
+template <int NX>
+cudaError_t launch_rows(const GridDev& g, const float* in, float* out, float4* spec, int mode,
+                        bool inv, const float* add, cudaStream_t st) {
+  using T = RowsTile<NX>;
+  if ((long long)6 * g.nz * (g.ny / 2) >= 600LL * T::BIG)
+    return launch_rows_r<NX, T::BIG>(g, in, out, spec, mode, inv, add, st);
+  return launch_rows_r<NX, T::SMALL>(g, in, out, spec, mode, inv, add, st);
+}
+
+template <int H, bool INV>
+cudaError_t launch_lines(const GridDev& g, float4* spec, cudaStream_t st) {
+  using C = PairLines<H, INV>;
+  cudaError_t e = set_smem(k_pair_lines<H, INV>, C::SMEM);
+  if (e != cudaSuccess) return e;
+  const int cols = 6 * g.nz * (g.nxh + 1);
+  const dim3 grid((cols + C::T - 1) / C::T);
+  // Next to a z block that takes most of an SM's shared memory (nz = 256) the
+  // lines that start early run with what L1 is left of it: 256^3 990 us a map
+  // so, 837 us with an ordinary launch after the z pass, 827 us with one
+  // before it too (a loss on smaller grids, 96 x 48 x 256: 75.8 against 77.7 us).
+  if (g.nz >= 256 && (INV || g.n >= 1 << 23)) {
+    k_pair_lines<H, INV><<<grid, C::TPB, C::SMEM, st>>>(g, spec);
+    return cudaGetLastError();
+  }
+  return launch_pdl(k_pair_lines<H, INV>, grid, C::TPB, C::SMEM, st, g, spec);
+}
+
 template <int NZ, int T>
 cudaError_t launch_green(const GridDev& g, float4* spec, int mode, const GammaArgs& ga,
                          cudaStream_t st) {
   using C = PairZ<NZ, T>;
-  if constexpr (C::SMEM <= 227 * 1024) {
+  if constexpr (NZ <= 4) {
+    const int pencils = (g.ny / 2) * (g.nxh + 1);
+    return launch_pdl(k_pair_green_short<NZ>, dim3((pencils + kShortTPB - 1) / kShortTPB), kShortTPB,
+                      0, st, g, spec, mode, ga);
+  } else if constexpr (NZ == 256 && T == 4) {
+    using S = PairZStream<NZ, T>;
+    cudaError_t e = set_smem(k_pair_green_stream<NZ, T>, S::SMEM);
+    if (e != cudaSuccess) return e;
+    const int pencils = (g.ny / 2) * (g.nxh + 1), tiles = (pencils + T - 1) / T;
+    return launch_pdl(k_pair_green_stream<NZ, T>, dim3(std::min(tiles, sm_count())), S::TPB,
+                      S::SMEM, st, g, spec, mode, ga);
+  } else if constexpr (C::SMEM <= 227 * 1024) {
     cudaError_t e = set_smem(k_pair_green<NZ, T>, C::SMEM);
     if (e != cudaSuccess) return e;
     const int pencils = (g.ny / 2) * (g.nxh + 1);
@@ -1004,6 +1520,28 @@ cudaError_t pass_green(const GridDev& g, float4* spec, int mode, const double E[
   }
 }
 
+#define RPM_XY_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
+
+cudaError_t pass_rows(const GridDev& g, const float* in, float* out, float4* spec, int mode,
+                      bool inv, const float* add, cudaStream_t st) {
+  switch (g.nx) {
+#define RPM_CASE(N) case N: return launch_rows<N>(g, in, out, spec, mode, inv, add, st);
+    RPM_XY_SIZES(RPM_CASE)
+#undef RPM_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t pass_lines(const GridDev& g, float4* spec, bool inv, cudaStream_t st) {
+  switch (g.ny) {
+#define RPM_CASE(N) \
+  case N: return inv ? launch_lines<N / 2, true>(g, spec, st) : launch_lines<N / 2, false>(g, spec, st);
+    RPM_XY_SIZES(RPM_CASE)
+#undef RPM_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 }  // namespace
 
 bool pair_plane_ok(const GridDev& g, const float2* spec) {
@@ -1044,6 +1582,17 @@ cudaError_t launch_pair_map(const GridDev& g, const float* in, float* out, float
 #undef RPM_CASE
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_pair_rows_map(const GridDev& g, const float* in, float* out, float2* spec,
+                                 const double E[6], int mode, cudaStream_t st, const float* add) {
+  float4* s4 = reinterpret_cast<float4*>(spec);
+  cudaError_t e;
+  if ((e = pass_rows(g, in, nullptr, s4, mode, false, nullptr, st)) != cudaSuccess) return e;
+  if ((e = pass_lines(g, s4, false, st)) != cudaSuccess) return e;
+  if ((e = pass_green(g, s4, mode, E, st)) != cudaSuccess) return e;
+  if ((e = pass_lines(g, s4, true, st)) != cudaSuccess) return e;
+  return pass_rows(g, nullptr, out, s4, mode, true, add, st);
 }
 
 cudaError_t launch_pair_polarization(const GridDev& g, const float4* post, const float* in,

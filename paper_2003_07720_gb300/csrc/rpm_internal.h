@@ -71,6 +71,9 @@ int pair_z_tile(const GridDev& g);                          // pencil pairs per 
 // launch_apply_gamma / launch_polarization_map on such a grid (float2-aligned fields)
 cudaError_t launch_pair_map(const GridDev& g, const float* in, float* out, float2* spec,
                             const double E[6], int mode, cudaStream_t st, const float* add);
+// the same in five passes, any supported grid
+cudaError_t launch_pair_rows_map(const GridDev& g, const float* in, float* out, float2* spec,
+                                 const double E[6], int mode, cudaStream_t st, const float* add);
 cudaError_t launch_pair_polarization(const GridDev& g, const float4* post, const float* in,
                                      float* out, float2* spec, const double Eb[6], int mode,
                                      cudaStream_t st);

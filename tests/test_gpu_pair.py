@@ -1,5 +1,5 @@
-"""The paired kernels (square planes of side 48-128) against the FP64 oracle
-over the z lengths and options their z pass distinguishes: single-step and
+"""The paired kernels (square planes of side 48-128, and the five-pass form on
+any grid) against the FP64 oracle over the z lengths and options their z pass distinguishes: single-step and
 two-step lengths, each number of pencils per block, a ragged last block,
 non-unit cell lengths, a material table of more than two phases."""
 import numpy as np
@@ -22,22 +22,38 @@ def _cell(shape, seed):
                    mu=np.array(mu), lam0=l0, mu0=m0)
 
 
-@pytest.mark.parametrize("nz,n", [(1, 128), (2, 64), (3, 96), (4, 48), (6, 64), (8, 48), (12, 96),
-                                  (16, 64), (24, 48), (32, 48), (48, 96), (64, 48), (96, 48),
-                                  (128, 96), (256, 64)])
-@pytest.mark.parametrize("pencil", [0, 1, 2])
-def test_paired_map_matches_oracle(nz, n, pencil):
+def _check(shape, pencil, plane):
     from paper_2003_07720_gb300 import rpm
-    cell = _cell((nz, n, n), 100 * nz + n)
+    nz, ny, nx = shape
+    cell = _cell(shape, 100 * nz + nx)
     lengths = (0.7, 1.0, 1.3)
     E = np.array([0.3, -0.2, 0.1, 0.05, -0.04, 0.07])
-    x = np.random.Generator(np.random.PCG64(nz)).standard_normal((6, nz, n, n)).astype(np.float32)
-    out = torch.full((6, nz, n, n), float("nan"), device="cuda")
-    opts = rpm.rpm_default_options(p_max=0, pencil_variant=pencil)
+    x = np.random.Generator(np.random.PCG64(nz)).standard_normal((6,) + shape).astype(np.float32)
+    out = torch.full((6,) + shape, float("nan"), device="cuda")
+    opts = rpm.rpm_default_options(p_max=0, pencil_variant=pencil, plane_variant=plane)
     with rpm.Context(cell, opts, lengths=lengths) as ctx:
-        assert rpm.rpm_plane_variant(ctx.handle) == 0
+        assert rpm.rpm_plane_variant(ctx.handle) == plane
         ctx.apply_gamma(torch.from_numpy(x).cuda(), E, out)
     got = out.cpu().numpy().astype(np.float64)
     prob = o.Problem(cell.phase, cell.lam, cell.mu, cell.lam0, cell.mu0, lengths=lengths)
     ref = o.apply_F(prob, x.astype(np.float64), E)
     assert np.linalg.norm(got - ref) / np.linalg.norm(ref) < TOL
+
+
+@pytest.mark.parametrize("nz,n", [(1, 128), (2, 64), (3, 96), (4, 48), (6, 64), (8, 48), (12, 96),
+                                  (16, 64), (24, 48), (32, 48), (48, 96), (64, 48), (96, 48),
+                                  (128, 96), (256, 64)])
+@pytest.mark.parametrize("pencil", [0, 1, 2])
+def test_paired_map_matches_oracle(nz, n, pencil):
+    _check((nz, n, n), pencil, 0)
+
+
+@pytest.mark.parametrize("shape", [
+    # every x length with few and with many rows; ragged last row and column blocks
+    (2, 8, 4), (64, 256, 4), (3, 4, 6), (12, 16, 8), (6, 6, 12), (4, 24, 16), (16, 96, 24),
+    (64, 128, 32), (24, 96, 48), (8, 12, 64), (48, 64, 96), (4, 96, 128), (1, 256, 256),
+    # every y length; nz = 256, whose z pass is persistent, with a ragged last tile
+    (32, 4, 48), (128, 6, 16), (96, 8, 24), (24, 32, 8), (256, 48, 12), (256, 64, 128)])
+@pytest.mark.parametrize("pencil", [0, 2])
+def test_five_passes_match_oracle(shape, pencil):
+    _check(shape, pencil, 2)
