@@ -35,11 +35,17 @@
 
 #include <cuda_bf16.h>
 
+#include "async_copy.cuh"
+#include "pair_fft.cuh"
 #include "rpm.h"
 #include "rpm_fno.h"
 #include "rpm_internal.h"
 
 namespace {
+
+using rpm::allow_dependent_launch;
+using rpm::grid_dependency_wait;
+using rpm::launch_pdl;
 
 constexpr int W = RPM_FNO_WIDTH;   // channels of the hidden layers
 constexpr int CV = 2;              // voxel features (the network's input channels)
@@ -277,6 +283,8 @@ struct XyTc {
 size_t xy_tc_smem(int N, int m) { return XyTc(N, m).bytes(N); }
 
 // Templated on the grid side so that the index arithmetic divides by constants.
+// gridDim.z blocks share the channels of a plane where planes alone would leave
+// SMs idle (see launch_xy_fwd).
 template <int N>
 __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restrict__ src,
                                                         float2* __restrict__ dst,
@@ -291,8 +299,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restri
   float* Ds = reinterpret_cast<float*>(XT + (size_t)c.G * c.MPY * c.KPB);   // [G][MY][MPY]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int z = blockIdx.x, b = blockIdx.y;
+  const int per = W / gridDim.z;       // channels of this block
   const long long NN = (long long)N * N;
   float2* d = dst + ((long long)b * N + z) * ncol * W;
+  allow_dependent_launch();
   for (int i = tid; i < c.NX2 * N; i += kThreads) {
     const int r = i / N, x = i - r * N, kx = r >> 1;
     float v = 0.f;
@@ -319,7 +329,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restri
   }
   const int nmt = N / 16, nnt = c.NX2 / 8;          // x-stage tiles per channel
   const int ymt = c.MY / 16, ynt = c.MPY / 8;        // y-stage tiles per channel
-  for (int c0 = 0; c0 < W; c0 += c.G) {
+  grid_dependency_wait();
+  for (int c0 = blockIdx.z * per; c0 < (int)(blockIdx.z + 1) * per; c0 += c.G) {
     __syncthreads();   // tables written; the previous group's readers are done
     for (int i = tid; i < c.G * N * N / 4; i += kThreads) {
       const int g = i / (N * N / 4), r = i - g * (N * N / 4);
@@ -383,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restri
 
 size_t spec_smem(int N, int m) {
   const size_t m2 = 2 * m;
-  return (m2 * W * W + (size_t)N * W + 3 * m2 * W + N + (size_t)N * m2) * sizeof(float2);
+  return (m2 * W * W + (size_t)N * W + 3 * m2 * W + (size_t)N * m2) * sizeof(float2);
 }
 
 // Tz[z][kz_i] = exp(-2 pi i kz z / N) for the kept kz (the inverse uses the conjugate).
@@ -395,19 +406,16 @@ __device__ __forceinline__ void z_table(const float2* twg, float2* Tz, int N, in
 }
 
 // z transform of the column's [N][W] values to the 2m kept kz: out[kz_i][c].
-__device__ __forceinline__ void z_dft(const float2* a, const float2* tw, float2* out, int N, int m,
+__device__ __forceinline__ void z_dft(const float2* a, const float2* Tz, float2* out, int N, int m,
                                       float scale) {
   for (int o = threadIdx.x; o < 2 * m * W; o += kThreads) {
     const int kzi = o / W, c = o % W;
-    const int kz = kfreq(kzi, m, N);
     float re = 0.f, im = 0.f;
-    int j = 0;
+#pragma unroll 8
     for (int z = 0; z < N; ++z) {
-      const float2 v = a[z * W + c], t = tw[j];
+      const float2 v = a[z * W + c], t = Tz[z * 2 * m + kzi];
       re += v.x * t.x - v.y * t.y;
       im += v.x * t.y + v.y * t.x;
-      j += kz;
-      if (j >= N) j -= N;
     }
     out[o] = make_float2(scale * re, scale * im);
   }
@@ -420,6 +428,7 @@ __device__ __forceinline__ void z_idft(const float2* U, const float2* Tz, float2
     const int z = o / W, c = o % W;
     float re = 0.f, im = 0.f;
     const float2* tz = Tz + z * 2 * m;
+#pragma unroll 8
     for (int kzi = 0; kzi < 2 * m; ++kzi) {
       const float2 u = U[kzi * W + c], t = tz[kzi];
       re += u.x * t.x + u.y * t.y;   // u * conj(t)
@@ -429,7 +438,8 @@ __device__ __forceinline__ void z_idft(const float2* U, const float2* Tz, float2
   }
 }
 
-// A2 [B][N][ncol][W] -> V (saved, [ncol][B][2m][W]), U = V R, Bz [B][N][ncol][W].
+// A2 [B][N][ncol][W] -> V (saved in Vs [ncol][B][2m][W] unless null), U = V R,
+// Bz [B][N][ncol][W].
 __global__ void __launch_bounds__(kThreads) k_spec_fwd(const float2* __restrict__ A2,
                                                        const float2* __restrict__ R,
                                                        float2* __restrict__ Vs,
@@ -442,21 +452,19 @@ __global__ void __launch_bounds__(kThreads) k_spec_fwd(const float2* __restrict_
   float2* a = Rs + m2 * W * W;      // [z][c]
   float2* V = a + N * W;            // [kz_i][c]
   float2* U = V + m2 * W;
-  float2* tw = U + 2 * m2 * W;
-  float2* Tz = tw + N;
+  float2* Tz = U + 2 * m2 * W;
   const int b = blockIdx.y;   // one sample per block
   const float4* r4 = (const float4*)(R + (long long)col * m2 * W * W);
   for (int i = tid; i < m2 * W * W / 2; i += kThreads) ((float4*)Rs)[i] = r4[i];
-  for (int i = tid; i < N; i += kThreads) tw[i] = twg[i];
   z_table(twg, Tz, N, m);
   for (int i = tid; i < N * W; i += kThreads)
     a[i] = A2[((long long)b * N + i / W) * ncol * W + col * W + i % W];
   __syncthreads();
-  z_dft(a, tw, V, N, m, 1.f);
+  z_dft(a, Tz, V, N, m, 1.f);
   __syncthreads();
-  float2* vs = Vs + ((long long)col * B + b) * m2 * W;
+  float2* vs = Vs ? Vs + ((long long)col * B + b) * m2 * W : nullptr;
   for (int o = tid; o < m2 * W; o += kThreads) {
-    vs[o] = V[o];
+    if (vs) vs[o] = V[o];
     const int kzi = o / W, oc = o % W;
     float re = 0.f, im = 0.f;
 #pragma unroll
@@ -472,32 +480,45 @@ __global__ void __launch_bounds__(kThreads) k_spec_fwd(const float2* __restrict_
 }
 
 // Tensor-core form of k_spec_fwd (RPM_FNO_BF16, N % 16 == 0): one block per
-// kept (ky, kx) column and all samples, in groups of 16.  Per sample, the z
-// transform to the kept kz is a BF16 product (rows Re / Im of each kz, K = 2N
+// kept (ky, kx) column and all samples, in groups of up to 16.  Per sample, the
+// z transform to the kept kz is a BF16 product (rows Re / Im of each kz, K = 2N
 // over (z, re/im)); the channel mixing of each kz is a BF16 product over the
 // group (M = 16 samples, K = 32 over (i, re/im), N = 32 over (o, re/im), the
 // real form of the complex R[kz]); the inverse z transform is again a product
 // (rows Re / Im of each z, K over (kz, re/im)).  float32 accumulation; the
-// forward spectra V are kept in float32 for the backward pass.
+// forward spectra V are kept in float32 for the backward pass (Vs non-null).
+// A product row depends on its own sample only, so rows past the group's
+// GB = min(16, B) samples repeat the last one and are not stored.
+// With one or two samples the block waits for its weights (49 KB at 12 modes,
+// read once): they travel to shared memory by asynchronous copies from the
+// start (`stage`).
 template <int N>
 struct SpecTc {
-  int m2, KPZ, MZ, KZB, KIB, MB;
-  __host__ __device__ SpecTc(int m) {
+  int m2, KPZ, MZ, KZB, KIB, MB, GB;
+  bool stage;
+  __host__ __device__ SpecTc(int m, int B) {
     m2 = 2 * m;
     KPZ = round_up(2 * m, 8);   // kz rows per part
     MZ = 2 * KPZ;
     KZB = 2 * N + 8;            // row stride of Az and BTa
     KIB = 2 * KPZ + 8;          // row stride of Ainv and BTU
     MB = 32 + 8;                // row stride of the mixing operand
+    GB = B < 16 ? B : 16;
+    stage = B <= 2;
   }
   __host__ __device__ size_t bytes() const {
     return (size_t)2 * ((size_t)MZ * KZB + (size_t)2 * N * KIB + (size_t)W * KZB +
-                        (size_t)KPZ * 16 * MB + (size_t)16 * W * KIB) +
-           (size_t)4 * ((size_t)MZ * 16 + (size_t)2 * N * 16);
+                        (size_t)KPZ * GB * MB + (size_t)GB * W * KIB) +
+           (size_t)4 * ((size_t)MZ * 16 + (size_t)2 * N * 16) +
+           (stage ? (size_t)m2 * W * W * sizeof(float2) : 0);
   }
 };
 template <int N>
-size_t spec_tc_smem(int m) { return SpecTc<N>(m).bytes(); }
+size_t spec_tc_max() {
+  return std::max(SpecTc<N>(kMaxModes, 2).bytes(), SpecTc<N>(kMaxModes, 16).bytes());
+}
+template <int N>
+size_t spec_tc_smem(int m, int B) { return SpecTc<N>(m, B).bytes(); }
 
 template <int N>
 __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __restrict__ A2,
@@ -507,17 +528,25 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
                                                           const float2* __restrict__ twg, int m,
                                                           int B) {
   extern __shared__ float4 smem4[];
-  const SpecTc<N> c(m);
+  const SpecTc<N> c(m, B);
   const int m2 = c.m2, ncol = 2 * m * m, col = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint16_t* Az = reinterpret_cast<uint16_t*>(smem4);       // [MZ][KZB]
+  float2* Rs = reinterpret_cast<float2*>(smem4);             // [m2][W][W] when staged
+  uint16_t* Az = reinterpret_cast<uint16_t*>(Rs + (c.stage ? m2 * W * W : 0));   // [MZ][KZB]
   uint16_t* Ainv = Az + (size_t)c.MZ * c.KZB;                // [2N][KIB]
   uint16_t* BTa = Ainv + (size_t)2 * N * c.KIB;              // [W][KZB]
-  uint16_t* Vm = BTa + (size_t)W * c.KZB;                    // [KPZ][16][MB]
-  uint16_t* BTU = Vm + (size_t)c.KPZ * 16 * c.MB;            // [16][W][KIB]
-  float* Dz = reinterpret_cast<float*>(BTU + (size_t)16 * W * c.KIB);   // [MZ][16]
+  uint16_t* Vm = BTa + (size_t)W * c.KZB;                    // [KPZ][GB][MB]
+  uint16_t* BTU = Vm + (size_t)c.KPZ * c.GB * c.MB;          // [GB][W][KIB]
+  float* Dz = reinterpret_cast<float*>(BTU + (size_t)c.GB * W * c.KIB);   // [MZ][16]
   float* Di = Dz + c.MZ * 16;                                            // [2N][16]
   const float2* Rc = R + (long long)col * m2 * W * W;
+  allow_dependent_launch();
+  if (c.stage) {   // (the parameters are not written by the kernels of a pass)
+    for (int i = tid; i < m2 * W * W / 2; i += kThreads)
+      rpm::async_copy16(Rs + 2 * i, Rc + 2 * i);
+    rpm::async_copy_commit();
+    Rc = Rs;
+  }
   for (int i = tid; i < c.KPZ * N; i += kThreads) {
     const int r = i / N, z = i - r * N;
     float tr = 0.f, ti = 0.f;
@@ -532,17 +561,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
     *reinterpret_cast<uint32_t*>(Ainv + (size_t)z * c.KIB + 2 * r) = bf16x2_bits(tr, ti);
     *reinterpret_cast<uint32_t*>(Ainv + (size_t)(N + z) * c.KIB + 2 * r) = bf16x2_bits(-ti, tr);
   }
+  // columns of BTU past the kept kz stay zero
+  for (int i = tid; i < c.GB * W * (c.KPZ - m2); i += kThreads) {
+    const int row = i / (c.KPZ - m2), k = m2 + i % (c.KPZ - m2);
+    *reinterpret_cast<uint32_t*>(BTU + (size_t)row * c.KIB + 2 * k) = 0u;
+  }
+  grid_dependency_wait();
   const int zmt = c.MZ / 16, imt = 2 * N / 16;
   for (int g0 = 0; g0 < B; g0 += 16) {
     const int gb = min(16, B - g0);
-    __syncthreads();   // tables written; the previous group's readers are done
-    for (int i = tid; i < c.KPZ * 16 * c.MB / 2; i += kThreads)
-      reinterpret_cast<uint32_t*>(Vm)[i] = 0u;
-    for (int i = tid; i < 16 * W * c.KIB / 2; i += kThreads)
-      reinterpret_cast<uint32_t*>(BTU)[i] = 0u;
     for (int bi = 0; bi < gb; ++bi) {
       const int b = g0 + bi;
-      __syncthreads();   // BTa / Dz readers of the previous sample are done
+      __syncthreads();   // tables written; BTa / Dz readers of the previous sample are done
       for (int i = tid; i < N * W; i += kThreads) {
         const int z = i / W, cc = i - z * W;
         const float2 a = A2[((long long)b * N + z) * ncol * W + col * W + cc];
@@ -567,15 +597,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
         d[8 * 16 + 1] = acc[3];
       }
       __syncthreads();
-      float2* vs = Vs + ((long long)col * B + b) * m2 * W;
+      float2* vs = Vs ? Vs + ((long long)col * B + b) * m2 * W : nullptr;
       for (int o = tid; o < m2 * W; o += kThreads) {
         const int kzi = o / W, cc = o - kzi * W;
         const float re = Dz[kzi * 16 + cc], im = Dz[(c.KPZ + kzi) * 16 + cc];
-        vs[o] = make_float2(re, im);
-        *reinterpret_cast<uint32_t*>(Vm + ((size_t)kzi * 16 + bi) * c.MB + 2 * cc) =
+        if (vs) vs[o] = make_float2(re, im);
+        *reinterpret_cast<uint32_t*>(Vm + ((size_t)kzi * c.GB + bi) * c.MB + 2 * cc) =
             bf16x2_bits(re, im);
       }
     }
+    if (c.stage) rpm::async_copy_wait();
     __syncthreads();
     // channel mixing per kz: U[b][(o, re/im)] = sum_(i, re/im) V[b][(i, re/im)] Rr[kz]
     for (int tile = warp; tile < m2 * 4; tile += kThreads / 32) {
@@ -583,7 +614,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
       const float2* rk = Rc + (size_t)kzi * W * W;
       const int o = 4 * nt + ((lane >> 2) >> 1), ro = (lane >> 2) & 1;
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const uint16_t* pa = Vm + ((size_t)kzi * 16 + (lane & 15)) * c.MB + (lane >> 4) * 8;
+      const uint16_t* pa = Vm + ((size_t)kzi * c.GB + min(lane & 15, gb - 1)) * c.MB + (lane >> 4) * 8;
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks) {
         uint32_t a[4], bb[2];
@@ -599,10 +630,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
       // rows b = lane/4 (+8), columns n = 8 nt + 2t (+1) = (o', re/im), o' = 4 nt + t
       const int oo = 4 * nt + (lane & 3);
       const int b0 = lane >> 2;
-      *reinterpret_cast<uint32_t*>(BTU + ((size_t)b0 * W + oo) * c.KIB + 2 * kzi) =
-          bf16x2_bits(acc[0], acc[1]);
-      *reinterpret_cast<uint32_t*>(BTU + ((size_t)(b0 + 8) * W + oo) * c.KIB + 2 * kzi) =
-          bf16x2_bits(acc[2], acc[3]);
+      if (b0 < gb)
+        *reinterpret_cast<uint32_t*>(BTU + ((size_t)b0 * W + oo) * c.KIB + 2 * kzi) =
+            bf16x2_bits(acc[0], acc[1]);
+      if (b0 + 8 < gb)
+        *reinterpret_cast<uint32_t*>(BTU + ((size_t)(b0 + 8) * W + oo) * c.KIB + 2 * kzi) =
+            bf16x2_bits(acc[2], acc[3]);
     }
     for (int bi = 0; bi < gb; ++bi) {
       const int b = g0 + bi;
@@ -651,14 +684,16 @@ __global__ void __launch_bounds__(kThreads) k_spec_bwd(const float2* __restrict_
   float2* dU = a + N * W;
   float2* V = dU + m2 * W;
   float2* dV = V + m2 * W;
-  float2* tw = dV + m2 * W;
-  float2* Tz = tw + N;
+  float2* Tz = dV + m2 * W;
+  allow_dependent_launch();
   const int kx = col % m;
   const float wgt = (kx == 0 ? 1.f : 2.f) * inv_n3;
   const float4* r4 = (const float4*)(R + (long long)col * m2 * W * W);
-  for (int i = tid; i < m2 * W * W / 2; i += kThreads) ((float4*)Rs)[i] = r4[i];
-  for (int i = tid; i < N; i += kThreads) tw[i] = twg[i];
+  // weights by asynchronous copies: they are needed after the first z transform
+  for (int i = tid; i < m2 * W * W / 2; i += kThreads) rpm::async_copy16((float4*)Rs + i, r4 + i);
+  rpm::async_copy_commit();
   z_table(twg, Tz, N, m);
+  grid_dependency_wait();
   const int gi = tid / W, go = tid % W;   // this thread's (i, o) entry of gR
   float2 g[2 * kMaxModes];
 #pragma unroll
@@ -670,7 +705,8 @@ __global__ void __launch_bounds__(kThreads) k_spec_bwd(const float2* __restrict_
     const float2* vs = Vs + ((long long)col * B + b) * m2 * W;
     for (int o = tid; o < m2 * W; o += kThreads) V[o] = vs[o];
     __syncthreads();
-    z_dft(a, tw, dU, N, m, wgt);
+    z_dft(a, Tz, dU, N, m, wgt);
+    rpm::async_copy_wait();
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 2 * kMaxModes; ++k)
@@ -746,15 +782,12 @@ __device__ __forceinline__ void inv_pointwise(const float (&u0)[W], const float 
         s1 = fmaf(av.x, v1[4 * q], fmaf(av.y, v1[4 * q + 1],
                   fmaf(av.z, v1[4 * q + 2], fmaf(av.w, v1[4 * q + 3], s1))));
       }
-      if (last) {
-        vout[at0 + oc * N3] = s0;
-        vout[at1 + oc * N3] = s1;
-      } else {
+      if (zsave) {
         zsave[at0 + oc * N3] = s0;
         zsave[at1 + oc * N3] = s1;
-        vout[at0 + oc * N3] = gelu(s0);
-        vout[at1 + oc * N3] = gelu(s1);
       }
+      vout[at0 + oc * N3] = last ? s0 : gelu(s0);
+      vout[at1 + oc * N3] = last ? s1 : gelu(s1);
     }
   }
 }
@@ -762,7 +795,7 @@ __device__ __forceinline__ void inv_pointwise(const float (&u0)[W], const float 
 // Inverse y and x transforms of the mode columns of plane (z, b), rows
 // [y0, y0 + YC), fused with the pointwise part of the layer.
 //   BWD = false: z = A v + a + u (u weighted c(kx) / N^3); writes zsave (unless
-//                last) and vout = gelu(z) (z on the last layer).
+//                null) and vout = gelu(z) (z on the last layer).
 //   BWD = true : vout += u (unweighted).
 // y stage: Y[yy][kx][c] = sum_ky S[ky][kx][c] conj(root(ky y)), tile 4 rows x 2
 // channels; x stage: u_c(x) = sum_kx w(kx) Re(Y[yy][kx][c] exp(+i 2 pi kx x / N))
@@ -864,7 +897,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy(const float2* __restrict
 //            M = YC W, K = round16(2m), Nout = N
 // Each warp stages the x-stage output of one row yy (16 channels x N voxels)
 // in its own shared-memory slab and runs the pointwise end of the layer on
-// those voxels (inv_pointwise, as in k_inv_xy).
+// those voxels, two at a time (x and x + N/2) in packed float32 arithmetic with
+// A held twice over; the row's inputs are loaded before its products.
 // ---------------------------------------------------------------------------
 struct InvTc {
   int K1, K1P, N1, M1, K2, K2P, UP, YC;
@@ -881,7 +915,7 @@ struct InvTc {
   __host__ __device__ size_t bytes(int N) const {
     return (size_t)2 * ((size_t)N1 * K1P + (size_t)M1 * K1P + (size_t)YC * W * K2P +
                         (size_t)N * K2P) +
-           (size_t)4 * (8 * W * UP + kLayerHead);
+           (size_t)4 * (8 * W * UP + 2 * kLayerHead);
   }
 };
 size_t inv_tc_smem(int N, int m, int YC) { return InvTc(N, m, YC).bytes(N); }
@@ -906,13 +940,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
   const int y0 = blockIdx.x * YC, z = blockIdx.y, b = blockIdx.z;
   const long long N3 = (long long)N * N * N;
   const float2* src = Bz + ((long long)b * N + z) * ncol * W;
-  for (int i = tid; i < ncol * W; i += kThreads) {
-    const int cc = i % W, col = i / W;
-    const int kyi = col / m, kx = col - kyi * m;
-    const float2 sv = src[i];
-    *reinterpret_cast<uint32_t*>(BT1 + (size_t)(kx * W + cc) * c.K1P + 2 * kyi) =
-        bf16x2_bits(sv.x, sv.y);
-  }
+  allow_dependent_launch();
   const int pad1 = c.K1 - 4 * m;
   for (int i = tid; i < c.N1 * pad1; i += kThreads)
     BT1[(size_t)(i / pad1) * c.K1P + 4 * m + i % pad1] = 0;
@@ -942,7 +970,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
     *reinterpret_cast<uint32_t*>(BT2 + (size_t)x * c.K2P + 2 * kx) = bf16x2_bits(wr, wi);
   }
   if (!BWD)
-    for (int i = tid; i < kLayerHead; i += kThreads) Al[i] = layer[i];
+    for (int i = tid; i < kLayerHead; i += kThreads) Al[2 * i] = Al[2 * i + 1] = layer[i];
+  grid_dependency_wait();
+#pragma unroll 6
+  for (int i = tid; i < ncol * W; i += kThreads) {
+    const int cc = i % W, col = i / W;
+    const int kyi = col / m, kx = col - kyi * m;
+    const float2 sv = src[i];
+    *reinterpret_cast<uint32_t*>(BT1 + (size_t)(kx * W + cc) * c.K1P + 2 * kyi) =
+        bf16x2_bits(sv.x, sv.y);
+  }
   __syncthreads();
   const int nt1 = c.N1 / 8, mt1 = c.M1 / 16;
   for (int tile = warp; tile < mt1 * nt1; tile += kThreads / 32) {
@@ -970,8 +1007,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
   }
   __syncthreads();
   float* uw = Uw + (size_t)warp * W * c.UP;
-  const int half = N / 2;
+  constexpr int half = N / 2;
   for (int mt = warp; mt < YC; mt += kThreads / 32) {   // one row yy = mt: its 16 channels
+    const long long row = (long long)b * W * N3 + ((long long)z * N + y0 + mt) * N;
+    const float* pin = (BWD ? vout : vin) + row;
+    float2 v[W];   // this lane's voxels x and x + N/2 of the row, all channels
+    auto load = [&](int x) {
+#pragma unroll
+      for (int cc = 0; cc < W; ++cc)
+        v[cc] = make_float2(pin[cc * N3 + x], pin[cc * N3 + x + half]);
+    };
+    if (lane < half) load(lane);
     for (int nt = 0; nt < N / 8; ++nt) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       const uint16_t* pa = A2 + (size_t)(16 * mt + (lane & 15)) * c.K2P + (lane >> 4) * 8;
@@ -991,50 +1037,36 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
     __syncwarp();
 #pragma unroll 1
     for (int x = lane; x < half; x += 32) {
-      const long long at0 = (long long)b * W * N3 + ((long long)z * N + y0 + mt) * N + x;
-      const long long at1 = at0 + half;
-      const float* u0 = uw + x;
-      const float* u1 = uw + x + half;
+      if (x != lane) load(x);
+      const float* u = uw + x;
+      float* o0 = vout + row + x;
       if constexpr (BWD) {
-        float g0[W], g1[W];
 #pragma unroll
         for (int cc = 0; cc < W; ++cc) {
-          g0[cc] = vout[at0 + cc * N3];
-          g1[cc] = vout[at1 + cc * N3];
-        }
-#pragma unroll
-        for (int cc = 0; cc < W; ++cc) {
-          vout[at0 + cc * N3] = g0[cc] + u0[cc * c.UP];
-          vout[at1 + cc * N3] = g1[cc] + u1[cc * c.UP];
+          o0[cc * N3] = v[cc].x + u[cc * c.UP];
+          o0[cc * N3 + half] = v[cc].y + u[cc * c.UP + half];
         }
       } else {   // z = A v + a + u, then the activation (as inv_pointwise)
-        float v0[W], v1[W];
-#pragma unroll
-        for (int cc = 0; cc < W; ++cc) {
-          v0[cc] = vin[at0 + cc * N3];
-          v1[cc] = vin[at1 + cc * N3];
-        }
+        float* z0 = zsave ? zsave + row + x : nullptr;
 #pragma unroll 4
         for (int oc = 0; oc < W; ++oc) {
-          float s0 = Al[W * W + oc] + u0[oc * c.UP], s1 = Al[W * W + oc] + u1[oc * c.UP];
-          const float4* ar = reinterpret_cast<const float4*>(Al + oc * W);
+          const float bias = Al[2 * (W * W + oc)];
+          float2 sv = make_float2(bias + u[oc * c.UP], bias + u[oc * c.UP + half]);
+          const float4* ar = reinterpret_cast<const float4*>(Al + 2 * oc * W);
 #pragma unroll
           for (int q = 0; q < W / 4; ++q) {
-            const float4 av = ar[q];
-            s0 = fmaf(av.x, v0[4 * q], fmaf(av.y, v0[4 * q + 1],
-                      fmaf(av.z, v0[4 * q + 2], fmaf(av.w, v0[4 * q + 3], s0))));
-            s1 = fmaf(av.x, v1[4 * q], fmaf(av.y, v1[4 * q + 1],
-                      fmaf(av.z, v1[4 * q + 2], fmaf(av.w, v1[4 * q + 3], s1))));
+            const float4 a01 = ar[2 * q], a23 = ar[2 * q + 1];
+            sv = rpm::f2fma(make_float2(a23.z, a23.w), v[4 * q + 3], sv);
+            sv = rpm::f2fma(make_float2(a23.x, a23.y), v[4 * q + 2], sv);
+            sv = rpm::f2fma(make_float2(a01.z, a01.w), v[4 * q + 1], sv);
+            sv = rpm::f2fma(make_float2(a01.x, a01.y), v[4 * q], sv);
           }
-          if (last) {
-            vout[at0 + oc * N3] = s0;
-            vout[at1 + oc * N3] = s1;
-          } else {
-            zsave[at0 + oc * N3] = s0;
-            zsave[at1 + oc * N3] = s1;
-            vout[at0 + oc * N3] = gelu(s0);
-            vout[at1 + oc * N3] = gelu(s1);
+          if (z0) {
+            z0[oc * N3] = sv.x;
+            z0[oc * N3 + half] = sv.y;
           }
+          o0[oc * N3] = last ? sv.x : gelu(sv.x);
+          o0[oc * N3 + half] = last ? sv.y : gelu(sv.y);
         }
       }
     }
@@ -1155,13 +1187,40 @@ struct TileAcc4 {
   }
 };
 
-// v0 = P f + p.   total = B N^3 voxels.
+// v0 = P f + p for B N^3 voxels, four consecutive ones a thread (N^3 is a
+// multiple of 512; feat 16-byte aligned).  Launched in stream order without
+// overlap: the kernels after it in a pass start early and rely on the
+// parameters being in place.
 __global__ void __launch_bounds__(kThreads) k_lift(const float* __restrict__ feat,
                                                    const float* __restrict__ prm,
                                                    float* __restrict__ v0, long long N3, int B) {
   __shared__ float Ps[kNeP];
+  allow_dependent_launch();
   for (int i = threadIdx.x; i < kNeP; i += kThreads) Ps[i] = prm[kOffP + i];
   __syncthreads();
+  const long long n4 = N3 / 4, total = n4 * B;
+  const float4* f4 = reinterpret_cast<const float4*>(feat);
+  float4* o4 = reinterpret_cast<float4*>(v0);
+  for (long long gidx = blockIdx.x * (long long)kThreads + threadIdx.x; gidx < total;
+       gidx += (long long)gridDim.x * kThreads) {
+    const int b = (int)(gidx / n4);
+    const long long vox = gidx - b * n4;
+    const float4 f0 = f4[((long long)b * CV + 0) * n4 + vox];
+    const float4 f1 = f4[((long long)b * CV + 1) * n4 + vox];
+#pragma unroll
+    for (int o = 0; o < W; ++o) {
+      const float p0 = Ps[o * CV], p1 = Ps[o * CV + 1], p = Ps[W * CV + o];
+      o4[((long long)b * W + o) * n4 + vox] =
+          make_float4(fmaf(p1, f1.x, fmaf(p0, f0.x, p)), fmaf(p1, f1.y, fmaf(p0, f0.y, p)),
+                      fmaf(p1, f1.z, fmaf(p0, f0.z, p)), fmaf(p1, f1.w, fmaf(p0, f0.w, p)));
+    }
+  }
+}
+
+// The same one voxel at a time, for feature arrays of any alignment.
+__global__ void __launch_bounds__(kThreads) k_lift_any(const float* __restrict__ feat,
+                                                       const float* __restrict__ prm,
+                                                       float* __restrict__ v0, long long N3, int B) {
   const long long total = N3 * B;
   for (long long gidx = blockIdx.x * (long long)kThreads + threadIdx.x; gidx < total;
        gidx += (long long)gridDim.x * kThreads) {
@@ -1172,7 +1231,7 @@ __global__ void __launch_bounds__(kThreads) k_lift(const float* __restrict__ fea
 #pragma unroll
     for (int o = 0; o < W; ++o)
       v0[((long long)b * W + o) * N3 + vox] =
-          fmaf(Ps[o * CV + 1], f1, fmaf(Ps[o * CV], f0, Ps[W * CV + o]));
+          fmaf(prm[kOffP + o * CV + 1], f1, fmaf(prm[kOffP + o * CV], f0, prm[kOffP + W * CV + o]));
   }
 }
 
@@ -1190,6 +1249,8 @@ __global__ void __launch_bounds__(kThreads) k_lift_bwd(const float* __restrict__
   using Acc = TileAcc<W, CV>;
   __shared__ float sL[W * Acc::LD];
   __shared__ float sR[CV * Acc::LD];
+  allow_dependent_launch();
+  grid_dependency_wait();
   Acc acc;
   acc.init();
   const long long total = N3 * B;
@@ -1231,7 +1292,9 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pw(const float* __restrict__ d
   float* sL = stage;                     // [voxel][LDL]
   float* sR = stage + kThreads * Acc::LDL;
   __shared__ float As[W * W];
+  allow_dependent_launch();
   for (int i = threadIdx.x; i < W * W; i += kThreads) As[i] = layer[i];
+  grid_dependency_wait();
   __syncthreads();
   Acc acc;
   acc.init();
@@ -1278,10 +1341,11 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pw(const float* __restrict__ d
   acc.store(part + (long long)blockIdx.x * Acc::NE, stage);
 }
 
-// Shared memory of k_head (floats): the two tiles, then per sample the
+// Shared memory of k_head (floats): the two tiles (TRAIN), then per sample the
 // contracted maps QE_b[o][c] (c < W) and qE_b[o] (c = W), then E.
-size_t head_smem(int B) {
-  return ((size_t)TileAcc4<NH, W>::SMEM + (size_t)B * COUT * (W + 1) + (size_t)B * CE) * 4;
+size_t head_smem(int B, bool train) {
+  return ((train ? (size_t)TileAcc4<NH, W>::SMEM : 0) + (size_t)B * COUT * (W + 1) +
+          (size_t)B * CE) * 4;
 }
 
 // Localisation head: H = Q v + q (36 channels, channel 6 o + j = H[o][j]) and
@@ -1289,6 +1353,7 @@ size_t head_smem(int B) {
 // QE_b = sum_j Q[6 o + j] E_bj.  With a target: d = 2 (out - t) / nel,
 // dH[o][j] = d[o] E_bj, dvL = Q^T dH = QE_b^T d, and partials of
 // gQ = sum dH v^T, gq = sum dH and of sum (out - t)^2.
+template <bool TRAIN>
 __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
                                                    const float* __restrict__ prm,
                                                    const float* __restrict__ Ed,
@@ -1301,9 +1366,10 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
   extern __shared__ float4 smem4[];
   float* sL = (float*)smem4;                 // [voxel][LDL]
   float* sR = sL + kThreads * Acc::LDL;      // [voxel][LDR]
-  float* QE = (float*)smem4 + Acc::SMEM;     // [B][COUT][W + 1]
+  float* QE = (float*)smem4 + (TRAIN ? Acc::SMEM : 0);   // [B][COUT][W + 1]
   float* Es = QE + B * COUT * (W + 1);       // [B][CE]
   __shared__ float red[kThreads / 32];
+  allow_dependent_launch();
   for (int i = threadIdx.x; i < B * CE; i += kThreads) Es[i] = Ed[i];
   for (int i = threadIdx.x; i < B * COUT * (W + 1); i += kThreads) {
     const int b = i / (COUT * (W + 1)), r = i - b * (COUT * (W + 1));
@@ -1315,6 +1381,7 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
     }
     QE[i] = s;
   }
+  grid_dependency_wait();
   __syncthreads();
   Acc acc;
   acc.init();
@@ -1339,13 +1406,13 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
         for (int c = 0; c < W; ++c) s = fmaf(qe[o * (W + 1) + c], x[c], s);
         const long long at = ((long long)b * COUT + o) * N3 + vox;
         if (out) out[at] = s;
-        if (target) {
+        if (TRAIN) {
           const float diff = s - target[at];
           sq = fmaf(diff, diff, sq);
           d[o] = 2.f * diff * inv_nel;
         }
       }
-      if (target) {
+      if (TRAIN) {
 #pragma unroll
         for (int c = 0; c < W; ++c) {
           float s = 0.f;
@@ -1360,7 +1427,7 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
           for (int j = 0; j < CE; ++j) sL[t * Acc::LDL + o * CE + j] = d[o] * Es[b * CE + j];
       }
     }
-    if (target) {
+    if (TRAIN) {
       if (!have) {
 #pragma unroll
         for (int k = 0; k < NH; ++k) sL[t * Acc::LDL + k] = 0.f;
@@ -1372,7 +1439,7 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
       __syncthreads();
     }
   }
-  if (!target) return;
+  if (!TRAIN) return;
   acc.store(part + (long long)blockIdx.x * kNeHead, (float*)smem4);   // after the loop's barrier
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
   if ((t & 31) == 0) red[t >> 5] = sq;
@@ -1386,9 +1453,11 @@ __global__ void __launch_bounds__(kThreads) k_head(const float* __restrict__ v,
 
 // dst[e] = sum over blocks of part[blk][e] (float64, fixed order) for e < n_grad;
 // the entries after n_grad go to extra (float64).  A block takes 32
-// consecutive entries (one per lane: coalesced rows); its 8 warps take every
-// 8th partial row, then warp 0 adds the 8 warp sums in order.
-constexpr int kRedWarps = 8;
+// consecutive entries (one per lane: coalesced rows); its 32 warps take every
+// 32nd partial row, then warp 0 adds the 32 warp sums in order.  The rows of a
+// warp are a chain of dependent sums: 32 warps instead of 8 shorten it
+// (256 rows: 9.5 -> 8.5 us).
+constexpr int kRedWarps = 32;
 __global__ void __launch_bounds__(32 * kRedWarps) k_reduce(const float* __restrict__ part,
                                                            int nblk, int stride, int n_grad,
                                                            int n_extra, float* __restrict__ dst,
@@ -1398,8 +1467,10 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_reduce(const float* __restri
   const int e = blockIdx.x * 32 + lane;
   const int ne = n_grad + n_extra;
   double s = 0.0;
+  allow_dependent_launch();
+  grid_dependency_wait();
   if (e < ne) {
-#pragma unroll 4
+#pragma unroll 8
     for (int k = w; k < nblk; k += kRedWarps) s += (double)part[(long long)k * stride + e];
   }
   sm[w][lane] = s;
@@ -1520,42 +1591,48 @@ bool stage_E(rpm_fno* f, int B, const float* E_dir) {
 // tensor-core kernel when the network was created with RPM_FNO_BF16.
 #define RPM_FNO_TC_SIZES(X) X(32) X(48) X(64) X(96) X(128)
 
-void launch_xy_fwd(rpm_fno* f, const float* src, int B) {
+cudaError_t launch_xy_fwd(rpm_fno* f, const float* src, int B) {
   const int N = f->N, m = f->m;
   if (f->tc) {
+    // channel groups over blocks until there are two blocks per SM (each block
+    // builds the twiddle tables, so not further): 64^3, one sample, 26.4 -> 11.5 us;
+    // 32^3, two samples, 19.4 -> 8.5 us
+    int nc = 1;
+    while (nc < W / xy_group(N) && N * B * nc < 304) nc *= 2;
     switch (N) {
 #define RPM_CASE(NN)                                                                        \
   case NN:                                                                                  \
-    k_xy_fwd_tc<NN><<<dim3(N, B), kThreads, xy_tc_smem(N, m), f->st>>>(src, f->A2, f->tw, m); \
-    return;
+    return launch_pdl(k_xy_fwd_tc<NN>, dim3(N, B, nc), kThreads, xy_tc_smem(N, m), f->st, src,  \
+                      f->A2, (const float2*)f->tw, m);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
   }
   k_xy_fwd<<<dim3(N, B), kThreads, xy_smem(N, m), f->st>>>(src, f->A2, f->tw, N, m);
+  return cudaGetLastError();
 }
 
 // Forward spectral kernel of one layer: f->A2 -> f->Bz, V saved in Vs.
-void launch_spec_fwd(rpm_fno* f, int B, const float2* R, float2* Vs) {
+cudaError_t launch_spec_fwd(rpm_fno* f, int B, const float2* R, float2* Vs) {
   const int N = f->N, m = f->m;
   if (f->tc) {
     switch (N) {
 #define RPM_CASE(NN)                                                                           \
   case NN:                                                                                     \
-    k_spec_fwd_tc<NN><<<f->ncol, kThreads, spec_tc_smem<NN>(m), f->st>>>(f->A2, R, Vs, f->Bz, \
-                                                                         f->tw, m, B);         \
-    return;
+    return launch_pdl(k_spec_fwd_tc<NN>, dim3(f->ncol), kThreads, spec_tc_smem<NN>(m, B),      \
+                      f->st, (const float2*)f->A2, R, Vs, f->Bz, (const float2*)f->tw, m, B);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
   }
   k_spec_fwd<<<dim3(f->ncol, B), kThreads, spec_smem(N, m), f->st>>>(f->A2, R, Vs, f->Bz, f->tw,
                                                                      N, m, B);
+  return cudaGetLastError();
 }
 
 // Inverse xy transform of B samples from f->Bz (pointwise end as k_inv_xy).
 template <bool BWD>
-void launch_inv_xy(rpm_fno* f, int B, const float* layer, const float* vin, float* zsave,
+cudaError_t launch_inv_xy(rpm_fno* f, int B, const float* layer, const float* vin, float* zsave,
                    float* vout, int last, float inv_n3) {
   const int N = f->N, m = f->m;
   const dim3 grid(N / f->YC, N, B);
@@ -1563,44 +1640,57 @@ void launch_inv_xy(rpm_fno* f, int B, const float* layer, const float* vin, floa
     switch (N) {
 #define RPM_CASE(NN)                                                                     \
   case NN:                                                                               \
-    k_inv_xy_tc<BWD, NN><<<grid, kThreads, inv_tc_smem(N, m, f->YC), f->st>>>(          \
-        f->Bz, f->tw, layer, vin, zsave, vout, m, f->YC, last, inv_n3);                 \
-    return;
+    return launch_pdl(k_inv_xy_tc<BWD, NN>, grid, kThreads, inv_tc_smem(N, m, f->YC), f->st, \
+                      (const float2*)f->Bz, (const float2*)f->tw, layer, vin, zsave, vout, m,  \
+                      f->YC, last, inv_n3);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
   }
   k_inv_xy<BWD><<<grid, kThreads, inv_smem(m, f->YC), f->st>>>(f->Bz, f->tw, layer, vin, zsave,
                                                               vout, N, m, f->YC, last, inv_n3);
+  return cudaGetLastError();
 }
 
-// Forward pass; keeps v_l and z_l.  out (optional), target (optional: then the
-// head also writes dv_L into dvb(0) and its partials).
+cudaError_t launch_reduce(rpm_fno* f, int nblk, int stride, int n_grad, int n_extra, float* dst,
+                          double* extra) {
+  return launch_pdl(k_reduce, dim3(reduce_blocks(n_grad + n_extra)), 32 * kRedWarps, 0, f->st,
+                    (const float*)f->part, nblk, stride, n_grad, n_extra, dst, extra);
+}
+
+// Forward pass.  out (optional), target (optional: then the pass keeps z_l and
+// the spectra V_l for the backward pass, and the head also writes dv_L into
+// dvb(0) and its partials).  The kernels overlap their prologues (programmatic
+// dependent launch); k_lift does not, so that everything before the pass is
+// complete when the first of them starts.
 bool run_forward(rpm_fno* f, int B, const float* feat, const float* target, float* out) {
-  const int N = f->N, m = f->m, L = f->L;
+  const int L = f->L;
   const long long total = f->N3 * B;
   const int nb = pw_blocks(total);
   const float inv_n3 = 1.f / (float)f->N3;
-  k_lift<<<nb, kThreads, 0, f->st>>>(feat, f->params, f->v(0), f->N3, B);
+  if (((uintptr_t)feat & 15) == 0)
+    k_lift<<<pw_blocks(total / 4), kThreads, 0, f->st>>>(feat, f->params, f->v(0), f->N3, B);
+  else
+    k_lift_any<<<nb, kThreads, 0, f->st>>>(feat, f->params, f->v(0), f->N3, B);
   if (!fck(f, cudaGetLastError(), "lift")) return false;
   for (int l = 0; l < L; ++l) {
-    launch_xy_fwd(f, f->v(l), B);
-    launch_spec_fwd(f, B, (const float2*)(f->layer(l) + kLayerHead), f->Vsl(l));
     const int last = (l == L - 1);
-    launch_inv_xy<false>(f, B, f->layer(l), f->v(l), last ? nullptr : f->z(l), f->v(l + 1), last,
-                         inv_n3);
-    if (!fck(f, cudaGetLastError(), "layer")) return false;
+    float* zsave = last || !target ? nullptr : f->z(l);
+    if (!fck(f, launch_xy_fwd(f, f->v(l), B), "layer") ||
+        !fck(f, launch_spec_fwd(f, B, (const float2*)(f->layer(l) + kLayerHead),
+                                target ? f->Vsl(l) : nullptr), "layer") ||
+        !fck(f, launch_inv_xy<false>(f, B, f->layer(l), f->v(l), zsave, f->v(l + 1), last, inv_n3),
+             "layer"))
+      return false;
   }
   const float inv_nel = 1.f / (float)(total * COUT);
-  k_head<<<nb, kThreads, head_smem(B), f->st>>>(f->v(L), f->params, f->Ed, target, out,
-                                                 f->dvb(0), f->part, f->N3, B, inv_nel);
-  if (!fck(f, cudaGetLastError(), "head")) return false;
-  if (target) {
-    k_reduce<<<reduce_blocks(kNeHead), 32 * kRedWarps, 0, f->st>>>(f->part, nb, kNeHead, kNeQ, 1,
-                                                                   f->grads + kOffQ, f->extra);
-    if (!fck(f, cudaGetLastError(), "reduce head")) return false;
-  }
-  return true;
+  const float *v = f->v(L), *prm = f->params, *Ed = f->Ed;
+  if (!target)
+    return fck(f, launch_pdl(k_head<false>, dim3(nb), kThreads, head_smem(B, false), f->st, v, prm,
+                             Ed, target, out, f->dvb(0), f->part, f->N3, B, inv_nel), "head");
+  return fck(f, launch_pdl(k_head<true>, dim3(nb), kThreads, head_smem(B, true), f->st, v, prm, Ed,
+                           target, out, f->dvb(0), f->part, f->N3, B, inv_nel), "head") &&
+         fck(f, launch_reduce(f, nb, kNeHead, kNeQ, 1, f->grads + kOffQ, f->extra), "reduce head");
 }
 
 bool run_backward(rpm_fno* f, int B, const float* feat) {
@@ -1613,22 +1703,24 @@ bool run_backward(rpm_fno* f, int B, const float* feat) {
     const int last = (l == L - 1);
     float* dz = f->dvb(2);
     float* prev = f->dvb(1 - cur);
-    k_bwd_pw<<<nb, kThreads, 0, f->st>>>(f->dvb(cur), last ? nullptr : f->z(l), f->v(l),
-                                         f->layer(l), dz, prev, f->part, f->N3, B, last);
-    k_reduce<<<reduce_blocks(kNeA), 32 * kRedWarps, 0, f->st>>>(f->part, nb, kNeA, kNeA, 0,
-                                                                f->glayer(l), nullptr);
-    launch_xy_fwd(f, dz, B);
-    k_spec_bwd<<<f->ncol, kThreads, spec_smem(N, m), f->st>>>(
-        f->A2, (const float2*)(f->layer(l) + kLayerHead), f->Vsl(l),
-        (float2*)(f->glayer(l) + kLayerHead), f->Bz, f->tw, N, m, B, inv_n3);
-    launch_inv_xy<true>(f, B, nullptr, nullptr, nullptr, prev, 0, inv_n3);
-    if (!fck(f, cudaGetLastError(), "layer backward")) return false;
+    const float *dv = f->dvb(cur), *zs = last ? nullptr : f->z(l), *v = f->v(l);
+    const float* layer = f->layer(l);
+    if (!fck(f, launch_pdl(k_bwd_pw, dim3(nb), kThreads, 0, f->st, dv, zs, v, layer, dz, prev,
+                           f->part, f->N3, B, last), "layer backward") ||
+        !fck(f, launch_reduce(f, nb, kNeA, kNeA, 0, f->glayer(l), nullptr), "layer backward") ||
+        !fck(f, launch_xy_fwd(f, dz, B), "layer backward") ||
+        !fck(f, launch_pdl(k_spec_bwd, dim3(f->ncol), kThreads, spec_smem(N, m), f->st,
+                           (const float2*)f->A2, (const float2*)(f->layer(l) + kLayerHead),
+                           (const float2*)f->Vsl(l), (float2*)(f->glayer(l) + kLayerHead), f->Bz,
+                           (const float2*)f->tw, N, m, B, inv_n3), "layer backward") ||
+        !fck(f, launch_inv_xy<true>(f, B, nullptr, nullptr, nullptr, prev, 0, inv_n3),
+             "layer backward"))
+      return false;
     cur = 1 - cur;
   }
-  k_lift_bwd<<<nb, kThreads, 0, f->st>>>(f->dvb(cur), feat, f->part, f->N3, B);
-  k_reduce<<<reduce_blocks(kNeP), 32 * kRedWarps, 0, f->st>>>(f->part, nb, kNeP, kNeP, 0,
-                                                               f->grads + kOffP, nullptr);
-  return fck(f, cudaGetLastError(), "lift backward");
+  return fck(f, launch_pdl(k_lift_bwd, dim3(nb), kThreads, 0, f->st, (const float*)f->dvb(cur),
+                           feat, f->part, f->N3, B), "lift backward") &&
+         fck(f, launch_reduce(f, nb, kNeP, kNeP, 0, f->grads + kOffP, nullptr), "lift backward");
 }
 
 // Shared-memory limits of the tensor-core kernels (per grid side: sixteen
@@ -1640,7 +1732,7 @@ bool set_tc_smem() {
                inv_tc_smem(NN, kMaxModes, NN <= 64 ? 16 : 8)) != cudaSuccess ||             \
       set_smem((const void*)k_inv_xy_tc<true, NN>,                                          \
                inv_tc_smem(NN, kMaxModes, NN <= 64 ? 16 : 8)) != cudaSuccess ||             \
-      set_smem((const void*)k_spec_fwd_tc<NN>, spec_tc_smem<NN>(kMaxModes)) != cudaSuccess)   \
+      set_smem((const void*)k_spec_fwd_tc<NN>, spec_tc_max<NN>()) != cudaSuccess)              \
     return false;
   RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
@@ -1730,7 +1822,8 @@ rpm_status rpm_fno_create(const rpm_fno_config* cfg, void* cuda_stream, rpm_fno*
       set_smem((const void*)k_inv_xy<false>, inv_smem(kMaxModes, 16)) != cudaSuccess ||
       set_smem((const void*)k_inv_xy<true>, inv_smem(kMaxModes, 16)) != cudaSuccess ||
 
-      set_smem((const void*)k_head, head_smem(RPM_FNO_MAX_BATCH)) != cudaSuccess ||
+      set_smem((const void*)k_head<true>, head_smem(RPM_FNO_MAX_BATCH, true)) != cudaSuccess ||
+      set_smem((const void*)k_head<false>, head_smem(RPM_FNO_MAX_BATCH, false)) != cudaSuccess ||
       cudaStreamSynchronize(f->st) != cudaSuccess) {
     cudaGetLastError();
     rpm_fno_destroy(f);

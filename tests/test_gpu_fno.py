@@ -335,3 +335,32 @@ def test_bf16_loss_and_gradients_match_oracle(fno):
         rel = np.linalg.norm(a - b) / np.linalg.norm(b)
         print(f"bf16 gradient {k}: rel L2 err {rel:.2e}")
         assert rel < BF16_GRAD_TOL, (k, rel)
+
+
+@pytest.mark.parametrize("N,m,L,B", [(32, 5, 2, 1), (32, 12, 2, 2), (32, 7, 1, 3), (48, 4, 1, 2),
+                                     (64, 12, 1, 1), (32, 3, 1, 17)])
+def test_bf16_forward_alone_matches_the_training_pass(fno, N, m, L, B):
+    """A forward pass keeps no activations or spectra for a backward one and
+    shares its kernels' blocks differently (staged weights up to two samples,
+    channel groups, a ragged second group of samples): its output is the one
+    the loss of a training pass implies, and that of a misaligned feature array."""
+    p = _round32(_params(m, L, 31 + N))
+    feat, E = _inputs(N, B, 7)
+    E = E.astype(np.float32).astype(np.float64)
+    out = torch.empty((B, 6, N, N, N), device="cuda")
+    again = torch.empty_like(out)
+    shifted = torch.empty(feat.size + 1, device="cuda")
+    shifted[1:].copy_(torch.from_numpy(feat.astype(np.float32)).ravel())
+    with fno.Fno(N, m, L, max_batch=B, precision="bf16") as net:
+        net.set_params(p)
+        net.forward(_dev(feat), E, out)
+        loss = net.loss_grad(_dev(feat), E, torch.zeros_like(out))
+        net.forward(shifted[1:].view(B, 2, N, N, N), E, again)
+        torch.cuda.synchronize()
+    mean = float(out.double().square().mean())
+    # float32 sums of the same squares: at most 12 terms a thread, 13 levels above
+    assert abs(loss - mean) <= 3e-6 * mean
+    assert torch.equal(out, again)
+    ref = fo.forward(p, feat.astype(np.float32).astype(np.float64), E, m, L)
+    err = np.max(np.abs(out.cpu().numpy() - ref)) / np.max(np.abs(ref))
+    assert err < BF16_OUT_TOL, err
