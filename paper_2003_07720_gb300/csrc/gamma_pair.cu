@@ -1,5 +1,5 @@
 // The Lippmann-Schwinger map on paired lines: the three passes of
-// gamma_kernels.cu for square planes nx = ny in {48, 64, 96, 128}, with every
+// gamma_kernels.cu for square planes nx = ny up to 128, with every
 // transform working on two lines at once in packed float32 arithmetic
 // (pair_fft.cuh).
 //
@@ -17,13 +17,20 @@
 // holds 2 X: the factor 1/2 of the real-to-complex untangling is left out of
 // pass A and taken up by the zero frequency (2 E n) and the final scale.
 //
+// Each kernel lets the next one start when its own last phase begins, not
+// earlier: blocks of a kernel two launches on would otherwise sit on every SM
+// through a whole pass, holding slots and, by their shared memory, the split
+// between shared memory and L1 (256^3: 1046 us a map with the trigger at the
+// start of every kernel, 800 us so; 32^3 13.0 and 8.8 us, 24 x 96 x 48 21 and
+// 15 us).
+//
 // What bounds the passes: with one line per thread they were bound by issue
 // slots (128^3: 19.1, 21.7 and 13.8 M warp instructions in passes A, B, C,
 // 47-61 % issue active).  Pairing brought them to 11.8, 11.6 and 7.5 M; now
 // shared-memory bandwidth (C: 67 % of the L1 pipe's cycles) and the latency of
-// two or three resident blocks bound them.  One map of 128^3: 96 -> 87 us, of
-// 64^3 20.5 -> 16.1 us, of 48^3 15.3 -> 12.8 us; 96^3 passes A + B + C
-// 71 -> 40 us (single-kernel times).
+// two or three resident blocks bound them.  One map of 128^3: 96 -> 86 us, of
+// 64^3 20.5 -> 15.5 us, of 48^3 15.3 -> 11.2 us, of 16^3 16.4 -> 9.3 us; 96^3
+// passes A + B + C 71 -> 40 us (single-kernel times).
 #include <algorithm>
 #include <cmath>
 
@@ -40,9 +47,15 @@ namespace {
 // where a plane fills a third of the SM's shared memory (128^2: 87 against
 // 96 us a map) and where one block has few tasks per phase (64^2: 17.1 against
 // 23.1 us, 48^2: 13.3 against 16.5 us); at 96^2 four blocks of 128 fit (40.4
-// against 47.1 us).
-constexpr int pair_threads(int n) { return n == 96 ? 128 : 256; }
-constexpr int pair_blocks(int n) { return n == 96 ? 4 : 2; }
+// against 47.1 us).  Sides up to 24 take one warp: a thread transforms a whole
+// row pair, then a whole column pair, and nothing but the exchange between the
+// two goes through shared memory.
+constexpr int pair_threads(int n, bool few) {
+  return n <= 24 ? 32 : (n == 32 ? 64 : (n == 96 && !few ? 128 : 256));
+}
+constexpr int pair_blocks(int n, int threads) {
+  return n <= 16 ? 16 : (n <= 32 ? 8 : (n == 96 && threads == 128 ? 4 : 2));
+}
 
 // The x transform of a block's row pairs: rows nx long, ROWS pairs in shared
 // memory as [ROWS][nx/2 + 1], TPB threads.
@@ -55,12 +68,15 @@ struct PairX {
   static_assert(SX % 2 == 1 || X2 == 1, "odd row stride: rows fall in distinct 16-byte banks");
 };
 
-template <int N>
+template <int N, int TPB_>
 struct PairPlane {
   static constexpr int NXH = N / 2, SX = NXH + 1, H = N / 2, PL = H * SX;
   static constexpr int X1 = pair_n1(NXH), X2 = NXH / X1;
   static constexpr int Y1 = pair_n1(H), Y2 = H / Y1;
-  static constexpr int TPB = pair_threads(N), MINB = pair_blocks(N);
+  static constexpr int TPB = TPB_, MINB = pair_blocks(N, TPB_);
+  // two-step x lengths pack the columns 0 and nx/2 into one
+  static constexpr bool PACK = X2 > 1;
+  static constexpr int COLS = PACK ? NXH : SX;
   using X = PairX<N, H, TPB>;
 };
 
@@ -131,6 +147,15 @@ __device__ __forceinline__ void pair_untangle_row(const C2* v, const float4* r2c
   }
 }
 
+// (lam, 2 mu) of C - C0.  With at most two phases every thread reads both pairs
+// itself and selects (phase ids are < n_phases): no table, and the strain loads
+// do not wait for one.  Otherwise a table of all 256 ids in shared memory.
+__device__ __forceinline__ float2 pair_material(float2 m) { return make_float2(m.x, 2.f * m.y); }
+__device__ __forceinline__ void pair_materials(const GridDev& g, float2* dm, int threads) {
+  if (g.n_phases > 2)
+    for (int i = threadIdx.x; i < 256; i += threads) dm[i] = pair_material(g.dmat[i]);
+}
+
 // x step 1 of pass A: the strain rows j and j + ny/2 are read from global
 // memory, the polarization formed on the way in (KIND: one component's rows as
 // they are, a shear component, or a normal one, which needs the trace and so
@@ -141,11 +166,13 @@ template <class C, int KIND, bool TWO, bool PACK>
 __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const float2* __restrict__ e1,
                                         const float2* __restrict__ e2,
                                         const uchar2* __restrict__ phase, int low, int rows,
-                                        const float2* dm, float4* P, const float4* twx,
+                                        const float2* __restrict__ dmat, const float2* dm,
+                                        float4* P, const float4* twx,
                                         const float4* r2c, const float2* hw) {
   constexpr int NXH = C::NXH, SX = C::SX, X1 = C::X1, X2 = C::X2;
   constexpr int B = KIND == kNormal && X1 > 4 ? 4 : X1;   // voxel pairs loaded per batch
-  const float2 dm0 = dm[0], dm1 = dm[1];
+  const float2 dm0 = TWO && KIND != kRaw ? pair_material(dmat[0]) : f2splat(0.f);
+  const float2 dm1 = TWO && KIND != kRaw ? pair_material(dmat[1]) : f2splat(0.f);
   auto material = [&](unsigned char id) {
     return TWO ? make_float2(id ? dm1.x : dm0.x, id ? dm1.y : dm0.y) : dm[id];
   };
@@ -223,23 +250,20 @@ __device__ __forceinline__ void pair_x1_component(const GridDev& g, const float2
                                                   const float4* r2c, const float2* hw) {
   const size_t nf2 = (size_t)g.n / 2;
   const float2* own = in + c * nf2;
-  // With at most two phases the material table is two register pairs and a
-  // select (phase ids are < n_phases), which takes the table lookups off the
-  // shared-memory pipe.
   if (mode == GM_RAW_TAU) {
-    pair_x1<C, kRaw, true, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
+    pair_x1<C, kRaw, true, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   } else if (c >= 3) {
     if (g.n_phases <= 2)
-      pair_x1<C, kShear, true, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
+      pair_x1<C, kShear, true, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
     else
-      pair_x1<C, kShear, false, PACK>(own, in, in, phase, low, rows, dm, P, twx, r2c, hw);
+      pair_x1<C, kShear, false, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   } else {
     const float2* other = in + (c == 0 ? 1 : 0) * nf2;
     const float2* last = in + (c == 2 ? 1 : 2) * nf2;
     if (g.n_phases <= 2)
-      pair_x1<C, kNormal, true, PACK>(own, other, last, phase, low, rows, dm, P, twx, r2c, hw);
+      pair_x1<C, kNormal, true, PACK>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
     else
-      pair_x1<C, kNormal, false, PACK>(own, other, last, phase, low, rows, dm, P, twx, r2c, hw);
+      pair_x1<C, kNormal, false, PACK>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   }
 }
 
@@ -315,12 +339,12 @@ __device__ __forceinline__ void pair_x2(float4* P, int rows, const float4* r2c, 
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
+template <int N, int TPB>
+__global__ void __launch_bounds__(TPB, PairPlane<N, TPB>::MINB)
     k_pair_fwd(GridDev g, const float* __restrict__ in, float4* __restrict__ spec, int mode) {
-  using C = PairPlane<N>;
+  using C = PairPlane<N, TPB>;
   using X = typename C::X;
-  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, TPB = C::TPB;
+  constexpr int NXH = C::NXH, SX = C::SX, H = C::H;
   constexpr int Y1 = C::Y1, Y2 = C::Y2;
   extern __shared__ __align__(128) float4 sm4[];
   float4* P = sm4;                     // [H][SX]
@@ -330,7 +354,6 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
   float2* hw = reinterpret_cast<float2*>(r2c + NXH);   // W_ny^j, j < ny/2
   float2* dm = hw + H;
   const int c = blockIdx.x, z = blockIdx.y;
-  allow_dependent_launch();
   for (int i = threadIdx.x; i < NXH; i += TPB) {
     twx[i] = splat_twiddle(g.p_twx[i]);
     r2c[i] = splat_twiddle(g.r2c_w[i]);
@@ -340,15 +363,26 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
     hw[i] = g.p_hw[i];
   }
   grid_dependency_wait();   // the FFT tables are fixed; everything below may be in flight
-  for (int i = threadIdx.x; i < 256; i += TPB) {   // (lam, 2 mu) of C - C0 per phase
-    const float2 m = g.dmat[i];
-    dm[i] = make_float2(m.x, 2.f * m.y);
+  pair_materials(g, dm, TPB);
+  __syncthreads();
+  pair_x1_component<X, C::PACK>(g, reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH, c,
+                                reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH,
+                                H * NXH, H, mode, dm, P, twx, r2c, hw);
+  __syncthreads();
+  float4* out = spec + ((size_t)c * g.nz + z) * C::PL;
+  if constexpr (!C::PACK) {   // one y step, straight to global memory
+    static_assert(Y2 == 1, "single-step x and y lengths go together");
+    allow_dependent_launch();
+    for (int b = threadIdx.x; b < C::COLS; b += TPB) {
+      C2 v[Y1];
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) v[i] = c2_load(P + i * SX + b);
+      PairDft<Y1, false>::run(v);
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) c2_store(out + i * SX + b, v[i]);
+    }
+    return;
   }
-  __syncthreads();
-  pair_x1_component<X, true>(g, reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH, c,
-                             reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH,
-                             H * NXH, H, mode, dm, P, twx, r2c, hw);
-  __syncthreads();
   pair_x2<X, true>(P, H, r2c, hw);
   __syncthreads();
   for (int t = threadIdx.x; t < NXH * Y2; t += TPB) {   // y step 1
@@ -364,7 +398,7 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
       c2_store(p + k1 * Y2 * SX, c2_mul<false>(v[k1], twy + k1 * Y2 + n2));
   }
   __syncthreads();
-  float4* out = spec + ((size_t)c * g.nz + z) * C::PL;
+  allow_dependent_launch();
   for (int t = threadIdx.x; t < NXH * Y1; t += TPB) {   // y step 2 -> global
     const int b = t % NXH, k1 = t / NXH;
     float4* p = P + b + k1 * Y2 * SX;
@@ -518,13 +552,13 @@ __device__ __forceinline__ float post_shear(float e, float b, float4 pm, float m
 // blocks of a plane, which need tr(eps_b), keep their real planes in shared
 // memory and each finishes all three normal components on a third of the
 // plane, reading the other two planes from the cluster's shared memory.
-template <int N, bool POST>
-__global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
+template <int N, int TPB, bool POST>
+__global__ void __launch_bounds__(TPB, PairPlane<N, TPB>::MINB)
     k_pair_inv(GridDev g, const float4* __restrict__ spec, float* __restrict__ outp, float scale,
                const float* __restrict__ eps, const float4* __restrict__ post) {
-  using C = PairPlane<N>;
+  using C = PairPlane<N, TPB>;
   using X = typename C::X;
-  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, PL = C::PL, TPB = C::TPB;
+  constexpr int NXH = C::NXH, SX = C::SX, H = C::H, PL = C::PL;
   constexpr int X1 = C::X1, X2 = C::X2, Y1 = C::Y1, Y2 = C::Y2;
   extern __shared__ __align__(128) float4 sm4[];
   float4* P = sm4;
@@ -538,7 +572,6 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
   const int c = POST ? (int)blockIdx.x % 6 : (int)blockIdx.x / g.nz;
   const int z = POST ? (int)blockIdx.x / 6 : (int)blockIdx.x - c * g.nz;
   const bool gather = POST && c < 3;   // a normal block of a post-step cluster
-  allow_dependent_launch();
   if (threadIdx.x == 0) {
     fail = 0;
     mbar_init(&bar, 1);
@@ -573,6 +606,16 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
     }
     return;
   }
+  if constexpr (!C::PACK) {
+    for (int b = threadIdx.x; b < C::COLS; b += TPB) {
+      C2 v[Y1];
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) v[i] = c2_load(P + i * SX + b);
+      PairDft<Y1, true>::run(v);
+#pragma unroll
+      for (int i = 0; i < Y1; ++i) c2_store(P + i * SX + b, v[i]);
+    }
+  } else {
   for (int t = threadIdx.x; t < NXH * Y1; t += TPB) {   // y step 1 (inverse)
     const int b = t % NXH, k1 = t / NXH;
     float4* p = P + k1 * Y2 * SX + b;
@@ -601,7 +644,9 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
   }
   __syncthreads();
   pair_x1_inv<X, true>(P, H, twx, r2c, hw);
+  }
   __syncthreads();
+  allow_dependent_launch();
   constexpr int LOW = H * NXH;         // row j + ny/2 lies LOW float2 after row j
   const size_t nf2 = (size_t)g.n / 2, zoff = (size_t)z * N * NXH;
   float2* out2 = reinterpret_cast<float2*>(outp) + zoff;
@@ -627,8 +672,12 @@ __global__ void __launch_bounds__(PairPlane<N>::TPB, PairPlane<N>::MINB)
       }
     }
     C2 v[X1];
+    if constexpr (X2 == 1) {
+      pair_tangle_row<NXH>(p, r2c, hw[j], v);
+    } else {
 #pragma unroll
-    for (int i = 0; i < X1; ++i) v[i] = c2_load(p + i * X2);
+      for (int i = 0; i < X1; ++i) v[i] = c2_load(p + i * X2);
+    }
     PairDft<X1, true>::run(v);
     float2* o = out2 + c * nf2 + r;
     if (gather) {   // -> the block's own slots, for the cluster's post-step
@@ -767,23 +816,20 @@ __global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
   float2* dm = hw + R;
   const int c = blockIdx.x, j0 = blockIdx.y * R, z = blockIdx.z;
   const int h = g.ny / 2, rows = min(R, h - j0);
-  allow_dependent_launch();
   for (int i = threadIdx.x; i < NXH; i += TPB) {
     twx[i] = splat_twiddle(g.p_twx[i]);
     r2c[i] = splat_twiddle(g.r2c_w[i]);
   }
   for (int i = threadIdx.x; i < rows; i += TPB) hw[i] = g.p_hw[j0 + i];
   grid_dependency_wait();
-  for (int i = threadIdx.x; i < 256; i += TPB) {   // (lam, 2 mu) of C - C0 per phase
-    const float2 m = g.dmat[i];
-    dm[i] = make_float2(m.x, 2.f * m.y);
-  }
+  pair_materials(g, dm, TPB);
   __syncthreads();
   const size_t row0 = ((size_t)z * g.ny + j0) * NXH;
   pair_x1_component<X, false>(g, reinterpret_cast<const float2*>(in) + row0, c,
                               reinterpret_cast<const uchar2*>(g.phase) + row0, h * NXH, rows,
                               mode, dm, P, twx, r2c, hw);
   __syncthreads();
+  allow_dependent_launch();
   pair_x2<X, false>(P, rows, r2c, hw);
   fence_async_smem();
   __syncthreads();
@@ -809,7 +855,6 @@ __global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
   __shared__ int fail;
   const int c = blockIdx.x, j0 = blockIdx.y * R, z = blockIdx.z;
   const int h = g.ny / 2, rows = min(R, h - j0);
-  allow_dependent_launch();
   if (threadIdx.x == 0) {
     fail = 0;
     mbar_init(&bar, 1);
@@ -837,6 +882,7 @@ __global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
   }
   pair_x1_inv<X, false>(P, rows, twx, r2c, hw);
   if (X2 > 1) __syncthreads();
+  allow_dependent_launch();
   const size_t nf2 = (size_t)g.n / 2;
   const int low = h * NXH;
   const size_t at0 = c * nf2 + ((size_t)z * g.ny + j0) * NXH;
@@ -885,8 +931,9 @@ __global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
 template <int H, bool INV>
 struct PairLines {
   static constexpr int Y1 = pair_n1(H), Y2 = H / Y1;
-  static constexpr int TPB = 128, T = Y2 == 1 ? TPB : (INV ? 8 : 16), HP = H | 1;
-  static constexpr size_t SMEM = Y2 == 1 ? 0 : (size_t)(T * HP + H) * sizeof(float4);
+  static constexpr bool ONE = H <= 16;   // a thread takes a whole line
+  static constexpr int TPB = 128, T = ONE ? TPB : (INV ? 8 : 16), HP = H | 1;
+  static constexpr size_t SMEM = ONE ? 0 : (size_t)(T * HP + H) * sizeof(float4);
 };
 
 template <int H, bool INV>
@@ -899,24 +946,24 @@ __global__ void __launch_bounds__(PairLines<H, INV>::TPB, 4)
   float4* twy = B + T * HP;
   const int SX = g.nxh + 1, cols = 6 * g.nz * SX;
   const int m0 = blockIdx.x * T;
-  allow_dependent_launch();
-  if (Y2 > 1)
+  if (!C::ONE)
     for (int i = threadIdx.x; i < H; i += TPB) twy[i] = splat_twiddle(g.p_twy[i]);
   grid_dependency_wait();
-  if (Y2 > 1) __syncthreads();
+  if (!C::ONE) __syncthreads();
   auto column = [&](int t) {   // first element of column m0 + t (rows SX apart)
     const int m = m0 + t, pl = m / SX;
     return spec + (size_t)pl * H * SX + (m - pl * SX);
   };
-  if constexpr (Y2 == 1) {
+  if constexpr (C::ONE) {
     if (m0 + (int)threadIdx.x < cols) {
       float4* p = column(threadIdx.x);
-      C2 v[Y1];
+      C2 v[H];
 #pragma unroll
-      for (int i = 0; i < Y1; ++i) v[i] = c2_load(p + (size_t)i * SX);
-      PairDft<Y1, INV>::run(v);
+      for (int i = 0; i < H; ++i) v[i] = c2_load(p + (size_t)(INV ? split_slot(H, Y1, i) : i) * SX);
+      allow_dependent_launch();
+      PairDft<H, INV>::run(v);
 #pragma unroll
-      for (int i = 0; i < Y1; ++i) c2_store(p + (size_t)i * SX, v[i]);
+      for (int i = 0; i < H; ++i) c2_store(p + (size_t)(INV ? i : split_slot(H, Y1, i)) * SX, v[i]);
     }
     return;
   }
@@ -936,6 +983,7 @@ __global__ void __launch_bounds__(PairLines<H, INV>::TPB, 4)
       c2_store(b + (INV ? i : i * Y2), c2_mul<INV>(v[i], twy + (INV ? k * Y2 + i : i * Y2 + k)));
   }
   __syncthreads();
+  allow_dependent_launch();
   for (int q = threadIdx.x; q < T * A1; q += TPB) {
     const int t = q % T, k = q / T;   // k: k1 forward, n2 inverse
     if (m0 + t >= cols) continue;
@@ -1195,7 +1243,6 @@ __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
   __shared__ int flag[T];
   const int m0 = blockIdx.x * T;
   const int plane = (g.ny / 2) * (g.nxh + 1);   // pencil pairs
-  allow_dependent_launch();
   for (int i = threadIdx.x; i < NZ; i += TPB) twz[i] = splat_twiddle(g.p_twz[i]);
   if (threadIdx.x < T) pair_pencil(g, m0 + threadIdx.x, plane, pen + threadIdx.x, flag + threadIdx.x);
   grid_dependency_wait();
@@ -1220,6 +1267,7 @@ __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
   __syncthreads();
   pair_z_middle<NZ, T, TPB>(g, B, twz, pen, flag, mode, ga);
   __syncthreads();
+  allow_dependent_launch();
   for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {   // inverse step 2 -> global
     const int t = q % T, c = (q / T) % 6, n2 = q / (6 * T);
     const int m = m0 + t;
@@ -1245,7 +1293,6 @@ __global__ void __launch_bounds__(kShortTPB) k_pair_green_short(GridDev g,
                                                                 float4* __restrict__ spec, int mode,
                                                                 GammaArgs ga) {
   const int plane = (g.ny / 2) * (g.nxh + 1), m = blockIdx.x * kShortTPB + threadIdx.x;
-  allow_dependent_launch();
   float4 q;
   int fl;
   pair_pencil(g, m, plane, &q, &fl);
@@ -1256,6 +1303,7 @@ __global__ void __launch_bounds__(kShortTPB) k_pair_green_short(GridDev g,
   for (int c = 0; c < 6; ++c)
 #pragma unroll
     for (int i = 0; i < NZ; ++i) v[c][i] = c2_load(spec + ((size_t)c * NZ + i) * plane + m);
+  allow_dependent_launch();
 #pragma unroll
   for (int c = 0; c < 6; ++c) PairDft<NZ, false>::run(v[c]);
 #pragma unroll
@@ -1303,7 +1351,6 @@ __global__ void __launch_bounds__(PairZStream<NZ, T>::TPB, 1)
   __shared__ float4 pen[T];
   __shared__ int flag[T];
   const int plane = (g.ny / 2) * (g.nxh + 1), tiles = (plane + T - 1) / T;
-  allow_dependent_launch();
   for (int i = threadIdx.x; i < NZ; i += TPB) twz[i] = splat_twiddle(g.p_twz[i]);
   grid_dependency_wait();
   auto prefetch = [&](int tile) {
@@ -1333,6 +1380,8 @@ __global__ void __launch_bounds__(PairZStream<NZ, T>::TPB, 1)
     }
     __syncthreads();
     if (tile + (int)gridDim.x < tiles) prefetch(tile + gridDim.x);
+    else
+      allow_dependent_launch();   // the block's last tile
     pair_z_middle<NZ, T, TPB>(g, B, twz, pen, flag, mode, ga);
     __syncthreads();
     for (int q = threadIdx.x; q < 6 * T * Z2; q += TPB) {   // inverse step 2 -> global
@@ -1374,39 +1423,41 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 template <int N>
 size_t plane_smem(bool table) {
-  using C = PairPlane<N>;
+  using C = PairPlane<N, 32>;
   return (size_t)(C::PL + 2 * C::NXH + C::H) * sizeof(float4) + C::H * sizeof(float2) +
          (table ? 256 * sizeof(float2) : 0);
 }
 
-template <int N>
+template <int N, int TPB>
 cudaError_t launch_fwd(const GridDev& g, const float* in, float4* spec, int mode, cudaStream_t st) {
   const size_t smem = plane_smem<N>(true);
-  cudaError_t e = set_smem(k_pair_fwd<N>, smem);
+  cudaError_t e = set_smem(k_pair_fwd<N, TPB>, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_pair_fwd<N>, dim3(6, g.nz), PairPlane<N>::TPB, smem, st, g, in, spec, mode);
+  return launch_pdl(k_pair_fwd<N, TPB>, dim3(6, g.nz), TPB, smem, st, g, in, spec, mode);
 }
 
-template <int N>
-cudaError_t launch_inv(const GridDev& g, float* out, const float4* spec, const float* add,
-                       cudaStream_t st) {
+// pass C, or with a post table its form with Algorithm 3's post-step (clusters
+// of three blocks, `eps` being the map's input)
+template <int N, int TPB>
+cudaError_t launch_inv(const GridDev& g, float* out, const float4* spec, const float* eps,
+                       const float4* post, cudaStream_t st) {
+  const float scale = 0.5f / (float)g.n;
+  cudaError_t e;
+  if (post) {
+    const size_t smem = plane_smem<N>(false) + 256 * sizeof(float4);
+    if ((e = set_smem(k_pair_inv<N, TPB, true>, smem)) != cudaSuccess) return e;
+    return launch_pdl_cluster(k_pair_inv<N, TPB, true>, dim3(6 * g.nz), TPB, smem, st, 3u, g, spec,
+                              out, scale, eps, post);
+  }
   const size_t smem = plane_smem<N>(false);
-  cudaError_t e = set_smem(k_pair_inv<N, false>, smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_pair_inv<N, false>, dim3(6 * g.nz), PairPlane<N>::TPB, smem, st, g, spec,
-                    out, 0.5f / (float)g.n, add, (const float4*)nullptr);
+  if ((e = set_smem(k_pair_inv<N, TPB, false>, smem)) != cudaSuccess) return e;
+  return launch_pdl(k_pair_inv<N, TPB, false>, dim3(6 * g.nz), TPB, smem, st, g, spec, out, scale,
+                    eps, post);
 }
 
-// pass C with Algorithm 3's post-step (clusters of three blocks)
-template <int N>
-cudaError_t launch_inv_post(const GridDev& g, float* out, const float4* spec, const float* eps,
-                            const float4* post, cudaStream_t st) {
-  const size_t smem = plane_smem<N>(false) + 256 * sizeof(float4);
-  cudaError_t e = set_smem(k_pair_inv<N, true>, smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl_cluster(k_pair_inv<N, true>, dim3(6 * g.nz), PairPlane<N>::TPB, smem, st, 3u,
-                            g, spec, out, 0.5f / (float)g.n, eps, post);
-}
+// At 96^2, blocks of 128 threads pay once there are enough of them for two per
+// SM; below, a block of 256 finishes its plane sooner (24 x 96 x 96: map 25 -> 19 us).
+bool few_planes(const GridDev& g) { return 6 * g.nz <= 304; }
 
 // Row pairs per block: enough for four blocks an SM, or few where the grid is small.
 template <int NX>
@@ -1435,7 +1486,7 @@ template <int NX>
 cudaError_t launch_rows(const GridDev& g, const float* in, float* out, float4* spec, int mode,
                         bool inv, const float* add, cudaStream_t st) {
   using T = RowsTile<NX>;
-  if ((long long)6 * g.nz * (g.ny / 2) >= 600LL * T::BIG)
+  if ((long long)6 * g.nz * (g.ny / 2) >= 140LL * T::BIG)
     return launch_rows_r<NX, T::BIG>(g, in, out, spec, mode, inv, add, st);
   return launch_rows_r<NX, T::SMALL>(g, in, out, spec, mode, inv, add, st);
 }
@@ -1447,14 +1498,6 @@ cudaError_t launch_lines(const GridDev& g, float4* spec, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const int cols = 6 * g.nz * (g.nxh + 1);
   const dim3 grid((cols + C::T - 1) / C::T);
-  // Next to a z block that takes most of an SM's shared memory (nz = 256) the
-  // lines that start early run with what L1 is left of it: 256^3 990 us a map
-  // so, 837 us with an ordinary launch after the z pass, 827 us with one
-  // before it too (a loss on smaller grids, 96 x 48 x 256: 75.8 against 77.7 us).
-  if (g.nz >= 256 && (INV || g.n >= 1 << 23)) {
-    k_pair_lines<H, INV><<<grid, C::TPB, C::SMEM, st>>>(g, spec);
-    return cudaGetLastError();
-  }
   return launch_pdl(k_pair_lines<H, INV>, grid, C::TPB, C::SMEM, st, g, spec);
 }
 
@@ -1495,13 +1538,28 @@ cudaError_t launch_green_tile(const GridDev& g, float4* spec, int mode, const Ga
   }
 }
 
-#define RPM_PAIR_SIZES(X) X(48) X(64) X(96) X(128)
+#define RPM_PAIR_SIZES(X) \
+  X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128)
 #define RPM_PAIR_Z_SIZES(X) \
   X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
 
 cudaError_t pass_fwd(const GridDev& g, const float* in, float4* spec, int mode, cudaStream_t st) {
+  if (g.nx == 96 && few_planes(g))
+    return launch_fwd<96, pair_threads(96, true)>(g, in, spec, mode, st);
   switch (g.nx) {
-#define RPM_CASE(N) case N: return launch_fwd<N>(g, in, spec, mode, st);
+#define RPM_CASE(N) case N: return launch_fwd<N, pair_threads(N, false)>(g, in, spec, mode, st);
+    RPM_PAIR_SIZES(RPM_CASE)
+#undef RPM_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t pass_inv(const GridDev& g, float* out, const float4* spec, const float* eps,
+                     const float4* post, cudaStream_t st) {
+  if (g.nx == 96 && few_planes(g))
+    return launch_inv<96, pair_threads(96, true)>(g, out, spec, eps, post, st);
+  switch (g.nx) {
+#define RPM_CASE(N) case N: return launch_inv<N, pair_threads(N, false)>(g, out, spec, eps, post, st);
     RPM_PAIR_SIZES(RPM_CASE)
 #undef RPM_CASE
     default: return cudaErrorInvalidValue;
@@ -1555,18 +1613,22 @@ bool pair_plane_ok(const GridDev& g, const float2* spec) {
   }
 }
 
-// Pencil pairs per z block: the largest of 8 (128-byte rows), 4 and 2 that
-// still gives some 250 blocks, so that every SM has more than one (64^3: T = 4
-// 5.6 us, T = 8 7.7 us; 48^3: T = 2 4.2 us, T = 4 4.4 us; 96^3: T = 8 11.7 us,
-// T = 4 15.2 us).  From nz = 128 on a block of 8 takes 100 KB of shared memory,
-// and the last pass cannot start while it drains: the 128^3 map takes 96 us
-// with T = 8, 84 us with T = 4, although the pass alone differs by 1 us.
+// Pencil pairs per z block T: the largest that still gives every SM a block or
+// two (measured: a second, partly filled round of blocks costs more than 32- or
+// 64-byte rows do).  64^3: T = 4, 264 blocks, 5.6 us a pass (T = 2 9.0, T = 8
+// 7.7); 64 x 24 x 128: T = 4, 195 blocks, 5.3 us (T = 2 8.2); 48^3: T = 2, 300
+// blocks, 4.2 us (T = 4 4.4).  nz = 96, where three blocks of T = 4 fit an SM:
+// T = 8 from 290 blocks on (96^3 11.7 us, T = 4 15.2; 96 x 64 x 96 T = 4 10.2,
+// T = 8 11.6).  nz = 128: never above 4, the last pass cannot start while the
+// 100 KB blocks drain.  nz = 256: T = 4 is the persistent kernel, worth it from
+// one tile per SM on (256 x 48 x 48: 9.2 us, T = 2 12.8).
 int pair_z_tile(const GridDev& g) {
   const int pencils = (g.ny / 2) * (g.nxh + 1);
-  int t = g.nz >= 128 ? 4 : 8;
-  while (t > 2 && pencils < 250 * t) t /= 2;
+  const int blocks = g.nz == 96 ? 290 : (g.nz == 256 ? 140 : 190);
+  int t = g.nz <= 16 ? 16 : (g.nz >= 128 ? 4 : 8);
+  while (t > 2 && pencils < blocks * t) t /= 2;
   if (g.pencil_t == 1) t = t > 2 ? t / 2 : 2;
-  if (g.pencil_t == 2) t *= 2;
+  if (g.pencil_t == 2) t = t < 16 ? 2 * t : 16;
   return t;
 }
 
@@ -1576,12 +1638,7 @@ cudaError_t launch_pair_map(const GridDev& g, const float* in, float* out, float
   cudaError_t e;
   if ((e = pass_fwd(g, in, s4, mode, st)) != cudaSuccess) return e;
   if ((e = pass_green(g, s4, mode, E, st)) != cudaSuccess) return e;
-  switch (g.nx) {
-#define RPM_CASE(N) case N: return launch_inv<N>(g, out, s4, add, st);
-    RPM_PAIR_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
-  }
+  return pass_inv(g, out, s4, add, nullptr, st);
 }
 
 cudaError_t launch_pair_rows_map(const GridDev& g, const float* in, float* out, float2* spec,
@@ -1602,12 +1659,7 @@ cudaError_t launch_pair_polarization(const GridDev& g, const float4* post, const
   cudaError_t e;
   if ((e = pass_fwd(g, in, s4, mode, st)) != cudaSuccess) return e;
   if ((e = pass_green(g, s4, mode, Eb, st)) != cudaSuccess) return e;
-  switch (g.nx) {
-#define RPM_CASE(N) case N: return launch_inv_post<N>(g, out, s4, in, post, st);
-    RPM_PAIR_SIZES(RPM_CASE)
-#undef RPM_CASE
-    default: return cudaErrorInvalidValue;
-  }
+  return pass_inv(g, out, s4, in, post, st);
 }
 
 void pair_tables(int nx, int ny, int nz, PairTables* t) {

@@ -228,11 +228,15 @@ struct PairDft<16, INV> {
 };
 
 // Split of a paired line into its two register steps, L = n1 * (L / n1).  Plane
-// lines (x: nx/2, y: ny/2): radix 8 first, 32 data registers a thread.  z lines:
+// lines (x: nx/2, y: ny/2): one step up to 12 points, 4 x 4 at 16 (four times
+// the threads of one 16-point step: 32^3 map 17.9 -> 14.0 us), then radix 8 first, 32 data
+// registers a thread.  z lines:
 // a 16-point first step, so that the middle step of the z pass, which holds
 // three components of each frequency, stays short (nz = 64: 16 x 4 points
 // 5.6 us a pass, 8 x 8 points 7.9 us; nz = 48: 16 x 3 4.9 us, 8 x 6 5.1 us).
-__host__ __device__ constexpr int pair_n1(int L) { return L <= 16 ? L : (L <= 64 ? 8 : 16); }
+__host__ __device__ constexpr int pair_n1(int L) {
+  return L <= 12 ? L : (L == 16 ? 4 : (L <= 64 ? 8 : 16));
+}
 __host__ __device__ constexpr int pair_z1(int L) { return L <= 16 ? L : (L <= 32 ? 8 : 16); }
 // Slot s = k1 * n2 + k2 of a line with first factor n1 holds frequency k1 + n1 * k2.
 __host__ __device__ constexpr int split_freq(int L, int n1, int s) {

@@ -1,4 +1,4 @@
-"""The paired kernels (square planes of side 48-128, and the five-pass form on
+"""The paired kernels (square planes of side up to 128, and the five-pass form on
 any grid) against the FP64 oracle over the z lengths and options their z pass distinguishes: single-step and
 two-step lengths, each number of pencils per block, a ragged last block,
 non-unit cell lengths, a material table of more than two phases."""
@@ -42,7 +42,10 @@ def _check(shape, pencil, plane):
 
 @pytest.mark.parametrize("nz,n", [(1, 128), (2, 64), (3, 96), (4, 48), (6, 64), (8, 48), (12, 96),
                                   (16, 64), (24, 48), (32, 48), (48, 96), (64, 48), (96, 48),
-                                  (128, 96), (256, 64)])
+                                  (128, 96), (256, 64),
+                                  # one-warp planes
+                                  (32, 32), (24, 24), (16, 16), (6, 12), (8, 8), (6, 6), (3, 4),
+                                  (128, 32), (1, 16), (256, 24)])
 @pytest.mark.parametrize("pencil", [0, 1, 2])
 def test_paired_map_matches_oracle(nz, n, pencil):
     _check((nz, n, n), pencil, 0)
