@@ -11,12 +11,13 @@
 
 #include <atomic>
 
+#include "async_copy.cuh"
 #include "rpm_internal.h"
 
 namespace rpm {
 
 constexpr int kRedThreads = 256;
-constexpr int kPerThread = 8;        // float4 per thread per dot pass (32 products)
+constexpr int kPerThread = 8;        // float4 per thread per dot pass on large grids (32 products)
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -84,64 +85,75 @@ __device__ __forceinline__ float dot4(float4 a, float4 b) {
 // any product, so Z^T (xi - eps) keeps its accuracy when xi and eps agree to
 // many digits (near convergence).
 // Partial sums go to rows [0] (the norm) and [1 + row0 + j] of `partials`.
-template <int KMAX>
+// NX = 2: the same of a second field x2 (no xm), its rows after the first's
+// K + 1; every Y_j is read once for both.
+// PT: float4 per thread (see dots_per_thread).
+template <int KMAX, int PT, int NX>
 __device__ __forceinline__ void dots_body(const float4* __restrict__ x,
+                                          const float4* __restrict__ x2,
                                           const float4* __restrict__ xm,
                                           const float4* __restrict__ Y, long long ys4, int K,
                                           int row0, long long n4, double* partials, int nblk) {
-  // The thread's kPerThread difference vectors stay in registers; each basis
-  // vector is then read as kPerThread independent 16-byte loads issued
-  // together, and its warp sum is taken at once (no accumulator stays live
-  // across the vectors, which keeps the register count at three blocks per SM).
-  __shared__ double red[kRedThreads / 32][KMAX + 1];
+  // The thread's PT difference vectors stay in registers; each basis vector is
+  // then read as PT independent 16-byte loads issued together, and its warp
+  // sum is taken at once (no accumulator stays live across the vectors, which
+  // keeps the register count at three blocks per SM).
+  __shared__ double red[kRedThreads / 32][NX * (KMAX + 1)];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long total = 6 * n4;
-  const long long base = (long long)blockIdx.x * kRedThreads * kPerThread + threadIdx.x;
-  float4 d[kPerThread];
-  float w[kPerThread];
+  const long long base = (long long)blockIdx.x * kRedThreads * PT + threadIdx.x;
+  const float4* xs[2] = {x, x2};
+  float4 d[NX][PT];
+  float w[PT];
 #pragma unroll
-  for (int r = 0; r < kPerThread; ++r) {
-    const long long q = base + (long long)r * kRedThreads;
-    const bool in = q < total;
-    w[r] = in ? ((q >= 3 * n4) ? 2.f : 1.f) : 0.f;
-    d[r] = in ? x[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  if (xm) {
+  for (int v = 0; v < NX; ++v)
 #pragma unroll
-    for (int r = 0; r < kPerThread; ++r) {
+    for (int r = 0; r < PT; ++r) {
+      const long long q = base + (long long)r * kRedThreads;
+      const bool in = q < total;
+      w[r] = in ? ((q >= 3 * n4) ? 2.f : 1.f) : 0.f;
+      d[v][r] = in ? xs[v][q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  if (NX == 1 && xm) {
+#pragma unroll
+    for (int r = 0; r < PT; ++r) {
       const long long q = base + (long long)r * kRedThreads;
       if (q < total) {
         const float4 b = xm[q];
-        d[r] = make_float4(d[r].x - b.x, d[r].y - b.y, d[r].z - b.z, d[r].w - b.w);
+        d[0][r] = make_float4(d[0][r].x - b.x, d[0][r].y - b.y, d[0][r].z - b.z, d[0][r].w - b.w);
       }
     }
   }
-  {
+#pragma unroll
+  for (int v = 0; v < NX; ++v) {
     float a = 0.f, hi, lo;
 #pragma unroll
-    for (int r = 0; r < kPerThread; ++r) a = fmaf(w[r], dot4(d[r], d[r]), a);
+    for (int r = 0; r < PT; ++r) a = fmaf(w[r], dot4(d[v][r], d[v][r]), a);
     warp_sum_compensated(a, hi, lo);
-    if (lane == 0) red[warp][0] = (double)hi + (double)lo;
+    if (lane == 0) red[warp][v * (K + 1)] = (double)hi + (double)lo;
   }
 #pragma unroll
   for (int j = 0; j < KMAX; ++j) {
     if (j < K) {
       const float4* yj = Y + j * ys4;
-      float4 y[kPerThread];
+      float4 y[PT];
 #pragma unroll
-      for (int r = 0; r < kPerThread; ++r) {
+      for (int r = 0; r < PT; ++r) {
         const long long q = base + (long long)r * kRedThreads;
         y[r] = q < total ? yj[q] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      float a = 0.f, hi, lo;
 #pragma unroll
-      for (int r = 0; r < kPerThread; ++r) a = fmaf(w[r], dot4(d[r], y[r]), a);
-      warp_sum_compensated(a, hi, lo);
-      if (lane == 0) red[warp][1 + j] = (double)hi + (double)lo;
+      for (int v = 0; v < NX; ++v) {
+        float a = 0.f, hi, lo;
+#pragma unroll
+        for (int r = 0; r < PT; ++r) a = fmaf(w[r], dot4(d[v][r], y[r]), a);
+        warp_sum_compensated(a, hi, lo);
+        if (lane == 0) red[warp][v * (K + 1) + 1 + j] = (double)hi + (double)lo;
+      }
     }
   }
   __syncthreads();
-  for (int j = threadIdx.x; j <= K; j += blockDim.x) {
+  for (int j = threadIdx.x; j < NX * (K + 1); j += blockDim.x) {
     if (j == 0 && row0 != 0) continue;
     double t = 0.0;
 #pragma unroll
@@ -156,21 +168,30 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_dots(const float4* __restric
                                                       const float4* __restrict__ Y, long long ys4,
                                                       int K, int row0, long long n4,
                                                       double* partials, int nblk) {
-  dots_body<KMAX>(x, xm, Y, ys4, K, row0, n4, partials, nblk);
+  dots_body<KMAX, kPerThread, 1>(x, nullptr, xm, Y, ys4, K, row0, n4, partials, nblk);
 }
 
-// k_dots (K <= 32) whose last block to finish also adds the per-block rows in
+// Dots (K <= 32) whose last block to finish also adds the per-block rows in
 // a fixed order (a warp per row: lanes take every 32nd block, then a fixed
-// shuffle tree) into sums[0..K] and, when M is given, takes the Newton step
-// of k_newton with p = K.  The ticket counter is zero between launches (the
-// last block resets it).  One launch instead of three.
-template <int KMAX>
-__global__ void __launch_bounds__(kRedThreads, 3) k_dots_fused(
-    const float4* __restrict__ x, const float4* __restrict__ xm, const float4* __restrict__ Y,
-    long long ys4, int K, long long n4, double* partials, int nblk, double* sums,
-    unsigned int* ticket, const double* __restrict__ M, double* c, double* res_out,
-    double inv_norm) {
-  dots_body<KMAX>(x, xm, Y, ys4, K, 0, n4, partials, nblk);
+// shuffle tree) into sums[0..NX (K + 1)) and, when M is given, takes the Newton
+// step of k_newton with p = K.  The ticket counter is zero between launches
+// (the last block resets it).  One launch instead of three.
+// Large grids: bound by HBM (128^3, p = 20: 174 us, 94 % of the copy rate).
+// Small ones by latency: 32^3 solve 1.64 -> 0.90 ms, 48^3 1.63 -> 1.16 ms with
+// the polled reads, more blocks, launches that overlap and both differences of
+// a growth at once; 96^3 cold solve 9.8 -> 8.2 ms.
+// With a host block (pinned memory) the sums, and the residual when M is
+// given, also go there, followed by the sequence number the host polls: a read
+// costs neither a copy nor a stream synchronisation.
+template <int KMAX, int PT, int NX>
+__global__ void __launch_bounds__(kRedThreads, NX == 2 ? 2 : 3) k_dots_fused(
+    const float4* __restrict__ x, const float4* __restrict__ x2, const float4* __restrict__ xm,
+    const float4* __restrict__ Y, long long ys4, int K, long long n4, double* partials, int nblk,
+    double* sums, unsigned int* ticket, const double* __restrict__ M, double* c, double* res_out,
+    double inv_norm, HostRead host) {
+  grid_dependency_wait();
+  dots_body<KMAX, PT, NX>(x, x2, xm, Y, ys4, K, 0, n4, partials, nblk);
+  allow_dependent_launch();
   __shared__ bool last;
   __threadfence();
   __syncthreads();
@@ -179,7 +200,7 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_dots_fused(
   if (!last) return;
   __threadfence();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int j = warp; j <= K; j += kRedThreads / 32) {
+  for (int j = warp; j < NX * (K + 1); j += kRedThreads / 32) {
     // 8 independent chains per lane (loads in flight), added in a fixed order
     const double* row = partials + (size_t)j * nblk;
     double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -193,7 +214,10 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_dots_fused(
       if (b + q * 32 < nblk) v[q] += __ldcg(row + b + q * 32);
     double t = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
     t = warp_sum(t);
-    if (lane == 0) sums[j] = t;
+    if (lane == 0) {
+      sums[j] = t;
+      if (host.sums) host.sums[j] = t;
+    }
   }
   __syncthreads();
   if (M) {
@@ -205,39 +229,74 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_dots_fused(
       for (int k = 0; k < K; ++k) t += M[(size_t)j * K + k] * d[k];
       c[j] = t;
     }
-    if (threadIdx.x == 0) res_out[0] = sqrt(sums[0]) * inv_norm;   // NaN stays NaN
+    if (threadIdx.x == 0) {
+      const double r = sqrt(sums[0]) * inv_norm;   // NaN stays NaN
+      res_out[0] = r;
+      if (host.res) *host.res = r;
+    }
   }
-  if (threadIdx.x == 0) *ticket = 0u;
+  if (host.sums) __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *ticket = 0u;
+    if (host.seq) {
+      __threadfence_system();
+      *reinterpret_cast<volatile unsigned long long*>(host.seq) = host.value;
+    }
+  }
 }
 
-cudaError_t launch_dots_fused(const float* x, const float* x_minus, const float* Y,
-                              long long ystride, int K, long long n, double* partials, int nblk,
-                              double* sums, unsigned int* ticket, const double* M, double* c,
-                              double* res_out, double inv_norm, cudaStream_t st) {
+// float4 per thread of a dots pass: eight where that still gives two blocks per
+// SM, fewer on smaller grids, whose passes would leave most SMs idle.
+static int dots_per_thread(long long n) {
+  const long long total = 6 * (n / 4);
+  return total >= 304LL * kRedThreads * 8 ? 8 : (total >= 304LL * kRedThreads * 4 ? 4 : 2);
+}
+
+template <int PT, int NX>
+static cudaError_t dots_fused_k(const float4* x, const float4* x2, const float4* xm,
+                                const float4* Y, long long ys4, int K, long long n4,
+                                double* partials, int nblk, double* sums, unsigned int* ticket,
+                                const double* M, double* c, double* res_out, double inv_norm,
+                                const HostRead& host, cudaStream_t st) {
+#define RPM_FUSED(KM)                                                                          \
+  launch_pdl(k_dots_fused<KM, PT, NX>, dim3(nblk), kRedThreads, 0, st, x, x2, xm, Y, ys4, K, n4, \
+             partials, nblk, sums, ticket, M, c, res_out, inv_norm, host)
+  if (K <= 2) return RPM_FUSED(2);
+  if (K <= 8) return RPM_FUSED(8);
+  if (K <= 16) return RPM_FUSED(16);
+  return RPM_FUSED(32);
+#undef RPM_FUSED
+}
+
+cudaError_t launch_dots_fused(const float* x, const float* x2, const float* x_minus,
+                              const float* Y, long long ystride, int K, long long n,
+                              double* partials, int nblk, double* sums, unsigned int* ticket,
+                              const double* M, double* c, double* res_out, double inv_norm,
+                              const HostRead& host, cudaStream_t st) {
   if (K > 32) return cudaErrorInvalidValue;
   const long long n4 = n / 4;
   const float4* x4 = reinterpret_cast<const float4*>(x);
+  const float4* z4 = reinterpret_cast<const float4*>(x2);
   const float4* m4 = reinterpret_cast<const float4*>(x_minus);
   const float4* y4 = reinterpret_cast<const float4*>(Y);
   const long long ys4 = ystride / 4;
-#define RPM_FUSED(KM)                                                                       \
-  k_dots_fused<KM><<<nblk, kRedThreads, 0, st>>>(x4, m4, y4, ys4, K, n4, partials, nblk, sums, \
-                                                 ticket, M, c, res_out, inv_norm)
-  if (K <= 2)
-    RPM_FUSED(2);
-  else if (K <= 8)
-    RPM_FUSED(8);
-  else if (K <= 16)
-    RPM_FUSED(16);
-  else
-    RPM_FUSED(32);
-#undef RPM_FUSED
-  return cudaGetLastError();
+#define RPM_PT(P)                                                                             \
+  (x2 ? dots_fused_k<P, 2>(x4, z4, m4, y4, ys4, K, n4, partials, nblk, sums, ticket, M, c,    \
+                           res_out, inv_norm, host, st)                                       \
+      : dots_fused_k<P, 1>(x4, z4, m4, y4, ys4, K, n4, partials, nblk, sums, ticket, M, c,    \
+                           res_out, inv_norm, host, st))
+  switch (dots_per_thread(n)) {
+    case 2: return RPM_PT(2);
+    case 4: return RPM_PT(4);
+    default: return RPM_PT(8);
+  }
+#undef RPM_PT
 }
 
 int dots_blocks_for(long long n) {
-  const long long total = 6 * (n / 4);
-  return (int)((total + (long long)kRedThreads * kPerThread - 1) / ((long long)kRedThreads * kPerThread));
+  const long long total = 6 * (n / 4), per = (long long)kRedThreads * dots_per_thread(n);
+  return (int)((total + per - 1) / per);
 }
 
 cudaError_t launch_dots(const float* x, const float* x_minus, const float* Y, long long ystride,
@@ -292,19 +351,29 @@ cudaError_t launch_reduce_partials(const double* partials, int nblk, int m, doub
 // out = xs * x + sum_j coef[j] * Y_j   (coef in float64 on the device)
 // (out may alias x).  The basis vectors are read in groups of 8 so that each
 // thread keeps 8 independent 16-byte loads in flight at a modest register count.
-template <int KMAX>
-__global__ void __launch_bounds__(kRedThreads, 3) k_combine(float4* out, const float4* x, float xs,
-                                                            const float4* __restrict__ Y,
-                                                            long long ys4, int K,
-                                                            const double* __restrict__ coef,
-                                                            float cscale, long long total4) {
-  __shared__ float cf[KMAX > 0 ? KMAX : 1];
-  for (int j = threadIdx.x; j < K; j += blockDim.x) cf[j] = (float)(coef[j] * (double)cscale);
+// NX = 2: a second field the same way (x2 -> out2, coefficients coef2), every
+// basis vector read once for both.
+template <int KMAX, int NX>
+__global__ void __launch_bounds__(kRedThreads, 3) k_combine(
+    float4* out, float4* out2, const float4* x, const float4* x2, float xs,
+    const float4* __restrict__ Y, long long ys4, int K, const double* __restrict__ coef,
+    const double* __restrict__ coef2, float cscale, long long total4) {
+  __shared__ float cf[NX][KMAX > 0 ? KMAX : 1];
+  grid_dependency_wait();
+  for (int j = threadIdx.x; j < K; j += blockDim.x) {
+    cf[0][j] = (float)(coef[j] * (double)cscale);
+    if (NX == 2) cf[NX - 1][j] = (float)(coef2[j] * (double)cscale);
+  }
   __syncthreads();
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total4;
        q += (long long)gridDim.x * blockDim.x) {
-    float4 a = x ? x[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-    a = make_float4(a.x * xs, a.y * xs, a.z * xs, a.w * xs);
+    float4 a[NX];
+#pragma unroll
+    for (int v = 0; v < NX; ++v) {
+      const float4* xv = v ? x2 : x;
+      a[v] = xv ? xv[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+      a[v] = make_float4(a[v].x * xs, a[v].y * xs, a[v].z * xs, a[v].w * xs);
+    }
 #pragma unroll 1
     for (int j0 = 0; j0 < K; j0 += 8) {
       float4 y[8];
@@ -314,15 +383,20 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_combine(float4* out, const f
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         if (j0 + u < K) {
-          const float c = cf[j0 + u];
-          a.x = fmaf(c, y[u].x, a.x);
-          a.y = fmaf(c, y[u].y, a.y);
-          a.z = fmaf(c, y[u].z, a.z);
-          a.w = fmaf(c, y[u].w, a.w);
+#pragma unroll
+          for (int v = 0; v < NX; ++v) {
+            const float c = cf[v][j0 + u];
+            a[v].x = fmaf(c, y[u].x, a[v].x);
+            a[v].y = fmaf(c, y[u].y, a[v].y);
+            a[v].z = fmaf(c, y[u].z, a[v].z);
+            a[v].w = fmaf(c, y[u].w, a[v].w);
+          }
         }
       }
     }
-    out[q] = a;
+    allow_dependent_launch();
+    out[q] = a[0];
+    if (NX == 2) out2[q] = a[NX - 1];
   }
 }
 
@@ -364,37 +438,49 @@ static int resident_grid(Kern kernel, long long total4, std::atomic<int>& slot) 
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
-static std::atomic<int> g_combine_occ[4];   // resident blocks per SM of k_combine<2, 8, 16, 32>
+static std::atomic<int> g_combine_occ[2][4];   // resident blocks per SM of k_combine<2, 8, 16, 32>
 
-cudaError_t launch_combine(float* out, const float* x, float xscale, const float* Y,
-                           long long ystride, int K, const double* coef, float cscale,
-                           long long n, cudaStream_t st) {
+template <int NX>
+static cudaError_t combine_k(float* out, float* out2, const float* x, const float* x2,
+                             float xscale, const float* Y, long long ystride, int K,
+                             const double* coef, const double* coef2, float cscale, long long n,
+                             cudaStream_t st) {
   const long long total4 = 6 * (n / 4);
-  float4* o4 = reinterpret_cast<float4*>(out);
+  float4 *o4 = reinterpret_cast<float4*>(out), *p4 = reinterpret_cast<float4*>(out2);
   const long long ys4 = ystride / 4;
   // K > 32: the first chunk forms xs * x + ..., later chunks accumulate into out
   for (int k0 = 0; k0 == 0 || k0 < K; k0 += 32) {
     const int Kc = K - k0 < 32 ? K - k0 : 32;
     const float4* x4 = k0 == 0 ? reinterpret_cast<const float4*>(x) : o4;
+    const float4* z4 = k0 == 0 ? reinterpret_cast<const float4*>(x2) : p4;
     const float xs = k0 == 0 ? xscale : 1.f;
     const float4* y4 = reinterpret_cast<const float4*>(Y) + (Y ? k0 * ys4 : 0);
     const double* cf = coef ? coef + k0 : nullptr;
-    if (Kc <= 2)
-      k_combine<2><<<resident_grid(k_combine<2>, total4, g_combine_occ[0]), kRedThreads, 0, st>>>(
-          o4, x4, xs, y4, ys4, Kc, cf, cscale, total4);
-    else if (Kc <= 8)
-      k_combine<8><<<resident_grid(k_combine<8>, total4, g_combine_occ[1]), kRedThreads, 0, st>>>(
-          o4, x4, xs, y4, ys4, Kc, cf, cscale, total4);
-    else if (Kc <= 16)
-      k_combine<16><<<resident_grid(k_combine<16>, total4, g_combine_occ[2]), kRedThreads, 0, st>>>(
-          o4, x4, xs, y4, ys4, Kc, cf, cscale, total4);
-    else
-      k_combine<32><<<resident_grid(k_combine<32>, total4, g_combine_occ[3]), kRedThreads, 0, st>>>(
-          o4, x4, xs, y4, ys4, Kc, cf, cscale, total4);
-    const cudaError_t e = cudaGetLastError();
+    const double* cg = coef2 ? coef2 + k0 : nullptr;
+#define RPM_COMBINE(KM, SLOT)                                                                  \
+  launch_pdl(k_combine<KM, NX>,                                                                \
+             dim3(resident_grid(k_combine<KM, NX>, total4, g_combine_occ[NX - 1][SLOT])),      \
+             kRedThreads, 0, st, o4, p4, x4, z4, xs, y4, ys4, Kc, cf, cg, cscale, total4)
+    const cudaError_t e = Kc <= 2    ? RPM_COMBINE(2, 0)
+                          : Kc <= 8  ? RPM_COMBINE(8, 1)
+                          : Kc <= 16 ? RPM_COMBINE(16, 2)
+                                     : RPM_COMBINE(32, 3);
+#undef RPM_COMBINE
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t launch_combine(float* out, const float* x, float xscale, const float* Y,
+                           long long ystride, int K, const double* coef, float cscale,
+                           long long n, cudaStream_t st) {
+  return combine_k<1>(out, nullptr, x, nullptr, xscale, Y, ystride, K, coef, nullptr, cscale, n, st);
+}
+
+cudaError_t launch_combine2(float* out, float* out2, const float* Y, long long ystride, int K,
+                            const double* coef, const double* coef2, float cscale, long long n,
+                            cudaStream_t st) {
+  return combine_k<2>(out, out2, out, out2, 1.f, Y, ystride, K, coef, coef2, cscale, n, st);
 }
 
 int combine_launches(int K) { return K <= 32 ? 1 : (K + 31) / 32; }
@@ -452,6 +538,7 @@ cudaError_t launch_stress(const GridDev& g, const float* eps, float* sig, double
 // out = a x + b y (y nullable; out may alias x or y)
 __global__ void __launch_bounds__(kRedThreads) k_axpby(float4* out, float a, const float4* x,
                                                        float b, const float4* y, long long total4) {
+  grid_dependency_wait();
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total4;
        q += (long long)gridDim.x * blockDim.x) {
     const float4 u = x[q];
@@ -460,6 +547,7 @@ __global__ void __launch_bounds__(kRedThreads) k_axpby(float4* out, float a, con
       const float4 v = y[q];
       r = make_float4(fmaf(b, v.x, r.x), fmaf(b, v.y, r.y), fmaf(b, v.z, r.z), fmaf(b, v.w, r.w));
     }
+    allow_dependent_launch();
     out[q] = r;
   }
 }
@@ -467,10 +555,32 @@ __global__ void __launch_bounds__(kRedThreads) k_axpby(float4* out, float a, con
 cudaError_t launch_axpby(float* out, float a, const float* x, float b, const float* y, long long n,
                          cudaStream_t st) {
   const long long total4 = 6 * (n / 4);
-  k_axpby<<<stream_blocks(total4), kRedThreads, 0, st>>>(
-      reinterpret_cast<float4*>(out), a, reinterpret_cast<const float4*>(x), b,
-      reinterpret_cast<const float4*>(y), total4);
-  return cudaGetLastError();
+  return launch_pdl(k_axpby, dim3(stream_blocks(total4)), kRedThreads, 0, st,
+                    reinterpret_cast<float4*>(out), a, reinterpret_cast<const float4*>(x), b,
+                    reinterpret_cast<const float4*>(y), total4);
+}
+
+// d0 = a - b, d1 = b - c (five field sweeps for the two differences)
+__global__ void __launch_bounds__(kRedThreads) k_diff2(float4* d0, float4* d1, const float4* a,
+                                                       const float4* b, const float4* c,
+                                                       long long total4) {
+  grid_dependency_wait();
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total4;
+       q += (long long)gridDim.x * blockDim.x) {
+    const float4 u = a[q], v = b[q], w = c[q];
+    allow_dependent_launch();
+    d0[q] = make_float4(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
+    d1[q] = make_float4(v.x - w.x, v.y - w.y, v.z - w.z, v.w - w.w);
+  }
+}
+
+cudaError_t launch_diff2(float* d0, float* d1, const float* a, const float* b, const float* c,
+                         long long n, cudaStream_t st) {
+  const long long total4 = 6 * (n / 4);
+  return launch_pdl(k_diff2, dim3(stream_blocks(total4)), kRedThreads, 0, st,
+                    reinterpret_cast<float4*>(d0), reinterpret_cast<float4*>(d1),
+                    reinterpret_cast<const float4*>(a), reinterpret_cast<const float4*>(b),
+                    reinterpret_cast<const float4*>(c), total4);
 }
 
 // eps_next = (C + C0)^-1 : (s_a + C0 : eps_b), Algorithm 3, per voxel; the

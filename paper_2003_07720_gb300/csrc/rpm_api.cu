@@ -73,7 +73,8 @@ struct rpm_ctx {
   double* partials = nullptr;
   int nblk = 0;
   double* dsmall = nullptr;
-  double* hsmall = nullptr;          // pinned host mirror
+  double* hsmall = nullptr;          // pinned host mirror; the sequence word follows it
+  unsigned long long seq = 0;        // reads asked of the device so far (see HostRead)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   size_t bytes = 0;
   std::string err;
@@ -321,21 +322,36 @@ struct Ops {
     done(m);
     return ok;
   }
-  // sums[0..K] <- dots of x against Y (see launch_dots)
-  // sums[0..K] <- dots (see launch_dots); with M, also the Newton step into c
-  // and the residual.  K <= 32 on grids up to ~100^3: one fused launch (the
-  // last block's serial tail costs more than two launches beyond that)
+  // K <= 32 on grids up to ~100^3: one fused launch (the last block's serial
+  // tail costs more than two launches beyond that)
+  bool fused(int K) const { return K <= 32 && c->nblk <= kFusedMaxBlocks; }
+  unsigned long long* seq_word() { return reinterpret_cast<unsigned long long*>(c->hsmall + kSmall); }
+  // sums[0..K] <- dots of x against Y (see launch_dots); with M, also the Newton
+  // step into c and the residual.  A non-null x2 (fused(K) only) adds the sums
+  // of x2 after them.  Read: a fused reduction leaves sums (and residual) in
+  // the host mirror itself, and `fetch` waits for it; `more` promises another
+  // one, so that one wait serves several.
+  enum Read { kNone, kMore, kRead };
   bool dots(const float* x, const float* xm, const float* Y, int K, double* sums,
             const double* M = nullptr, double* cN = nullptr, double* res = nullptr,
-            double inv_norm = 0.0) {
+            double inv_norm = 0.0, Read read = kNone, const float* x2 = nullptr) {
     const size_t m = mark(1);
-    c->proj_bytes += (double)(K + 1 + (xm ? 1 : 0)) * (double)c->fsz * 4.0;
+    c->proj_bytes += (double)(K + 1 + (xm ? 1 : 0) + (x2 ? 1 : 0)) * (double)c->fsz * 4.0;
     bool ok;
-    if (K <= 32 && c->nblk <= kFusedMaxBlocks) {
+    if (fused(K)) {
       c->launches += 1;
-      ok = ck(c, launch_dots_fused(x, xm, Y, (long long)c->fst, K, c->n, c->partials, c->nblk,
+      HostRead h{};
+      if (read != kNone) {
+        h.sums = c->hsmall + (sums - c->dsmall);
+        h.res = res ? c->hsmall + (res - c->dsmall) : nullptr;
+        if (read == kRead) {
+          h.seq = seq_word();
+          h.value = ++c->seq;
+        }
+      }
+      ok = ck(c, launch_dots_fused(x, x2, xm, Y, (long long)c->fst, K, c->n, c->partials, c->nblk,
                                    sums, reinterpret_cast<unsigned int*>(c->dsmall + kTicket), M,
-                                   cN, res, inv_norm, c->st),
+                                   cN, res, inv_norm, h, c->st),
               "dots");
     } else {
       c->launches += 1 + dots_launches(K) + (M ? 1 : 0);
@@ -347,6 +363,25 @@ struct Ops {
     done(m);
     return ok;
   }
+  // The host mirror's [off, off + count) holds the device's values: left there
+  // by a fused dots(K, ..., kRead), else copied.  The wait polls the sequence
+  // word; now and then it asks the stream, whose error or end ends the wait.
+  bool fetch(int K, int off, int count) {
+    if (!fused(K)) return read_small(off, count);
+    const unsigned long long want = c->seq;
+    for (unsigned spins = 1;; ++spins) {
+      if (__atomic_load_n(seq_word(), __ATOMIC_ACQUIRE) >= want) return true;
+      if (spins % 64 == 0) std::this_thread::yield();
+      if (spins % 16384 == 0) {
+        const cudaError_t e = cudaStreamQuery(c->st);
+        if (e == cudaErrorNotReady) continue;
+        if (!ck(c, e, "sync")) return false;
+        if (__atomic_load_n(seq_word(), __ATOMIC_ACQUIRE) >= want) return true;
+        c->err = "a reduction's results did not arrive";
+        return false;
+      }
+    }
+  }
   bool combine(float* out, const float* x, float xs, const float* Y, int K, const double* coef,
                float cscale) {
     const size_t m = mark(1);
@@ -355,6 +390,17 @@ struct Ops {
     const bool ok =
         ck(c, launch_combine(out, x, xs, Y, (long long)c->fst, K, coef, cscale, c->n, c->st),
            "combine");
+    done(m);
+    return ok;
+  }
+  // out += cscale Y coef for two fields, each basis vector read once
+  bool combine2(float* a, float* b, const float* Y, int K, const double* ca, const double* cb,
+                float cscale) {
+    const size_t m = mark(1);
+    c->launches += combine_launches(K);
+    c->proj_bytes += (double)(K + 4) * (double)c->fsz * 4.0;
+    const bool ok =
+        ck(c, launch_combine2(a, b, Y, (long long)c->fst, K, ca, cb, cscale, c->n, c->st), "combine");
     done(m);
     return ok;
   }
@@ -594,11 +640,12 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
     rpm_destroy(c);
     return e == cudaErrorMemoryAllocation ? RPM_ERR_OOM : RPM_ERR_CUDA;
   }
-  if (cudaMallocHost((void**)&c->hsmall, kSmall * 8) != cudaSuccess ||
+  if (cudaMallocHost((void**)&c->hsmall, (kSmall + 8) * 8) != cudaSuccess ||
       cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess) {
     rpm_destroy(c);
     return RPM_ERR_CUDA;
   }
+  std::memset(c->hsmall, 0, (kSmall + 8) * 8);
   char* t = c->tables;
   auto put = [&](size_t o2, const void* src, size_t b) {
     return cudaMemcpyAsync(t + o2, src, b, cudaMemcpyHostToDevice, c->st);
@@ -818,10 +865,10 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
   // all the next step needs)
   auto eval = [&](double& r, bool read = true) -> bool {
     if (!ops.dots(xi[cur], eps_cur, c->Z, c->p, ds + kSums, ds + kM, ds + kC, ds + kRes,
-                  inv_norm))
+                  inv_norm, read ? Ops::kRead : Ops::kNone))
       return false;
     if (!read) return true;
-    if (!ops.read_small(kRes, 1)) return false;
+    if (!ops.fetch(c->p, kRes, 1)) return false;
     r = hs[kRes];
     return true;
   };
@@ -832,35 +879,56 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
     const int prev = (cur + 2) % 3, prev2 = (cur + 1) % 3;
     double* one = ds + kSums;   // scratch sums
     // D0 = xi^nu - xi^(nu-1), D1 = xi^(nu-1) - xi^(nu-2)
-    if (!ck(c, (++c->launches, launch_axpby)(D[0], 1.f, xi[cur], -1.f, xi[prev], c->n, c->st), "axpby") ||
-        !ck(c, (++c->launches, launch_axpby)(D[1], 1.f, xi[prev], -1.f, xi[prev2], c->n, c->st), "axpby"))
+    if (!ck(c, (++c->launches, launch_diff2)(D[0], D[1], xi[cur], xi[prev], xi[prev2], c->n, c->st),
+            "differences"))
       return false;
-    // Q-projection (classical Gram-Schmidt, twice)
-    for (int pass = 0; pass < 2 && c->p > 0; ++pass)
+    // Q-projection (classical Gram-Schmidt, twice); on the fused sizes of both
+    // differences at once (96^3, p = 8: a growth reads the basis 8 times, not 12)
+    for (int pass = 0; pass < 2 && c->p > 0; ++pass) {
+      if (ops.fused(c->p)) {
+        if (!ops.dots(D[0], nullptr, c->Z, c->p, one, nullptr, nullptr, nullptr, 0.0, Ops::kNone, D[1]) ||
+            !ops.combine2(D[0], D[1], c->Z, c->p, one + 1, one + c->p + 2, -1.f))
+          return false;
+        continue;
+      }
       for (int k = 0; k < 2; ++k) {
         if (!ops.dots(D[k], nullptr, c->Z, c->p, one)) return false;
         if (!ops.combine(D[k], D[k], 1.f, c->Z, c->p, one + 1, -1.f)) return false;
       }
-    // QR of [D0, D1]
-    if (!ops.dots(D[1], nullptr, D[0], 1, ds + kSums)) return false;   // |D1|^2, <D1,D0>
-    if (!ops.read_small(kSums, 2)) return false;
-    const double n11 = hs[kSums], d10 = hs[kSums + 1];
-    if (!ops.dots(D[0], nullptr, nullptr, 0, ds + kSums)) return false;
-    if (!ops.read_small(kSums, 1)) return false;
-    const double T11 = std::sqrt(std::max(hs[kSums], 0.0));
+    }
+    // QR of [D0, D1]: |D0|^2, <D0, D1>, and |xi|^2 for the noise test
+    double d00, d10, xx;
+    if (ops.fused(1)) {
+      if (!ops.dots(D[0], nullptr, D[1], 1, ds + kSums, nullptr, nullptr, nullptr, 0.0, Ops::kRead,
+                    xi[cur]) ||
+          !ops.fetch(1, kSums, 4))
+        return false;
+      d00 = hs[kSums];
+      d10 = hs[kSums + 1];
+      xx = hs[kSums + 2];
+    } else {
+      if (!ops.dots(D[0], nullptr, D[1], 1, ds + kSums) || !ops.read_small(kSums, 2)) return false;
+      d00 = hs[kSums];
+      d10 = hs[kSums + 1];
+      if (!ops.dots(xi[cur], nullptr, nullptr, 0, ds + kSums) || !ops.read_small(kSums, 1))
+        return false;
+      xx = hs[kSums];
+    }
+    const double T11 = std::sqrt(std::max(d00, 0.0));
     if (!(T11 > 0) || !std::isfinite(T11)) return true;
-    if (!ops.dots(xi[cur], nullptr, nullptr, 0, ds + kSums)) return false;
-    if (!ops.read_small(kSums, 1)) return false;
-    if (T11 < kGrowNoise * std::sqrt(std::max(hs[kSums], 0.0))) {   // rounding noise:
+    if (T11 < kGrowNoise * std::sqrt(std::max(xx, 0.0))) {   // rounding noise:
       want_rebase = true;   // re-centre, then grow from differences in the new coordinates
       return true;
     }
     const double T12 = d10 / T11;
-    (void)n11;
     if (!ck(c, (++c->launches, launch_axpby)(D[1], 1.f, D[1], (float)(-T12 / T11), D[0], c->n, c->st), "axpby"))
       return false;
-    if (!ops.dots(D[1], nullptr, nullptr, 0, ds + kSums)) return false;
-    if (!ops.read_small(kSums, 1)) return false;
+    auto norm2 = [&](const float* u) {   // |u|^2 into hs[kSums]
+      return ops.dots(u, nullptr, nullptr, 0, ds + kSums, nullptr, nullptr, nullptr, 0.0,
+                      Ops::kRead) &&
+             ops.fetch(0, kSums, 1);
+    };
+    if (!norm2(D[1])) return false;
     const double T22 = std::sqrt(std::max(hs[kSums], 0.0));
     int ncand = 1;
     double Tn[2] = {T11, T22};
@@ -876,8 +944,7 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
         if (!ops.dots(u, nullptr, c->Z, c->p, one)) return false;
         if (!ops.combine(u, u, 1.f, c->Z, c->p, one + 1, -1.f)) return false;
       }
-      if (!ops.dots(u, nullptr, nullptr, 0, ds + kSums)) return false;
-      if (!ops.read_small(kSums, 1)) return false;
+      if (!norm2(u)) return false;
       const double nu_ = std::sqrt(std::max(hs[kSums], 0.0));
       if (!(nu_ > 1e-10)) continue;
       float* zp = c->Z + (size_t)c->p * F;
@@ -893,13 +960,33 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
     std::vector<double> Hn((size_t)p * p, 0.0);
     for (int i = 0; i < p_old; ++i)
       for (int j = 0; j < p_old; ++j) Hn[(size_t)i * p + j] = c->H[(size_t)i * p_old + j];
+    // (rows and columns q of all new vectors are queued before one wait where
+    // the sums have room: 2 (p - p_old) (p + 1) of them)
+    const bool queue = ops.fused(p) && 4 * (p + 1) <= kC - kSums;
     for (int q = p_old; q < p; ++q) {
-      if (!ops.dots(c->W + (size_t)q * F, nullptr, c->Z, p, ds + kSums)) return false;
-      if (!ops.read_small(kSums, p + 1)) return false;
-      for (int i = 0; i < p; ++i) Hn[(size_t)i * p + q] = hs[kSums + 1 + i];
-      if (!ops.dots(c->Z + (size_t)q * F, nullptr, c->W, p, ds + kSums)) return false;
-      if (!ops.read_small(kSums, p + 1)) return false;
-      for (int j = 0; j < p; ++j) Hn[(size_t)q * p + j] = hs[kSums + 1 + j];
+      const int o = queue ? kSums + 2 * (q - p_old) * (p + 1) : kSums, o2 = queue ? o + p + 1 : o;
+      if (!ops.dots(c->W + (size_t)q * F, nullptr, c->Z, p, ds + o, nullptr, nullptr, nullptr, 0.0,
+                    queue ? Ops::kMore : Ops::kRead))
+        return false;
+      if (!queue) {
+        if (!ops.fetch(p, kSums, p + 1)) return false;
+        for (int i = 0; i < p; ++i) Hn[(size_t)i * p + q] = hs[kSums + 1 + i];
+      }
+      if (!ops.dots(c->Z + (size_t)q * F, nullptr, c->W, p, ds + o2, nullptr, nullptr, nullptr, 0.0,
+                    queue && q + 1 < p ? Ops::kMore : Ops::kRead))
+        return false;
+      if (!queue) {
+        if (!ops.fetch(p, kSums, p + 1)) return false;
+        for (int j = 0; j < p; ++j) Hn[(size_t)q * p + j] = hs[kSums + 1 + j];
+      }
+    }
+    if (queue) {
+      if (!ops.fetch(p, kSums, 0)) return false;
+      for (int q = p_old; q < p; ++q) {
+        const double* h = hs + kSums + 2 * (q - p_old) * (p + 1);
+        for (int i = 0; i < p; ++i) Hn[(size_t)i * p + q] = h[1 + i];
+        for (int j = 0; j < p; ++j) Hn[(size_t)q * p + j] = h[p + 2 + j];
+      }
     }
     c->H = Hn;
     std::vector<double> A((size_t)p * p);

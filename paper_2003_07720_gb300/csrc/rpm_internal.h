@@ -121,15 +121,34 @@ cudaError_t launch_dots(const float* x, const float* x_minus /*nullable*/, const
                         cudaStream_t st);
 cudaError_t launch_reduce_partials(const double* partials, int nblk, int m, double* out,
                                    cudaStream_t st);
+// Where a fused reduction leaves its results for the host (pinned memory the
+// device can write): the sums, the residual (when M is given), and last, when
+// seq is set, the sequence number the host waits for.  All null: nothing.
+struct HostRead {
+  double* sums;
+  double* res;
+  unsigned long long* seq;
+  unsigned long long value;
+};
 // launch_dots + launch_reduce_partials (+ launch_newton when M is given, p = K)
 // in one launch, for K <= 32; ticket: a device counter that is zero on entry.
-cudaError_t launch_dots_fused(const float* x, const float* x_minus, const float* Y,
-                              long long ystride, int K, long long n, double* partials, int nblk,
-                              double* sums, unsigned int* ticket, const double* M, double* c,
-                              double* res_out, double inv_norm, cudaStream_t st);
+// A non-null x2 (then no x_minus, no M) adds the K + 1 sums of a second field
+// after the first's.
+cudaError_t launch_dots_fused(const float* x, const float* x2, const float* x_minus,
+                              const float* Y, long long ystride, int K, long long n,
+                              double* partials, int nblk, double* sums, unsigned int* ticket,
+                              const double* M, double* c, double* res_out, double inv_norm,
+                              const HostRead& host, cudaStream_t st);
 cudaError_t launch_combine(float* out, const float* x, float xscale, const float* Y,
                            long long ystride, int K, const double* coef, float cscale,
                            long long n, cudaStream_t st);
+// out += cscale * sum_j coef[j] Y_j and the same for out2 with coef2
+cudaError_t launch_combine2(float* out, float* out2, const float* Y, long long ystride, int K,
+                            const double* coef, const double* coef2, float cscale, long long n,
+                            cudaStream_t st);
+// d0 = a - b, d1 = b - c
+cudaError_t launch_diff2(float* d0, float* d1, const float* a, const float* b, const float* c,
+                         long long n, cudaStream_t st);
 cudaError_t launch_axpby(float* out, float a, const float* x, float b, const float* y, long long n,
                          cudaStream_t st);
 cudaError_t launch_stress(const GridDev& g, const float* eps, float* sig /*nullable*/,

@@ -60,3 +60,26 @@ def test_paired_map_matches_oracle(nz, n, pencil):
 @pytest.mark.parametrize("pencil", [0, 2])
 def test_five_passes_match_oracle(shape, pencil):
     _check(shape, pencil, 2)
+
+
+@pytest.mark.parametrize("n,contrast,p_max", [(16, 1e3, 44), (16, 10.0, 12), (48, 10.0, 6)])
+def test_reductions_of_every_basis_size(n, contrast, p_max):
+    """RPM solves whose reductions take each form of the dot kernels: two and
+    more float4 a thread, both differences of a growth at once, results polled
+    by the host, and above 32 vectors the chunked launches (16^3 at contrast
+    1e3 fills its 44).  The stopping test leaves at most some 100 x 1e-6."""
+    from paper_2003_07720_gb300 import rpm
+    phase = ms.random_two_phase((n, n, n), 3, 0.3) if n < 48 else ms.centred_sphere(n)
+    (l1, m1), (l2, m2) = ms.lame(1.0, 0.3), ms.lame(contrast, 0.3)
+    l0, m0 = ms.lame(0.5 * (1.0 + contrast), 0.3)
+    cell = ms.Cell(phase=phase, lam=np.array([l1, l2]), mu=np.array([m1, m2]), lam0=l0, mu0=m0)
+    E = ms.unit_strain(0)
+    ref = o.rpm_solve(o.Problem.from_cell(cell), E,
+                      o.Options(tol=1e-8, p_max=p_max, n_max=5, max_iters=3000))
+    opts = rpm.rpm_default_options(tol=1e-6, p_max=p_max, n_max=5, max_iters=3000)
+    with rpm.Context(cell, opts) as ctx:
+        st, info = ctx.solve(E)
+    assert ref.converged and info["converged"]
+    assert p_max < 44 or info["basis_size"] > 32
+    got = np.array(info["mean_stress"])
+    assert np.max(np.abs(got - ref.mean_stress)) < 1e-4 * np.max(np.abs(ref.mean_stress))
