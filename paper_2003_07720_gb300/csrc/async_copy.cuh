@@ -108,6 +108,11 @@ __device__ __forceinline__ void async_copy_wait() {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// all of them but those of the last committed group
+__device__ __forceinline__ void async_copy_wait_but_last() {
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
+
 // Orders this thread's ordinary shared-memory accesses before later accesses
 // of the asynchronous copy engine (and the reverse).
 __device__ __forceinline__ void fence_async_smem() {

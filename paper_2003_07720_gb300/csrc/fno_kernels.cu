@@ -261,6 +261,14 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi) {
   return (uint32_t)bf16_bits(lo) | ((uint32_t)bf16_bits(hi) << 16);
 }
 
+// A table image from global to shared memory by asynchronous copies (whole
+// 16-byte units), one commit group.
+__device__ __forceinline__ void copy_table(void* dst, const uint4* src, size_t bytes, int tid) {
+  for (int i = tid; i < (int)(bytes / 16); i += kThreads)
+    rpm::async_copy16(reinterpret_cast<uint4*>(dst) + i, src + i);
+  rpm::async_copy_commit();
+}
+
 __host__ __device__ inline int round_up(int v, int q) { return (v + q - 1) / q * q; }
 
 struct XyTc {
@@ -273,6 +281,10 @@ struct XyTc {
     MY = 2 * KPY;
     MPY = round_up(m, 8);        // y-stage output columns (kx)
     KPB = 2 * N + 8;             // bf16 row stride of Ay and XT
+  }
+  // the DFT operands BTx and Ay, side by side in shared memory
+  __host__ __device__ size_t table_bytes(int N) const {
+    return (size_t)2 * ((size_t)NX2 * NPB + (size_t)MY * KPB);
   }
   __host__ __device__ size_t bytes(int N) const {
     return (size_t)2 * ((size_t)G * N * NPB + (size_t)NX2 * NPB + (size_t)MY * KPB +
@@ -288,7 +300,7 @@ size_t xy_tc_smem(int N, int m) { return XyTc(N, m).bytes(N); }
 template <int N>
 __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restrict__ src,
                                                         float2* __restrict__ dst,
-                                                        const float2* __restrict__ twg, int m) {
+                                                        const uint4* __restrict__ tab, int m) {
   extern __shared__ float4 smem4[];
   const XyTc c(N, m);
   const int ncol = 2 * m * m;
@@ -303,35 +315,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_fwd_tc(const float* __restri
   const long long NN = (long long)N * N;
   float2* d = dst + ((long long)b * N + z) * ncol * W;
   allow_dependent_launch();
-  for (int i = tid; i < c.NX2 * N; i += kThreads) {
-    const int r = i / N, x = i - r * N, kx = r >> 1;
-    float v = 0.f;
-    if (kx < m) {
-      const float2 t = twg[(kx * x) % N];
-      v = (r & 1) ? t.y : t.x;
-    }
-    BTx[r * c.NPB + x] = bf16_bits(v);
-  }
-  for (int i = tid; i < c.KPY * N; i += kThreads) {
-    const int r = i / N, y = i - r * N;
-    float tr = 0.f, ti = 0.f;
-    if (r < 2 * m) {
-      const float2 t = twg[(kfreq(r, m, N) * y) % N];
-      tr = t.x;
-      ti = t.y;
-    }
-    uint16_t* re = Ay + (size_t)r * c.KPB + 2 * y;
-    uint16_t* im = Ay + (size_t)(c.KPY + r) * c.KPB + 2 * y;
-    re[0] = bf16_bits(tr);
-    re[1] = bf16_bits(-ti);
-    im[0] = bf16_bits(ti);
-    im[1] = bf16_bits(tr);
-  }
+  copy_table(BTx, tab, c.table_bytes(N), tid);
   const int nmt = N / 16, nnt = c.NX2 / 8;          // x-stage tiles per channel
   const int ymt = c.MY / 16, ynt = c.MPY / 8;        // y-stage tiles per channel
   grid_dependency_wait();
   for (int c0 = blockIdx.z * per; c0 < (int)(blockIdx.z + 1) * per; c0 += c.G) {
-    __syncthreads();   // tables written; the previous group's readers are done
+    rpm::async_copy_wait();
+    __syncthreads();   // tables in place; the previous group's readers are done
     for (int i = tid; i < c.G * N * N / 4; i += kThreads) {
       const int g = i / (N * N / 4), r = i - g * (N * N / 4);
       const int y = r / (N / 4), x = 4 * (r - y * (N / 4));
@@ -506,6 +496,10 @@ struct SpecTc {
     GB = B < 16 ? B : 16;
     stage = B <= 2;
   }
+  // the DFT operands Az and Ainv, side by side in shared memory
+  __host__ __device__ size_t table_bytes() const {
+    return (size_t)2 * ((size_t)MZ * KZB + (size_t)2 * N * KIB);
+  }
   __host__ __device__ size_t bytes() const {
     return (size_t)2 * ((size_t)MZ * KZB + (size_t)2 * N * KIB + (size_t)W * KZB +
                         (size_t)KPZ * GB * MB + (size_t)GB * W * KIB) +
@@ -525,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
                                                           const float2* __restrict__ R,
                                                           float2* __restrict__ Vs,
                                                           float2* __restrict__ Bz,
-                                                          const float2* __restrict__ twg, int m,
+                                                          const uint4* __restrict__ tab, int m,
                                                           int B) {
   extern __shared__ float4 smem4[];
   const SpecTc<N> c(m, B);
@@ -541,26 +535,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
   float* Di = Dz + c.MZ * 16;                                            // [2N][16]
   const float2* Rc = R + (long long)col * m2 * W * W;
   allow_dependent_launch();
+  copy_table(Az, tab, c.table_bytes(), tid);
   if (c.stage) {   // (the parameters are not written by the kernels of a pass)
     for (int i = tid; i < m2 * W * W / 2; i += kThreads)
       rpm::async_copy16(Rs + 2 * i, Rc + 2 * i);
-    rpm::async_copy_commit();
     Rc = Rs;
   }
-  for (int i = tid; i < c.KPZ * N; i += kThreads) {
-    const int r = i / N, z = i - r * N;
-    float tr = 0.f, ti = 0.f;
-    if (r < m2) {
-      const float2 t = twg[(kfreq(r, m, N) * z) % N];
-      tr = t.x;
-      ti = t.y;
-    }
-    *reinterpret_cast<uint32_t*>(Az + (size_t)r * c.KZB + 2 * z) = bf16x2_bits(tr, -ti);
-    *reinterpret_cast<uint32_t*>(Az + (size_t)(c.KPZ + r) * c.KZB + 2 * z) = bf16x2_bits(ti, tr);
-    // inverse: row z (re) (Tr, Ti), row N + z (im) (-Ti, Tr) at column pair r
-    *reinterpret_cast<uint32_t*>(Ainv + (size_t)z * c.KIB + 2 * r) = bf16x2_bits(tr, ti);
-    *reinterpret_cast<uint32_t*>(Ainv + (size_t)(N + z) * c.KIB + 2 * r) = bf16x2_bits(-ti, tr);
-  }
+  rpm::async_copy_commit();   // (empty without staged weights)
   // columns of BTU past the kept kz stay zero
   for (int i = tid; i < c.GB * W * (c.KPZ - m2); i += kThreads) {
     const int row = i / (c.KPZ - m2), k = m2 + i % (c.KPZ - m2);
@@ -572,7 +553,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
     const int gb = min(16, B - g0);
     for (int bi = 0; bi < gb; ++bi) {
       const int b = g0 + bi;
-      __syncthreads();   // tables written; BTa / Dz readers of the previous sample are done
+      rpm::async_copy_wait_but_last();
+      __syncthreads();   // tables in place; BTa / Dz readers of the previous sample are done
       for (int i = tid; i < N * W; i += kThreads) {
         const int z = i / W, cc = i - z * W;
         const float2 a = A2[((long long)b * N + z) * ncol * W + col * W + cc];
@@ -606,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_spec_fwd_tc(const float2* __res
             bf16x2_bits(re, im);
       }
     }
-    if (c.stage) rpm::async_copy_wait();
+    rpm::async_copy_wait();
     __syncthreads();
     // channel mixing per kz: U[b][(o, re/im)] = sum_(i, re/im) V[b][(i, re/im)] Rr[kz]
     for (int tile = warp; tile < m2 * 4; tile += kThreads / 32) {
@@ -912,6 +894,9 @@ struct InvTc {
     K2P = K2 + 8;
     UP = N + 4;
   }
+  // the DFT operands: A1 of one block's rows, BT2
+  __host__ __device__ size_t a1_bytes() const { return (size_t)2 * M1 * K1P; }
+  __host__ __device__ size_t bt2_bytes(int N) const { return (size_t)2 * N * K2P; }
   __host__ __device__ size_t bytes(int N) const {
     return (size_t)2 * ((size_t)N1 * K1P + (size_t)M1 * K1P + (size_t)YC * W * K2P +
                         (size_t)N * K2P) +
@@ -922,12 +907,13 @@ size_t inv_tc_smem(int N, int m, int YC) { return InvTc(N, m, YC).bytes(N); }
 
 template <bool BWD, int N>
 __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restrict__ Bz,
-                                                        const float2* __restrict__ twg,
+                                                        const uint4* __restrict__ tabA,
+                                                        const uint4* __restrict__ tabB,
                                                         const float* __restrict__ layer,
                                                         const float* __restrict__ vin,
                                                         float* __restrict__ zsave,
                                                         float* __restrict__ vout, int m,
-                                                        int YC, int last, float inv_n3) {
+                                                        int YC, int last) {
   extern __shared__ float4 smem4[];
   const InvTc c(N, m, YC);
   const int ncol = 2 * m * m, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -944,31 +930,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
   const int pad1 = c.K1 - 4 * m;
   for (int i = tid; i < c.N1 * pad1; i += kThreads)
     BT1[(size_t)(i / pad1) * c.K1P + 4 * m + i % pad1] = 0;
-  for (int i = tid; i < YC * (c.K1 / 2); i += kThreads) {
-    const int yy = i / (c.K1 / 2), kyi = i - yy * (c.K1 / 2);
-    float tr = 0.f, ti = 0.f;
-    if (kyi < 2 * m) {
-      const float2 t = twg[(kfreq(kyi, m, N) * (y0 + yy)) % N];
-      tr = t.x;
-      ti = t.y;
-    }
-    *reinterpret_cast<uint32_t*>(A1 + (size_t)yy * c.K1P + 2 * kyi) = bf16x2_bits(tr, ti);
-    *reinterpret_cast<uint32_t*>(A1 + (size_t)(YC + yy) * c.K1P + 2 * kyi) = bf16x2_bits(-ti, tr);
-  }
+  copy_table(A1, tabA + (size_t)blockIdx.x * (c.a1_bytes() / 16), c.a1_bytes(), tid);
+  copy_table(BT2, tabB, c.bt2_bytes(N), tid);
   const int pad2 = c.K2 - 2 * m;
   for (int i = tid; i < YC * W * pad2; i += kThreads)
     A2[(size_t)(i / pad2) * c.K2P + 2 * m + i % pad2] = 0;
-  for (int i = tid; i < N * (c.K2 / 2); i += kThreads) {
-    const int x = i / (c.K2 / 2), kx = i - x * (c.K2 / 2);
-    float wr = 0.f, wi = 0.f;
-    if (kx < m) {
-      const float w = BWD ? 1.f : (kx == 0 ? inv_n3 : 2.f * inv_n3);
-      const float2 t = twg[(kx * x) % N];
-      wr = w * t.x;
-      wi = w * t.y;
-    }
-    *reinterpret_cast<uint32_t*>(BT2 + (size_t)x * c.K2P + 2 * kx) = bf16x2_bits(wr, wi);
-  }
   if (!BWD)
     for (int i = tid; i < kLayerHead; i += kThreads) Al[2 * i] = Al[2 * i + 1] = layer[i];
   grid_dependency_wait();
@@ -980,6 +946,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
     *reinterpret_cast<uint32_t*>(BT1 + (size_t)(kx * W + cc) * c.K1P + 2 * kyi) =
         bf16x2_bits(sv.x, sv.y);
   }
+  rpm::async_copy_wait();
   __syncthreads();
   const int nt1 = c.N1 / 8, mt1 = c.M1 / 16;
   for (int tile = warp; tile < mt1 * nt1; tile += kThreads / 32) {
@@ -1071,6 +1038,111 @@ __global__ void __launch_bounds__(kThreads, 2) k_inv_xy_tc(const float2* __restr
       }
     }
     __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The bfloat16 DFT operands of the three tensor-core kernels, laid out as they
+// sit in shared memory.  They depend on (N, m) alone: built once per network,
+// a block copies them instead of evaluating them (64^3 forward, one sample:
+// 163 -> 157 us).
+// ---------------------------------------------------------------------------
+template <int N>
+struct TcTables {
+  size_t xy, spec, a1, bt2f, bt2b, bytes;   // byte offsets of the images
+  __host__ __device__ TcTables(int m, int YC) {
+    const InvTc c(N, m, YC);
+    xy = 0;
+    spec = xy + XyTc(N, m).table_bytes(N);
+    a1 = spec + SpecTc<N>(m, 1).table_bytes();
+    bt2f = a1 + (size_t)(N / YC) * c.a1_bytes();
+    bt2b = bt2f + c.bt2_bytes(N);
+    bytes = bt2b + c.bt2_bytes(N);
+  }
+};
+
+template <int N>
+__global__ void __launch_bounds__(kThreads) k_tc_tables(const float2* __restrict__ twg, char* tab,
+                                                        int m, int YC, float inv_n3) {
+  const TcTables<N> t(m, YC);
+  const int tid = threadIdx.x;
+  {
+    const XyTc c(N, m);
+    uint16_t* BTx = reinterpret_cast<uint16_t*>(tab + t.xy);       // [NX2][NPB]
+    uint16_t* Ay = BTx + (size_t)c.NX2 * c.NPB;                     // [MY][KPB]
+    for (int i = tid; i < c.NX2 * N; i += kThreads) {
+      const int r = i / N, x = i - r * N, kx = r >> 1;
+      float v = 0.f;
+      if (kx < m) {
+        const float2 t = twg[(kx * x) % N];
+        v = (r & 1) ? t.y : t.x;
+      }
+      BTx[r * c.NPB + x] = bf16_bits(v);
+    }
+    for (int i = tid; i < c.KPY * N; i += kThreads) {
+      const int r = i / N, y = i - r * N;
+      float tr = 0.f, ti = 0.f;
+      if (r < 2 * m) {
+        const float2 t = twg[(kfreq(r, m, N) * y) % N];
+        tr = t.x;
+        ti = t.y;
+      }
+      uint16_t* re = Ay + (size_t)r * c.KPB + 2 * y;
+      uint16_t* im = Ay + (size_t)(c.KPY + r) * c.KPB + 2 * y;
+      re[0] = bf16_bits(tr);
+      re[1] = bf16_bits(-ti);
+      im[0] = bf16_bits(ti);
+      im[1] = bf16_bits(tr);
+    }
+  }
+  {
+    const SpecTc<N> c(m, 1);
+    const int m2 = c.m2;
+    uint16_t* Az = reinterpret_cast<uint16_t*>(tab + t.spec);      // [MZ][KZB]
+    uint16_t* Ainv = Az + (size_t)c.MZ * c.KZB;                     // [2N][KIB]
+    for (int i = tid; i < c.KPZ * N; i += kThreads) {
+      const int r = i / N, z = i - r * N;
+      float tr = 0.f, ti = 0.f;
+      if (r < m2) {
+        const float2 t = twg[(kfreq(r, m, N) * z) % N];
+        tr = t.x;
+        ti = t.y;
+      }
+      *reinterpret_cast<uint32_t*>(Az + (size_t)r * c.KZB + 2 * z) = bf16x2_bits(tr, -ti);
+      *reinterpret_cast<uint32_t*>(Az + (size_t)(c.KPZ + r) * c.KZB + 2 * z) = bf16x2_bits(ti, tr);
+      // inverse: row z (re) (Tr, Ti), row N + z (im) (-Ti, Tr) at column pair r
+      *reinterpret_cast<uint32_t*>(Ainv + (size_t)z * c.KIB + 2 * r) = bf16x2_bits(tr, ti);
+      *reinterpret_cast<uint32_t*>(Ainv + (size_t)(N + z) * c.KIB + 2 * r) = bf16x2_bits(-ti, tr);
+    }
+  }
+  const InvTc c(N, m, YC);
+  for (int y0 = 0; y0 < N; y0 += YC) {
+    uint16_t* A1 = reinterpret_cast<uint16_t*>(tab + t.a1 + (size_t)(y0 / YC) * c.a1_bytes());   // [M1][K1P]
+    for (int i = tid; i < YC * (c.K1 / 2); i += kThreads) {
+      const int yy = i / (c.K1 / 2), kyi = i - yy * (c.K1 / 2);
+      float tr = 0.f, ti = 0.f;
+      if (kyi < 2 * m) {
+        const float2 t = twg[(kfreq(kyi, m, N) * (y0 + yy)) % N];
+        tr = t.x;
+        ti = t.y;
+      }
+      *reinterpret_cast<uint32_t*>(A1 + (size_t)yy * c.K1P + 2 * kyi) = bf16x2_bits(tr, ti);
+      *reinterpret_cast<uint32_t*>(A1 + (size_t)(YC + yy) * c.K1P + 2 * kyi) = bf16x2_bits(-ti, tr);
+    }
+  }
+  for (int bwd = 0; bwd < 2; ++bwd) {
+    uint16_t* BT2 = reinterpret_cast<uint16_t*>(tab + (bwd ? t.bt2b : t.bt2f));   // [N][K2P]
+    for (int i = tid; i < N * (c.K2 / 2); i += kThreads) {
+      const int x = i / (c.K2 / 2), kx = i - x * (c.K2 / 2);
+      float wr = 0.f, wi = 0.f;
+      if (kx < m) {
+        const float w = bwd ? 1.f : (kx == 0 ? inv_n3 : 2.f * inv_n3);
+        const float2 t = twg[(kx * x) % N];
+        wr = w * t.x;
+        wi = w * t.y;
+      }
+      *reinterpret_cast<uint32_t*>(BT2 + (size_t)x * c.K2P + 2 * kx) = bf16x2_bits(wr, wi);
+    }
   }
 }
 
@@ -1535,6 +1607,7 @@ struct rpm_fno {
   float2* Bz = nullptr;
   float2* Vs = nullptr;       // per layer [ncol][Bmax][2m][W]
   float2* tw = nullptr;
+  char* tab = nullptr;        // bfloat16 DFT operands (TcTables) of a tensor-core network
   float* part = nullptr;
   double* extra = nullptr;
   float* Ed = nullptr;        // [Bmax][6]
@@ -1587,6 +1660,10 @@ bool stage_E(rpm_fno* f, int B, const float* E_dir) {
              "E");
 }
 
+const uint4* tc_table(const rpm_fno* f, size_t off) {
+  return reinterpret_cast<const uint4*>(f->tab + off);
+}
+
 // Truncated forward xy transform of B samples into f->A2: the BF16
 // tensor-core kernel when the network was created with RPM_FNO_BF16.
 #define RPM_FNO_TC_SIZES(X) X(32) X(48) X(64) X(96) X(128)
@@ -1595,15 +1672,15 @@ cudaError_t launch_xy_fwd(rpm_fno* f, const float* src, int B) {
   const int N = f->N, m = f->m;
   if (f->tc) {
     // channel groups over blocks until there are two blocks per SM (each block
-    // builds the twiddle tables, so not further): 64^3, one sample, 26.4 -> 11.5 us;
-    // 32^3, two samples, 19.4 -> 8.5 us
+    // builds the twiddle tables, so not further): 64^3, one sample, 26.4 -> 11.1 us;
+    // 32^3, two samples, 19.4 -> 7.9 us
     int nc = 1;
     while (nc < W / xy_group(N) && N * B * nc < 304) nc *= 2;
     switch (N) {
 #define RPM_CASE(NN)                                                                        \
   case NN:                                                                                  \
     return launch_pdl(k_xy_fwd_tc<NN>, dim3(N, B, nc), kThreads, xy_tc_smem(N, m), f->st, src,  \
-                      f->A2, (const float2*)f->tw, m);
+                      f->A2, tc_table(f, TcTables<NN>(m, f->YC).xy), m);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
@@ -1620,7 +1697,8 @@ cudaError_t launch_spec_fwd(rpm_fno* f, int B, const float2* R, float2* Vs) {
 #define RPM_CASE(NN)                                                                           \
   case NN:                                                                                     \
     return launch_pdl(k_spec_fwd_tc<NN>, dim3(f->ncol), kThreads, spec_tc_smem<NN>(m, B),      \
-                      f->st, (const float2*)f->A2, R, Vs, f->Bz, (const float2*)f->tw, m, B);
+                      f->st, (const float2*)f->A2, R, Vs, f->Bz,                                      \
+                      tc_table(f, TcTables<NN>(m, f->YC).spec), m, B);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
@@ -1641,8 +1719,10 @@ cudaError_t launch_inv_xy(rpm_fno* f, int B, const float* layer, const float* vi
 #define RPM_CASE(NN)                                                                     \
   case NN:                                                                               \
     return launch_pdl(k_inv_xy_tc<BWD, NN>, grid, kThreads, inv_tc_smem(N, m, f->YC), f->st, \
-                      (const float2*)f->Bz, (const float2*)f->tw, layer, vin, zsave, vout, m,  \
-                      f->YC, last, inv_n3);
+                      (const float2*)f->Bz, tc_table(f, TcTables<NN>(m, f->YC).a1),            \
+                      tc_table(f, BWD ? TcTables<NN>(m, f->YC).bt2b                            \
+                                      : TcTables<NN>(m, f->YC).bt2f),                          \
+                      layer, vin, zsave, vout, m, f->YC, last);
       RPM_FNO_TC_SIZES(RPM_CASE)
 #undef RPM_CASE
     }
@@ -1739,6 +1819,26 @@ bool set_tc_smem() {
   return true;
 }
 
+// The DFT operand images of a tensor-core network (after f->tw is uploaded).
+// (N % 16 == 0 sides without a tensor-core kernel run the float32 kernels.)
+cudaError_t make_tc_tables(rpm_fno* f) {
+  switch (f->N) {
+#define RPM_CASE(NN)                                                                          \
+  case NN: {                                                                                  \
+    const TcTables<NN> t(f->m, f->YC);                                                        \
+    cudaError_t e = cudaMalloc((void**)&f->tab, t.bytes);                                     \
+    if (e != cudaSuccess) return e;                                                           \
+    f->bytes += t.bytes;                                                                      \
+    if ((e = cudaMemsetAsync(f->tab, 0, t.bytes, f->st)) != cudaSuccess) return e;            \
+    k_tc_tables<NN><<<1, kThreads, 0, f->st>>>(f->tw, f->tab, f->m, f->YC, 1.f / (float)f->N3); \
+    return cudaGetLastError();                                                                \
+  }
+    RPM_FNO_TC_SIZES(RPM_CASE)
+#undef RPM_CASE
+    default: return cudaSuccess;
+  }
+}
+
 bool valid_batch(rpm_fno* f, int B) { return f && B >= 1 && B <= f->Bmax; }
 
 }  // namespace
@@ -1810,6 +1910,7 @@ rpm_status rpm_fno_create(const rpm_fno_config* cfg, void* cuda_stream, rpm_fno*
   if (smax > 227 * 1024 ||
       cudaMemcpyAsync(f->tw, tw.data(), N * sizeof(float2), cudaMemcpyHostToDevice, f->st) !=
           cudaSuccess ||
+      (f->tc && make_tc_tables(f) != cudaSuccess) ||
       cudaMemsetAsync(f->params, 0, P, f->st) != cudaSuccess ||
       cudaMemsetAsync(f->grads, 0, P, f->st) != cudaSuccess ||
       cudaMemsetAsync(f->adam1, 0, P, f->st) != cudaSuccess ||
@@ -2008,7 +2109,7 @@ void rpm_fno_destroy(rpm_fno* f) {
   if (!f) return;
   void* dev[] = {f->params, f->grads, f->adam1, f->adam2, f->acts, f->dvbuf,
                  f->A2,     f->Bz,    f->Vs,    f->tw,    f->part, f->extra,
-                 f->Ed,     f->feat1, f->out1,  f->eps0,  f->ftab};
+                 f->Ed,     f->feat1, f->out1,  f->eps0,  f->ftab, f->tab};
   for (void* p : dev)
     if (p) cudaFree(p);
   if (f->hE) cudaFreeHost(f->hE);
