@@ -1611,7 +1611,6 @@ struct rpm_fno {
   float* part = nullptr;
   double* extra = nullptr;
   float* Ed = nullptr;        // [Bmax][6]
-  float* hE = nullptr;        // pinned staging of E
   double* hloss = nullptr;    // pinned
   float* feat1 = nullptr;     // warm start: features and output of one sample
   float* out1 = nullptr;
@@ -1653,11 +1652,24 @@ cudaError_t set_smem(const void* k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// E of a batch travels as a kernel argument: the launch takes its own copy, so a
+// call may return, and the next one bring another E, before the stream gets here
+// (a staging buffer shared by the calls would be rewritten under a copy still
+// queued).  An ordinary launch: complete before any kernel of the pass starts.
+struct BatchE {
+  float e[RPM_FNO_MAX_BATCH * CE];
+};
+static_assert(sizeof(BatchE) <= 4000, "kernel argument space");
+
+__global__ void k_store_E(BatchE E, float* __restrict__ Ed, int count) {
+  for (int i = threadIdx.x; i < count; i += blockDim.x) Ed[i] = E.e[i];
+}
+
 bool stage_E(rpm_fno* f, int B, const float* E_dir) {
-  std::memcpy(f->hE, E_dir, sizeof(float) * CE * B);
-  return fck(f, cudaMemcpyAsync(f->Ed, f->hE, sizeof(float) * CE * B, cudaMemcpyHostToDevice,
-                                f->st),
-             "E");
+  BatchE E;
+  std::memcpy(E.e, E_dir, sizeof(float) * CE * B);
+  k_store_E<<<1, 128, 0, f->st>>>(E, f->Ed, CE * B);
+  return fck(f, cudaGetLastError(), "E");
 }
 
 const uint4* tc_table(const rpm_fno* f, size_t off) {
@@ -1891,8 +1903,7 @@ rpm_status rpm_fno_create(const rpm_fno_config* cfg, void* cuda_stream, rpm_fno*
       alloc((void**)&f->out1, f->N3 * COUT * sizeof(float)) &&
       alloc((void**)&f->eps0, f->N3 * COUT * sizeof(float)) &&
       alloc((void**)&f->ftab, 256 * sizeof(float2));
-  if (!ok || cudaMallocHost((void**)&f->hE, B * CE * sizeof(float)) != cudaSuccess ||
-      cudaMallocHost((void**)&f->hloss, 64) != cudaSuccess ||
+  if (!ok || cudaMallocHost((void**)&f->hloss, 64) != cudaSuccess ||
       cudaEventCreateWithFlags(&f->ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     rpm_fno_destroy(f);
@@ -2112,7 +2123,6 @@ void rpm_fno_destroy(rpm_fno* f) {
                  f->Ed,     f->feat1, f->out1,  f->eps0,  f->ftab, f->tab};
   for (void* p : dev)
     if (p) cudaFree(p);
-  if (f->hE) cudaFreeHost(f->hE);
   if (f->hloss) cudaFreeHost(f->hloss);
   if (f->ev) cudaEventDestroy(f->ev);
   delete f;

@@ -364,3 +364,28 @@ def test_bf16_forward_alone_matches_the_training_pass(fno, N, m, L, B):
     ref = fo.forward(p, feat.astype(np.float32).astype(np.float64), E, m, L)
     err = np.max(np.abs(out.cpu().numpy() - ref)) / np.max(np.abs(ref))
     assert err < BF16_OUT_TOL, err
+
+
+@pytest.mark.parametrize("precision,B", [("bf16", 1), ("fp32", 2), ("bf16", 64)])
+def test_forward_calls_in_a_row_keep_their_own_strain(fno, precision, B):
+    """A forward call is asynchronous: its E is the caller's at the time of the
+    call, also when later calls bring another before the stream gets to it."""
+    N, m, L = 32, 2, 1
+    p = _round32(_params(m, L, 23))
+    feat, _ = _inputs(N, B, 11)
+    feat = _dev(feat)
+    rng = np.random.Generator(np.random.PCG64(12))
+    Es = [rng.standard_normal((B, 6)).astype(np.float32) for _ in range(3)]
+    want = [torch.empty((B, 6, N, N, N), device="cuda") for _ in Es]
+    got = [torch.empty_like(w) for w in want]
+    with fno.Fno(N, m, L, max_batch=B, precision=precision) as net:
+        net.set_params(p)
+        for E, w in zip(Es, want):
+            net.forward(feat, E, w)
+            torch.cuda.synchronize()
+        torch.cuda._sleep(100_000_000)   # the stream is busy while the calls are queued
+        for E, g in zip(Es, got):
+            net.forward(feat, E, g)
+        torch.cuda.synchronize()
+    for k, (g, w) in enumerate(zip(got, want)):
+        assert torch.equal(g, w), k
