@@ -248,7 +248,9 @@ rpm_status rpm_apply_gamma_noalloc(const rpm_grid* grid, const uint8_t* phase, i
  * as eps = base + y and the iteration continues on y with the same linear
  * part and the defect F(base) - base (same fixed point; at most 16 times per
  * solve).
- * Synchronises the context stream before returning.
+ * Synchronises the context stream before returning.  Residuals are read in
+ * between; the calling thread polls for them, or sleeps where the process set
+ * the device to cudaDeviceScheduleBlockingSync.
  */
 rpm_status rpm_solve(rpm_ctx* ctx, const double E[6], const float* eps0, float* eps_out,
                      float* sig_out, int out_on_host, rpm_solve_info* info);

@@ -75,6 +75,7 @@ struct rpm_ctx {
   double* dsmall = nullptr;
   double* hsmall = nullptr;          // pinned host mirror; the sequence word follows it
   unsigned long long seq = 0;        // reads asked of the device so far (see HostRead)
+  bool blocking = false;             // the device is set to cudaDeviceScheduleBlockingSync
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   size_t bytes = 0;
   std::string err;
@@ -366,8 +367,10 @@ struct Ops {
   // The host mirror's [off, off + count) holds the device's values: left there
   // by a fused dots(K, ..., kRead), else copied.  The wait polls the sequence
   // word; now and then it asks the stream, whose error or end ends the wait.
+  // A process that asked for blocking synchronisation sleeps in the stream's.
   bool fetch(int K, int off, int count) {
     if (!fused(K)) return read_small(off, count);
+    if (c->blocking) return ck(c, cudaStreamSynchronize(c->st), "sync");
     const unsigned long long want = c->seq;
     for (unsigned spins = 1;; ++spins) {
       if (__atomic_load_n(seq_word(), __ATOMIC_ACQUIRE) >= want) return true;
@@ -804,6 +807,9 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
   c->H.clear();
   std::vector<double> M;
 
+  unsigned int sched = 0;
+  if (!ck(c, cudaGetDeviceFlags(&sched), "device flags")) return RPM_ERR_CUDA;
+  c->blocking = (sched & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   if (!ck(c, cudaEventRecord(c->ev0, c->st), "event")) return RPM_ERR_CUDA;
   if (!ck(c, cudaMemsetAsync(ds, 0, (kSmall + 1) * 8, c->st), "memset")) return RPM_ERR_CUDA;
   // A basis of the same map left in Z and W by an earlier solve (another load

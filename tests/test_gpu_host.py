@@ -1,0 +1,44 @@
+"""What the library's host code owes its caller on a GPU: how it waits, what a
+failed call leaves behind, what it needs of device memory."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+import microstructure as ms
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_BLOCKING = """
+import ctypes, time
+cu = ctypes.CDLL("libcuda.so.1")
+dev = ctypes.c_int()
+assert cu.cuInit(0) == 0 and cu.cuDeviceGet(ctypes.byref(dev), 0) == 0
+assert cu.cuDevicePrimaryCtxSetFlags_v2(dev, 4) == 0     # blocking synchronisation
+import torch
+import microstructure as ms
+from paper_2003_07720_gb300 import rpm
+torch.cuda.init()
+with rpm.Context(ms.cell_sphere32(32)) as ctx:
+    st, first = ctx.solve(ms.unit_strain(0))
+    torch.cuda._sleep(800_000_000)                        # some 0.4 s ahead of the solve
+    wall, cpu = time.perf_counter(), time.thread_time()
+    st, info = ctx.solve(ms.unit_strain(0))
+    wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+assert info["converged"] and info["mean_stress"] == first["mean_stress"]
+print(wall, cpu)
+"""
+
+
+def test_solve_sleeps_where_the_device_is_set_to_blocking_synchronisation():
+    """The flags are the process's, so the solve runs in a child.  A thread that
+    sleeps until its first residual arrives uses next to no processor time."""
+    r = subprocess.run([sys.executable, "-c", _BLOCKING], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr
+    wall, cpu = map(float, r.stdout.split())
+    assert wall > 0.2 and cpu < 0.25 * wall, (wall, cpu)
