@@ -167,6 +167,8 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
 // Launch with programmatic stream serialization: the kernel may begin (its
 // fixed-table prologue) while the previous kernel of the stream finishes.
 // cluster > 1 groups that many consecutive blocks (along x) into a cluster.
+// A launch that fails is the caller's to report: it leaves no pending error for
+// the check after a later, unrelated launch to find.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, int threads,
                                       size_t smem, cudaStream_t st, unsigned cluster,
@@ -188,7 +190,9 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, int t
     attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
   }
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 template <typename... KArgs, typename... Args>

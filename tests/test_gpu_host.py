@@ -42,3 +42,37 @@ def test_solve_sleeps_where_the_device_is_set_to_blocking_synchronisation():
     assert r.returncode == 0, r.stderr
     wall, cpu = map(float, r.stdout.split())
     assert wall > 0.2 and cpu < 0.25 * wall, (wall, cpu)
+
+
+def _cu(name, *args):
+    import ctypes
+    return getattr(ctypes.CDLL("libcuda.so.1"), name)(*args)
+
+
+@pytest.mark.parametrize("shape", [(16, 16, 16), (48, 48, 48), (4, 8, 12)])
+def test_a_refused_launch_leaves_no_error_behind(shape):
+    """A map on a stream whose capture was invalidated is refused; the next call,
+    on a sound stream, must not find that error."""
+    import ctypes
+
+    import numpy as np
+    from paper_2003_07720_gb300 import rpm
+    cell = ms.cell_sphere32(16)
+    cell = ms.Cell(phase=np.zeros(shape, np.uint8), lam=cell.lam, mu=cell.mu, lam0=cell.lam0,
+                   mu0=cell.mu0)
+    x = torch.zeros((6,) + shape, device="cuda")
+    y = torch.empty_like(x)
+    E = ms.unit_strain(0)
+    stream, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    assert _cu("cuStreamCreate", ctypes.byref(stream), 1) == 0
+    with rpm.Context(cell, rpm.rpm_default_options(p_max=0), stream=stream.value) as bad, \
+            rpm.Context(cell, rpm.rpm_default_options(p_max=0)) as good:
+        torch.cuda.synchronize()
+        assert _cu("cuStreamBeginCapture_v2", stream, 2) == 0
+        assert _cu("cuStreamSynchronize", stream) != 0        # invalidates the capture
+        with pytest.raises(rpm.RpmError):
+            bad.apply_gamma(x, E, y)
+        assert _cu("cuStreamEndCapture", stream, ctypes.byref(graph)) != 0
+        st, info = good.solve(E)
+        assert st == rpm.RPM_OK and info["converged"]
+    assert _cu("cuStreamDestroy_v2", stream) == 0
