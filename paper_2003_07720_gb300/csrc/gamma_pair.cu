@@ -1663,32 +1663,38 @@ cudaError_t launch_pair_polarization(const GridDev& g, const float4* post, const
 }
 
 void pair_tables(int nx, int ny, int nz, PairTables* t) {
+  *t = PairTables{};
   auto root = [](int k, int n) {
     const double a = -2.0 * M_PI * (double)k / (double)n;
     return make_float2((float)std::cos(a), (float)std::sin(a));
   };
-  auto twiddles = [&](int len, int n1, std::vector<float2>& out) {   // W_len^(n2 k1) at k1 * N2 + n2
-    out.clear();
+  auto twiddles = [&](int len, int n1, float2* out) {   // W_len^(n2 k1) at k1 * N2 + n2
     for (int k1 = 0; k1 < n1; ++k1)
-      for (int n2 = 0; n2 < len / n1; ++n2) out.push_back(root(n2 * k1, len));
+      for (int n2 = 0; n2 < len / n1; ++n2) *out++ = root(n2 * k1, len);
   };
   const int nxh = nx / 2, nyh = ny / 2;
   twiddles(nxh, pair_n1(nxh), t->twx);
   twiddles(nyh, pair_n1(nyh), t->twy);
   twiddles(nz, pair_z1(nz), t->twz);
-  t->hw.clear();
-  t->fx.clear();
-  t->fy.clear();
-  for (int j = 0; j < nyh; ++j) t->hw.push_back(root(j, ny));
+  for (int j = 0; j < nyh; ++j) t->hw[j] = root(j, ny);
   for (int s = 0; s <= nxh; ++s) {
     const int k = s < nxh ? split_freq(nxh, pair_n1(nxh), s) : nxh;
-    t->fx.push_back(k == nxh ? make_int2(-k, 1) : make_int2(k, 0));
+    t->fx[s] = k == nxh ? make_int2(-k, 1) : make_int2(k, 0);
   }
   auto signed_y = [&](int k) { return 2 * k < ny ? k : k - ny; };
   for (int s = 0; s < nyh; ++s) {
     const int e = 2 * split_freq(nyh, pair_n1(nyh), s), o = e + 1;
-    t->fy.push_back(make_int4(signed_y(e), 2 * e == ny, signed_y(o), 2 * o == ny));
+    t->fy[s] = make_int4(signed_y(e), 2 * e == ny, signed_y(o), 2 * o == ny);
   }
+}
+
+void set_pair_tables(GridDev* g, const PairTables* dev) {
+  g->p_twx = dev->twx;
+  g->p_twy = dev->twy;
+  g->p_twz = dev->twz;
+  g->p_hw = dev->hw;
+  g->p_fx = dev->fx;
+  g->p_fy = dev->fy;
 }
 
 }  // namespace rpm

@@ -4,17 +4,17 @@
 // Some callers may not call cudaMalloc at all: a host application that owns
 // every byte of device memory through its own pool or plug-in allocator, or a
 // latency-critical loop where cudaMalloc's implicit device synchronisation is
-// not acceptable.  This entry point needs no context and allocates nothing.
-// Its scratch -- the half spectrum and the FFT, frequency and material tables
-// -- lives in file-scope __device__ arrays of fixed size, which every GPU that
-// loads the library keeps until the process exits.  The caller passes the
-// phase map, the input field and the output field.
-#include <algorithm>
+// not acceptable.  This entry point needs no context and allocates nothing,
+// on the device or on the host.  Its scratch -- the half spectrum and the FFT,
+// frequency and material tables -- lives in file-scope __device__ arrays of
+// fixed size, which every GPU that loads the library keeps until the process
+// exits; the tables are filled on the caller's stack.  The caller passes the
+// phase map, the input field and the output field.  All grids it serves have
+// square planes: the paired kernels of gamma_pair.cu.
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "fft_smem.cuh"
 #include "rpm.h"
 #include "rpm_internal.h"
 
@@ -27,13 +27,8 @@ constexpr int kNaMax = 64;
 constexpr size_t kNaSpec = (size_t)6 * kNaMax * kNaMax * (kNaMax / 2 + 1);
 
 static __device__ __align__(256) float2 g_na_spec[kNaSpec];
-static __device__ __align__(256) float2 g_na_tw[3 * kNaMax];        // x (nx/2), y, z twiddles
 static __device__ __align__(256) float2 g_na_r2c[kNaMax / 2 + 1];
-static __device__ __align__(256) int2 g_na_f[kNaMax / 2 + 1 + kNaMax];  // x slots, then y slots
-// the paired kernels' tables: x (nx/2), y (ny/2), z twiddles, W_ny^j; x and y slots
-static __device__ __align__(256) float2 g_na_ptw[5 * kNaMax / 2];
-static __device__ __align__(256) int2 g_na_pfx[kNaMax / 2 + 1];
-static __device__ __align__(256) int4 g_na_pfy[kNaMax / 2];
+static __device__ __align__(256) PairTables g_na_pair;
 static __device__ __align__(256) float2 g_na_mat[2 * 256];           // (dlam, dmu), (lam, mu)
 static __device__ __align__(256) int g_na_err[4];                    // bounded-wait flag
 
@@ -44,12 +39,8 @@ struct NaDevice {
   std::once_flag once;
   cudaError_t setup = cudaSuccess;
   float2* spec = nullptr;
-  float2* tw = nullptr;
   float2* r2c = nullptr;
-  int2* f = nullptr;
-  float2* ptw = nullptr;
-  int2* pfx = nullptr;
-  int4* pfy = nullptr;
+  PairTables* pair = nullptr;
   float2* mat = nullptr;
   int* err = nullptr;
   std::mutex mu;            // guards the key below
@@ -68,27 +59,14 @@ cudaError_t na_setup(int dev, NaDevice** out) {
   std::call_once(d.once, [&d]() {
     cudaError_t e;
     if ((e = cudaGetSymbolAddress((void**)&d.spec, g_na_spec)) != cudaSuccess ||
-        (e = cudaGetSymbolAddress((void**)&d.tw, g_na_tw)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.r2c, g_na_r2c)) != cudaSuccess ||
-        (e = cudaGetSymbolAddress((void**)&d.f, g_na_f)) != cudaSuccess ||
-        (e = cudaGetSymbolAddress((void**)&d.ptw, g_na_ptw)) != cudaSuccess ||
-        (e = cudaGetSymbolAddress((void**)&d.pfx, g_na_pfx)) != cudaSuccess ||
-        (e = cudaGetSymbolAddress((void**)&d.pfy, g_na_pfy)) != cudaSuccess ||
+        (e = cudaGetSymbolAddress((void**)&d.pair, g_na_pair)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.mat, g_na_mat)) != cudaSuccess ||
         (e = cudaGetSymbolAddress((void**)&d.err, g_na_err)) != cudaSuccess)
       d.setup = e;
   });
   *out = &d;
   return d.setup;
-}
-
-void na_twiddles(int L, float2* out) {
-  const int N1 = split_n1(L), N2 = split_n2(L);
-  for (int n2 = 0; n2 < N2; ++n2)
-    for (int k1 = 0; k1 < N1; ++k1) {
-      const double a = -2.0 * M_PI * (double)n2 * (double)k1 / (double)L;
-      out[n2 * N1 + k1] = make_float2((float)std::cos(a), (float)std::sin(a));
-    }
 }
 
 }  // namespace
@@ -140,47 +118,16 @@ extern "C" rpm_status rpm_apply_gamma_noalloc(const rpm_grid* grid, const uint8_
       // host tables (the same definitions as a context's), then stream-ordered
       // copies into the file-scope arrays.  From pageable host memory a copy
       // returns once its source has been staged, so the stack arrays may go.
-      float2 tw[3 * kNaMax];
-      na_twiddles(nxh, tw);
-      na_twiddles(ny, tw + kNaMax);
-      na_twiddles(nz, tw + 2 * kNaMax);
       float2 r2c[kNaMax / 2 + 1];
       for (int k = 0; k <= nxh; ++k) {
         const double ang = -2.0 * M_PI * (double)k / (double)nx;
         r2c[k] = make_float2((float)std::cos(ang), (float)std::sin(ang));
       }
-      int2 f[kNaMax / 2 + 1 + kNaMax];
-      for (int s = 0; s <= nxh; ++s) {
-        const int k = s < nxh ? freq_of_rt(nxh, s) : nxh;
-        const bool nyq = (k == nxh);
-        f[s] = make_int2(nyq ? -k : k, nyq ? 1 : 0);
-      }
-      for (int s = 0; s < ny; ++s) {
-        const int k = freq_of_rt(ny, s);
-        f[nxh + 1 + s] =
-            make_int2((2 * k < ny) ? k : k - ny, (ny % 2 == 0 && 2 * k == ny) ? 1 : 0);
-      }
-      PairTables pt;
-      pair_tables(nx, ny, nz, &pt);
-      float2 ptw[5 * kNaMax / 2];
-      int2 pfx[kNaMax / 2 + 1];
-      int4 pfy[kNaMax / 2];
-      std::memset(ptw, 0, sizeof(ptw));
-      std::memset(pfx, 0, sizeof(pfx));
-      std::memset(pfy, 0, sizeof(pfy));
-      std::copy(pt.twx.begin(), pt.twx.end(), ptw);
-      std::copy(pt.twy.begin(), pt.twy.end(), ptw + kNaMax / 2);
-      std::copy(pt.twz.begin(), pt.twz.end(), ptw + kNaMax);
-      std::copy(pt.hw.begin(), pt.hw.end(), ptw + 2 * kNaMax);
-      std::copy(pt.fx.begin(), pt.fx.end(), pfx);
-      std::copy(pt.fy.begin(), pt.fy.end(), pfy);
+      PairTables pair;
+      pair_tables(nx, ny, nz, &pair);
       a->have_key = false;
-      if (cudaMemcpyAsync(a->ptw, ptw, sizeof(ptw), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-          cudaMemcpyAsync(a->pfx, pfx, sizeof(pfx), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-          cudaMemcpyAsync(a->pfy, pfy, sizeof(pfy), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-          cudaMemcpyAsync(a->tw, tw, sizeof(tw), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+      if (cudaMemcpyAsync(a->pair, &pair, sizeof(pair), cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(a->r2c, r2c, sizeof(r2c), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-          cudaMemcpyAsync(a->f, f, sizeof(f), cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(a->mat, mat, sizeof(mat), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return RPM_ERR_CUDA;
       a->key_grid[0] = nx;
@@ -198,18 +145,8 @@ extern "C" rpm_status rpm_apply_gamma_noalloc(const rpm_grid* grid, const uint8_
   g.nxh = nxh;
   g.n = (long long)nx * ny * nz;
   g.plane = ny * (nxh + 1);
-  g.tw_x = a->tw;
-  g.tw_y = a->tw + kNaMax;
-  g.tw_z = a->tw + 2 * kNaMax;
   g.r2c_w = a->r2c;
-  g.fx = a->f;
-  g.fy = a->f + nxh + 1;
-  g.p_twx = a->ptw;
-  g.p_twy = a->ptw + kNaMax / 2;
-  g.p_twz = a->ptw + kNaMax;
-  g.p_hw = a->ptw + 2 * kNaMax;
-  g.p_fx = a->pfx;
-  g.p_fy = a->pfy;
+  set_pair_tables(&g, a->pair);
   g.phase = phase;
   g.dmat = a->mat;
   g.cmat = a->mat + 256;

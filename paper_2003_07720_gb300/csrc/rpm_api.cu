@@ -607,12 +607,7 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
   const size_t o_pt = off; off = align_up(off + 256 * 16, 256);
   const size_t o_dp = off; off = align_up(off + 256 * 8, 256);
   const size_t o_err = off; off = align_up(off + 16, 256);
-  const size_t o_px = off; off = align_up(off + pt.twx.size() * 8, 256);
-  const size_t o_py = off; off = align_up(off + pt.twy.size() * 8, 256);
-  const size_t o_pz = off; off = align_up(off + pt.twz.size() * 8, 256);
-  const size_t o_ph = off; off = align_up(off + pt.hw.size() * 8, 256);
-  const size_t o_pfx = off; off = align_up(off + pt.fx.size() * 8, 256);
-  const size_t o_pfy = off; off = align_up(off + pt.fy.size() * 16, 256);
+  const size_t o_pair = off; off = align_up(off + sizeof(PairTables), 256);
   const size_t tab_bytes = off;
   c->nblk = std::max(dots_blocks_for(c->n), stress_blocks_for(c->n));
   const size_t fbytes = c->fst * sizeof(float);
@@ -666,12 +661,7 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
       put(o_fy, fy.data(), fy.size() * 8) != cudaSuccess ||
       put(o_dm, dm256.data(), 256 * 8) != cudaSuccess ||
       put(o_cm, cm256.data(), 256 * 8) != cudaSuccess ||
-      put(o_px, pt.twx.data(), pt.twx.size() * 8) != cudaSuccess ||
-      put(o_py, pt.twy.data(), pt.twy.size() * 8) != cudaSuccess ||
-      put(o_pz, pt.twz.data(), pt.twz.size() * 8) != cudaSuccess ||
-      put(o_ph, pt.hw.data(), pt.hw.size() * 8) != cudaSuccess ||
-      put(o_pfx, pt.fx.data(), pt.fx.size() * 8) != cudaSuccess ||
-      put(o_pfy, pt.fy.data(), pt.fy.size() * 16) != cudaSuccess ||
+      put(o_pair, &pt, sizeof(pt)) != cudaSuccess ||
       cudaMemsetAsync(c->dsmall, 0, (kSmall + 1) * 8, c->st) != cudaSuccess ||
       cudaMemsetAsync(t + o_err, 0, 16, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) {
@@ -686,12 +676,7 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
   g.fy = (const int2*)(t + o_fy);
   g.dmat = (const float2*)(t + o_dm);
   g.cmat = (const float2*)(t + o_cm);
-  g.p_twx = (const float2*)(t + o_px);
-  g.p_twy = (const float2*)(t + o_py);
-  g.p_twz = (const float2*)(t + o_pz);
-  g.p_hw = (const float2*)(t + o_ph);
-  g.p_fx = (const int2*)(t + o_pfx);
-  g.p_fy = (const int4*)(t + o_pfy);
+  set_pair_tables(&g, (const PairTables*)(t + o_pair));
   g.phase = c->phase;
   g.err = (int*)(t + o_err);
   c->dmat_b = (float2*)(t + o_db);

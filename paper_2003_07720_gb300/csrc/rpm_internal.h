@@ -3,8 +3,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <vector>
-
 #include "rpm.h"
 
 namespace rpm {
@@ -31,13 +29,13 @@ struct GridDev {
   const float2* r2c_w;   // W_{nx}^k, k = 0..nxh
   const int2* fx;        // per x slot: (signed frequency m, nyquist flag)
   const int2* fy;        // per y slot
-  // the same for the paired kernels (gamma_pair.cu), built by pair_tables
-  const float2* p_twx;   // W_{nx/2}^(n2*k1)
-  const float2* p_twy;   // W_{ny/2}^(n2*k1)
-  const float2* p_twz;   // W_{nz}^(n2*k1)
-  const float2* p_hw;    // W_{ny}^j, j < ny/2
-  const int2* p_fx;      // per x slot: (signed frequency, nyquist flag)
-  const int4* p_fy;      // per y slot: the same of the even and the odd line
+  // the same for the paired kernels (gamma_pair.cu): arrays of a PairTables
+  const float2* p_twx;
+  const float2* p_twy;
+  const float2* p_twz;
+  const float2* p_hw;
+  const int2* p_fx;
+  const int4* p_fy;
   const uint8_t* phase;  // [nz][ny][nx]
   const float2* dmat;    // per phase: (lam - lam0, mu - mu0)
   const float2* cmat;    // per phase: (lam, mu)
@@ -59,13 +57,18 @@ struct GammaArgs {
 GammaArgs gamma_args(const GridDev& g, const double E[6]);
 
 // ---- paired kernels (gamma_pair.cu) ----------------------------------------
-// Host tables of a grid; the vectors go to the p_* pointers of GridDev.
-struct PairTables {
-  std::vector<float2> twx, twy, twz, hw;
-  std::vector<int2> fx;
-  std::vector<int4> fy;
+// Tables of a grid, filled on the host and copied to the device as they are.
+// Fixed arrays for the largest sides (256): filling them allocates nothing.
+struct __align__(16) PairTables {
+  int4 fy[128];      // per y slot: (signed frequency, nyquist flag) of the even and the odd line
+  int2 fx[129];      // per x slot: (signed frequency, nyquist flag)
+  float2 twx[128];   // W_{nx/2}^(n2*k1)
+  float2 twy[128];   // W_{ny/2}^(n2*k1)
+  float2 twz[256];   // W_{nz}^(n2*k1)
+  float2 hw[128];    // W_{ny}^j, j < ny/2
 };
 void pair_tables(int nx, int ny, int nz, PairTables* t);
+void set_pair_tables(GridDev* g, const PairTables* dev);   // the p_* pointers
 bool pair_plane_ok(const GridDev& g, const float2* spec);   // grid and buffer take them
 int pair_z_tile(const GridDev& g);                          // pencil pairs per z block
 // launch_apply_gamma / launch_polarization_map on such a grid (float2-aligned fields)
