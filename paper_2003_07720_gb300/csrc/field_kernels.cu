@@ -294,10 +294,13 @@ cudaError_t launch_dots_fused(const float* x, const float* x2, const float* x_mi
 #undef RPM_PT
 }
 
-int dots_blocks_for(long long n) {
-  const long long total = 6 * (n / 4), per = (long long)kRedThreads * dots_per_thread(n);
+static int dots_blocks(long long n, int per_thread) {
+  const long long total = 6 * (n / 4), per = (long long)kRedThreads * per_thread;
   return (int)((total + per - 1) / per);
 }
+
+int dots_fused_blocks_for(long long n) { return dots_blocks(n, dots_per_thread(n)); }
+int dots_blocks_for(long long n) { return dots_blocks(n, kPerThread); }
 
 cudaError_t launch_dots(const float* x, const float* x_minus, const float* Y, long long ystride,
                         int K, long long n, double* partials, int nblk, cudaStream_t st) {

@@ -39,9 +39,8 @@ constexpr int kMaxRebase = 16;        // re-centrings of one solve (see solve_im
 // Basis growth is skipped while |xi^nu - xi^(nu-1)| < kGrowNoise |xi|: such a
 // difference is dominated by the float32 rounding of F (about 2e-7 |xi|).
 constexpr double kGrowNoise = 1e-5;
-constexpr int kM = kRes + 8;          // (I - H)^-1, kPCap x kPCap
-constexpr int kSmall = kM + kPCap * kPCap;
-constexpr int kTicket = kSmall;       // one more slot: the fused reduction's counter
+constexpr int kTicket = kRes + 1;     // the fused reduction's counter
+constexpr int kM = kRes + 8;          // (I - H)^-1, p_cap x p_cap; the host mirror ends before it
 constexpr int kFusedMaxBlocks = 1024; // dots blocks up to which the fused reduction pays
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -70,8 +69,10 @@ struct rpm_ctx {
   float* fields = nullptr;           // eps[2], xi[3], D[2], eps_b, base, defect
   float* Z = nullptr;
   float* W = nullptr;
-  double* partials = nullptr;
-  int nblk = 0;
+  double* partials = nullptr;        // see partial_doubles
+  int nblk = 0;                      // blocks of the fused dots
+  int nblk_wide = 0;                 // blocks of the other reductions (eight float4 a thread)
+  size_t small_bytes = 0;            // dsmall
   double* dsmall = nullptr;
   double* hsmall = nullptr;          // pinned host mirror; the sequence word follows it
   unsigned long long seq = 0;        // reads asked of the device so far (see HostRead)
@@ -277,6 +278,15 @@ void upload_materials(rpm_ctx* c, std::vector<float2>& dm, std::vector<float2>& 
   }
 }
 
+// Largest set of per-block rows a reduction of this context leaves: the fused
+// dots (where used) of two fields against min(p_cap, 32) vectors, the others'
+// 1 + p_cap sums and the six mean stresses.
+size_t partial_doubles(const rpm_ctx* c) {
+  const size_t fused = c->nblk <= kFusedMaxBlocks
+                           ? 2 * (std::min(c->p_cap, 32) + 1) * (size_t)c->nblk : 0;
+  return std::max(fused, std::max(c->p_cap + 1, 6) * (size_t)c->nblk_wide);
+}
+
 // --- thin wrappers that record the failing step ---------------------------
 struct Ops {
   rpm_ctx* c;
@@ -326,7 +336,7 @@ struct Ops {
   // K <= 32 on grids up to ~100^3: one fused launch (the last block's serial
   // tail costs more than two launches beyond that)
   bool fused(int K) const { return K <= 32 && c->nblk <= kFusedMaxBlocks; }
-  unsigned long long* seq_word() { return reinterpret_cast<unsigned long long*>(c->hsmall + kSmall); }
+  unsigned long long* seq_word() { return reinterpret_cast<unsigned long long*>(c->hsmall + kM); }
   // sums[0..K] <- dots of x against Y (see launch_dots); with M, also the Newton
   // step into c and the residual.  A non-null x2 (fused(K) only) adds the sums
   // of x2 after them.  Read: a fused reduction leaves sums (and residual) in
@@ -356,9 +366,9 @@ struct Ops {
               "dots");
     } else {
       c->launches += 1 + dots_launches(K) + (M ? 1 : 0);
-      ok = ck(c, launch_dots(x, xm, Y, (long long)c->fst, K, c->n, c->partials, c->nblk, c->st),
+      ok = ck(c, launch_dots(x, xm, Y, (long long)c->fst, K, c->n, c->partials, c->nblk_wide, c->st),
               "dots") &&
-           ck(c, launch_reduce_partials(c->partials, c->nblk, K + 1, sums, c->st), "reduce") &&
+           ck(c, launch_reduce_partials(c->partials, c->nblk_wide, K + 1, sums, c->st), "reduce") &&
            (!M || ck(c, launch_newton(sums, K, M, cN, res, inv_norm, c->st), "newton"));
     }
     done(m);
@@ -609,12 +619,14 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
   const size_t o_err = off; off = align_up(off + 16, 256);
   const size_t o_pair = off; off = align_up(off + sizeof(PairTables), 256);
   const size_t tab_bytes = off;
-  c->nblk = std::max(dots_blocks_for(c->n), stress_blocks_for(c->n));
+  c->nblk = dots_fused_blocks_for(c->n);
+  c->nblk_wide = std::max(dots_blocks_for(c->n), stress_blocks_for(c->n));
+  c->small_bytes = (kM + (size_t)c->p_cap * c->p_cap) * 8;
+  const size_t partial_bytes = partial_doubles(c) * 8;
   const size_t fbytes = c->fst * sizeof(float);
   const size_t spec_bytes = (size_t)6 * nz * g.plane * sizeof(float2);
   const size_t need = tab_bytes + align_up((size_t)c->n, 256) + spec_bytes + kFields * fbytes +
-                      2 * (size_t)c->p_cap * fbytes + (size_t)(kPCap + 1) * c->nblk * 8 +
-                      (kSmall + 1) * 8;
+                      2 * (size_t)c->p_cap * fbytes + partial_bytes + c->small_bytes;
   if (o.max_device_gb > 0 && (double)need > o.max_device_gb * 1e9) {
     rpm_destroy(c);
     return RPM_ERR_OOM;
@@ -632,18 +644,18 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
       (e = alloc((void**)&c->fields, kFields * fbytes)) != cudaSuccess ||
       (e = alloc((void**)&c->Z, (size_t)c->p_cap * fbytes)) != cudaSuccess ||
       (e = alloc((void**)&c->W, (size_t)c->p_cap * fbytes)) != cudaSuccess ||
-      (e = alloc((void**)&c->partials, (size_t)(kPCap + 1) * c->nblk * 8)) != cudaSuccess ||
-      (e = alloc((void**)&c->dsmall, (kSmall + 1) * 8)) != cudaSuccess) {
+      (e = alloc((void**)&c->partials, partial_bytes)) != cudaSuccess ||
+      (e = alloc((void**)&c->dsmall, c->small_bytes)) != cudaSuccess) {
     cudaGetLastError();
     rpm_destroy(c);
     return e == cudaErrorMemoryAllocation ? RPM_ERR_OOM : RPM_ERR_CUDA;
   }
-  if (cudaMallocHost((void**)&c->hsmall, (kSmall + 8) * 8) != cudaSuccess ||
+  if (cudaMallocHost((void**)&c->hsmall, (kM + 8) * 8) != cudaSuccess ||
       cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess) {
     rpm_destroy(c);
     return RPM_ERR_CUDA;
   }
-  std::memset(c->hsmall, 0, (kSmall + 8) * 8);
+  std::memset(c->hsmall, 0, (kM + 8) * 8);
   char* t = c->tables;
   auto put = [&](size_t o2, const void* src, size_t b) {
     return cudaMemcpyAsync(t + o2, src, b, cudaMemcpyHostToDevice, c->st);
@@ -662,7 +674,7 @@ rpm_status rpm_create(const rpm_grid* grid, const uint8_t* phase, int phase_on_d
       put(o_dm, dm256.data(), 256 * 8) != cudaSuccess ||
       put(o_cm, cm256.data(), 256 * 8) != cudaSuccess ||
       put(o_pair, &pt, sizeof(pt)) != cudaSuccess ||
-      cudaMemsetAsync(c->dsmall, 0, (kSmall + 1) * 8, c->st) != cudaSuccess ||
+      cudaMemsetAsync(c->dsmall, 0, c->small_bytes, c->st) != cudaSuccess ||
       cudaMemsetAsync(t + o_err, 0, 16, c->st) != cudaSuccess ||
       cudaStreamSynchronize(c->st) != cudaSuccess) {
     rpm_destroy(c);
@@ -796,7 +808,7 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
   if (!ck(c, cudaGetDeviceFlags(&sched), "device flags")) return RPM_ERR_CUDA;
   c->blocking = (sched & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   if (!ck(c, cudaEventRecord(c->ev0, c->st), "event")) return RPM_ERR_CUDA;
-  if (!ck(c, cudaMemsetAsync(ds, 0, (kSmall + 1) * 8, c->st), "memset")) return RPM_ERR_CUDA;
+  if (!ck(c, cudaMemsetAsync(ds, 0, c->small_bytes, c->st), "memset")) return RPM_ERR_CUDA;
   // A basis of the same map left in Z and W by an earlier solve (another load
   // E, or the same one): with share_basis the solve starts from its leading
   // min(size, p_max) vectors, H's leading block and M = (I - H)^-1.
@@ -1137,8 +1149,8 @@ rpm_status solve_impl(rpm_ctx* c, const double E[6], const float* eps0, float* e
   float* sig_dev = sig_out ? (out_on_host ? D[0] : sig_out) : nullptr;
   if (sig_dev == eps_cur) sig_dev = D[1];
   c->launches += 2;
-  if (!ck(c, launch_stress(c->g, eps_cur, sig_dev, c->partials, c->nblk, c->st), "stress") ||
-      !ck(c, launch_reduce_partials(c->partials, c->nblk, 6, ds + kSums, c->st), "reduce"))
+  if (!ck(c, launch_stress(c->g, eps_cur, sig_dev, c->partials, c->nblk_wide, c->st), "stress") ||
+      !ck(c, launch_reduce_partials(c->partials, c->nblk_wide, 6, ds + kSums, c->st), "reduce"))
     return RPM_ERR_CUDA;
   if (sig_out && out_on_host) {
     if (!ck(c, cudaMemcpyAsync(sig_out, sig_dev, fb, cudaMemcpyDeviceToHost, c->st), "sig_out"))

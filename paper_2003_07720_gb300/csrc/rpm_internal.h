@@ -115,7 +115,8 @@ bool fused_z_pass(const GridDev& g);   // g.pencil_t resolves to the fused z ker
 
 // ---- field kernels (field_kernels.cu) -------------------------------------
 // Partial sums per block, then one finishing block; see the definitions.
-int dots_blocks_for(long long n);
+int dots_blocks_for(long long n);        // blocks of launch_dots
+int dots_fused_blocks_for(long long n);  // of launch_dots_fused
 int dots_launches(int K);
 int combine_launches(int K);
 int stress_blocks_for(long long n);

@@ -76,3 +76,18 @@ def test_a_refused_launch_leaves_no_error_behind(shape):
         st, info = good.solve(E)
         assert st == rpm.RPM_OK and info["converged"]
     assert _cu("cuStreamDestroy_v2", stream) == 0
+
+
+@pytest.mark.parametrize("shape,p_max,need", [
+    # bytes per context before the reductions took more blocks on small grids
+    ((16, 16, 16), 0, 1690016), ((16, 16, 16), 10, 3743136), ((48, 48, 48), 20, 136513296),
+    ((24, 96, 48), 40, 242855952), ((64, 64, 64), 20, 322479240), ((1, 64, 64), 250, 53009824)])
+def test_a_context_needs_no_more_device_memory_than_it_did(shape, p_max, need):
+    """A cap that was enough for a context stays enough."""
+    import numpy as np
+    from paper_2003_07720_gb300 import rpm
+    cell = ms.cell_sphere32(16)
+    cell = ms.Cell(phase=np.zeros(shape, np.uint8), lam=cell.lam, mu=cell.mu, lam0=cell.lam0,
+                   mu0=cell.mu0)
+    with rpm.Context(cell, rpm.rpm_default_options(p_max=p_max, max_device_gb=need / 1e9)) as ctx:
+        assert rpm.rpm_device_bytes(ctx.handle) <= need
