@@ -1643,6 +1643,7 @@ cudaError_t launch_pair_map(const GridDev& g, const float* in, float* out, float
 
 cudaError_t launch_pair_rows_map(const GridDev& g, const float* in, float* out, float2* spec,
                                  const double E[6], int mode, cudaStream_t st, const float* add) {
+  if ((uintptr_t)spec & 15) return cudaErrorInvalidValue;   // as in pair_plane_ok: no other kernels
   float4* s4 = reinterpret_cast<float4*>(spec);
   cudaError_t e;
   if ((e = pass_rows(g, in, nullptr, s4, mode, false, nullptr, st)) != cudaSuccess) return e;

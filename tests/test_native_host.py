@@ -54,3 +54,32 @@ int main() {
   return count == 0 ? 0 : 1;
 }
 """)
+
+
+def test_five_passes_refuse_a_misaligned_spectrum(tmp_path):
+    """Their kernels access the spectrum in 16-byte elements; the check comes
+    before any launch (the pointers here are not memory)."""
+    _run(tmp_path, r"""
+#include <cstdio>
+#include "rpm_internal.h"
+int main() {
+  const int sides[][2] = {{8, 4}, {256, 256}, {64, 48}, {16, 16}};
+  for (auto& s : sides) {
+    rpm::GridDev g{};
+    g.nx = s[0];
+    g.ny = s[1];
+    g.nz = 4;
+    g.nxh = g.nx / 2;
+    g.n = (long long)g.nx * g.ny * g.nz;
+    g.plane = g.ny * (g.nxh + 1);
+    g.plane_v = 2;
+    const cudaError_t e = rpm::launch_apply_gamma(g, (const float*)0x1000, (float*)0x2000,
+                                                  (float2*)0x3008, nullptr, rpm::GM_LINEAR, nullptr);
+    if (e != cudaErrorInvalidValue) {
+      std::printf("%d x %d: %d\n", g.nx, g.ny, (int)e);
+      return 1;
+    }
+  }
+  return 0;
+}
+""")
