@@ -94,14 +94,15 @@ typedef struct {
                             z-pass variants below on the context's grid and keeps the
                             fastest (rpm_set_options then keeps that choice while
                             autotune stays 1); 0 (default): the variants below */
-  int plane_variant;     /* x/y passes: 0 (default) the paired plane kernels where the
-                            grid has them (square planes 48-128), else as 1; 1 the
-                            whole-plane kernels where the plane fits (nx = ny <= 128),
-                            else as 2; 2 the five-pass row and y-pencil kernels */
-  int pencil_variant;    /* z pass: 0 (default) the default tile (with the paired plane
-                            kernels their own z pass; otherwise the register-resident kernel
-                            where the grid has it, nz 32, 48, 96, 128); 1 half, 2 twice the
-                            default pencils per block; 3 the default tile */
+  int plane_variant;     /* x/y passes: 0 (default) the paired kernels, whole square planes
+                            up to 128 x 128 in three passes, other grids as 2; 1 the scalar
+                            whole-plane kernels where the plane fits (nx = ny <= 128), else
+                            as 2; 2 the paired row and y-line kernels in five passes */
+  int pencil_variant;    /* z pass: 0 (default) and 3 the default tile; 1 half, 2 twice the
+                            default pencils per block.  The paired z pass (plane variants 0
+                            and 2) keeps to 2 to 16 pencil pairs a block and has one form at
+                            nz <= 4.  With the scalar plane kernels 0 is the
+                            register-resident kernel at nz 32, 48, 96 and 128 */
   int share_basis;       /* 1: a solve starts from the unstable basis (Z, W = F_u Z, H)
                             that an earlier solve of the same map left in the context --
                             F_u does not depend on the load E, so the six loads of

@@ -84,11 +84,6 @@ __device__ __forceinline__ void bulk_commit() {
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// The issuing thread's bulk stores have finished reading shared memory.
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-
 // The issuing thread's bulk stores are complete.
 __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -137,7 +132,7 @@ __device__ __forceinline__ void allow_dependent_launch() {
 // cluster arrives (release) and waits (acquire), so shared-memory writes
 // before it are visible to the other blocks after it; all threads of a block
 // must execute it.  cluster_map: the address of `p` in the shared memory of
-// the cluster's block `rank`; ld_cluster_f2 / _f4 read through such an address.
+// the cluster's block `rank`; ld_cluster_f4 reads through such an address.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
@@ -148,12 +143,6 @@ __device__ __forceinline__ uint32_t cluster_map(const void* p, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
   return r;
-}
-
-__device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-  return v;
 }
 
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {

@@ -162,6 +162,7 @@ __device__ __forceinline__ void dots_body(const float4* __restrict__ x,
   }
 }
 
+// (bound by HBM: 128^3, K = 20: 174 us, 94 % of the copy rate)
 template <int KMAX>
 __global__ void __launch_bounds__(kRedThreads, 3) k_dots(const float4* __restrict__ x,
                                                       const float4* __restrict__ xm,
@@ -176,8 +177,7 @@ __global__ void __launch_bounds__(kRedThreads, 3) k_dots(const float4* __restric
 // shuffle tree) into sums[0..NX (K + 1)) and, when M is given, takes the Newton
 // step of k_newton with p = K.  The ticket counter is zero between launches
 // (the last block resets it).  One launch instead of three.
-// Large grids: bound by HBM (128^3, p = 20: 174 us, 94 % of the copy rate).
-// Small ones by latency: 32^3 solve 1.64 -> 0.90 ms, 48^3 1.63 -> 1.16 ms with
+// Grids up to about 100^3, bound by latency: 32^3 solve 1.64 -> 0.90 ms, 48^3 1.63 -> 1.16 ms with
 // the polled reads, more blocks, launches that overlap and both differences of
 // a growth at once; 96^3 cold solve 9.8 -> 8.2 ms.
 // With a host block (pinned memory) the sums, and the residual when M is

@@ -1683,9 +1683,9 @@ const uint4* tc_table(const rpm_fno* f, size_t off) {
 cudaError_t launch_xy_fwd(rpm_fno* f, const float* src, int B) {
   const int N = f->N, m = f->m;
   if (f->tc) {
-    // channel groups over blocks until there are two blocks per SM (each block
-    // builds the twiddle tables, so not further): 64^3, one sample, 26.4 -> 11.1 us;
-    // 32^3, two samples, 19.4 -> 7.9 us
+    // channel groups over blocks until there are two blocks per SM, what the
+    // registers allow: 64^3, one sample, 26.4 -> 11.1 us; 32^3, two samples, 19.4 ->
+    // 7.9 us
     int nc = 1;
     while (nc < W / xy_group(N) && N * B * nc < 304) nc *= 2;
     switch (N) {

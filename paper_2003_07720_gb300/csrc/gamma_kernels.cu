@@ -12,11 +12,12 @@
 //   pass C (one block per z-plane and component): inverse FFT along y,
 //       complex-to-real tangling, inverse FFT along x of length nx/2, scale.
 //
-// Square planes nx = ny in {48, 64, 96, 128} run the paired kernels of
-// gamma_pair.cu, which also serves 256^2 planes and nx != ny in five passes.
-// The kernels here serve the small square planes (and the forced whole-plane
-// variant): k_pass_a/b/c, and the z pass k_pencil_green, in which the forward
-// z step 2, the Green operator and the inverse z step 1 run in registers.
+// These scalar kernels (k_pass_a/b/c, and the z pass k_pencil_green, in which
+// the forward z step 2, the Green operator and the inverse z step 1 run in
+// registers) run where a caller forces the whole-plane variant or the autotuner
+// times it.  By default every grid takes the paired kernels of gamma_pair.cu:
+// square planes up to 128 in three passes, 256^2 and nx != ny in five.  The
+// dispatch between them is at the end of this file.
 //
 // The Green operator of the isotropic reference medium is evaluated on the
 // fly from the unit wave vector n = xi/|xi|:
@@ -669,17 +670,13 @@ static cudaError_t dispatch_fused_pencil(const GridDev& g, float2* spec, int mod
   }
 }
 
-#define RPM_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
-#define RPM_Z_SIZES(X) \
-  X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
-
 // three-pass (whole xy planes in shared memory) when the plane fits
 static bool plane_fits(int nx, int ny) { return nx == ny && nx <= 128; }
 
 static bool xy_size_ok(int n) {
   switch (n) {
 #define RPM_CASE(N) case N:
-    RPM_SIZES(RPM_CASE)
+    RPM_XY_SIZES(RPM_CASE)
 #undef RPM_CASE
     return true;
     default: return false;
@@ -695,8 +692,6 @@ static bool z_size_ok(int n) {
     default: return false;
   }
 }
-
-#define RPM_PLANE_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128)
 
 static cudaError_t dispatch_plane(const GridDev& g, const float* in, float* out, float2* spec,
                                   int mode, int which, cudaStream_t st) {

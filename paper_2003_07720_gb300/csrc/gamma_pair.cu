@@ -26,11 +26,13 @@
 //
 // What bounds the passes: with one line per thread they were bound by issue
 // slots (128^3: 19.1, 21.7 and 13.8 M warp instructions in passes A, B, C,
-// 47-61 % issue active).  Pairing brought them to 11.8, 11.6 and 7.5 M; now
-// shared-memory bandwidth (C: 67 % of the L1 pipe's cycles) and the latency of
-// two or three resident blocks bound them.  One map of 128^3: 96 -> 86 us, of
-// 64^3 20.5 -> 15.5 us, of 48^3 15.3 -> 11.2 us, of 16^3 16.4 -> 9.3 us; 96^3
-// passes A + B + C 71 -> 40 us (single-kernel times).
+// 47-61 % issue active).  Pairing brought them to 10.1, 11.7 and 8.5 M; now
+// shared-memory bandwidth (70 and 66 % of the L1 pipe's cycles in A and C) and
+// the latency of two or three resident blocks bound them.  One map among others
+// of 128^3: 96 -> 87 us, of 64^3 20.5 -> 15.2 us, of 48^3 15.3 -> 12.2 us, of
+// 16^3 15.8 -> 9.1 us; 96^3 passes A + B + C 71 -> 40 us (single-kernel times).
+// A first map on fresh inputs, waited for, gains less, being mostly launches:
+// 132 -> 121, 52.9 -> 47.5, 46.1 -> 46.5 and 46.6 -> 41.4 us.
 #include <algorithm>
 #include <cmath>
 
@@ -162,7 +164,7 @@ __device__ __forceinline__ void pair_materials(const GridDev& g, float2* dm, int
 // the other two normal components e1, e2).  Row j + ny/2 lies `low` float2
 // after row j; rows past `rows` are skipped.
 enum { kRaw, kShear, kNormal };
-template <class C, int KIND, bool TWO, bool PACK>
+template <class C, int KIND, bool TWO>
 __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const float2* __restrict__ e1,
                                         const float2* __restrict__ e2,
                                         const uchar2* __restrict__ phase, int low, int rows,
@@ -243,7 +245,7 @@ __device__ __forceinline__ void pair_x1(const float2* __restrict__ e0, const flo
 }
 
 // x step 1 of component c of a block's rows (`in`, `phase`: the first row).
-template <class C, bool PACK>
+template <class C>
 __device__ __forceinline__ void pair_x1_component(const GridDev& g, const float2* in, int c,
                                                   const uchar2* phase, int low, int rows, int mode,
                                                   const float2* dm, float4* P, const float4* twx,
@@ -251,19 +253,19 @@ __device__ __forceinline__ void pair_x1_component(const GridDev& g, const float2
   const size_t nf2 = (size_t)g.n / 2;
   const float2* own = in + c * nf2;
   if (mode == GM_RAW_TAU) {
-    pair_x1<C, kRaw, true, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
+    pair_x1<C, kRaw, true>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   } else if (c >= 3) {
     if (g.n_phases <= 2)
-      pair_x1<C, kShear, true, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
+      pair_x1<C, kShear, true>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
     else
-      pair_x1<C, kShear, false, PACK>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
+      pair_x1<C, kShear, false>(own, in, in, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   } else {
     const float2* other = in + (c == 0 ? 1 : 0) * nf2;
     const float2* last = in + (c == 2 ? 1 : 2) * nf2;
     if (g.n_phases <= 2)
-      pair_x1<C, kNormal, true, PACK>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
+      pair_x1<C, kNormal, true>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
     else
-      pair_x1<C, kNormal, false, PACK>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
+      pair_x1<C, kNormal, false>(own, other, last, phase, low, rows, g.dmat, dm, P, twx, r2c, hw);
   }
 }
 
@@ -365,8 +367,8 @@ __global__ void __launch_bounds__(TPB, PairPlane<N, TPB>::MINB)
   grid_dependency_wait();   // the FFT tables are fixed; everything below may be in flight
   pair_materials(g, dm, TPB);
   __syncthreads();
-  pair_x1_component<X, C::PACK>(g, reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH, c,
-                                reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH,
+  pair_x1_component<X>(g, reinterpret_cast<const float2*>(in) + (size_t)z * N * NXH, c,
+                       reinterpret_cast<const uchar2*>(g.phase) + (size_t)z * N * NXH,
                                 H * NXH, H, mode, dm, P, twx, r2c, hw);
   __syncthreads();
   float4* out = spec + ((size_t)c * g.nz + z) * C::PL;
@@ -772,12 +774,6 @@ __global__ void __launch_bounds__(TPB, PairPlane<N, TPB>::MINB)
   cluster_sync();   // no block leaves while another still reads its planes
 }
 
-// Pass B: T pencil pairs per block.  Forward z step 1 reads the spectrum from
-// global memory; forward step 2, the Green operator and inverse step 1 run in
-// registers on one (pencil pair, k1) group per pair of threads, lanes l and
-// l + 16 holding the normal and the shear components of the same frequencies
-// and exchanging their partial sums of tau_hat n by shuffles; inverse step 2
-// writes back to global memory.
 // ---------------------------------------------------------------------------
 // The same map in five passes, for planes that do not fit in shared memory
 // (256^2) and for nx != ny: x rows, y lines, the z pass, y lines and x rows
@@ -825,7 +821,7 @@ __global__ void __launch_bounds__(PairRows<NX, R>::TPB, PairRows<NX, R>::MINB)
   pair_materials(g, dm, TPB);
   __syncthreads();
   const size_t row0 = ((size_t)z * g.ny + j0) * NXH;
-  pair_x1_component<X, false>(g, reinterpret_cast<const float2*>(in) + row0, c,
+  pair_x1_component<X>(g, reinterpret_cast<const float2*>(in) + row0, c,
                               reinterpret_cast<const uchar2*>(g.phase) + row0, h * NXH, rows,
                               mode, dm, P, twx, r2c, hw);
   __syncthreads();
@@ -1231,6 +1227,12 @@ __device__ __forceinline__ void pair_z_middle(const GridDev& g, float4* B, const
   }
 }
 
+// Pass B: T pencil pairs per block.  Forward z step 1 reads the spectrum from
+// global memory; forward step 2, the Green operator and inverse step 1 run in
+// registers on one (pencil pair, k1) group per pair of threads, lanes l and
+// l + 16 holding the normal and the shear components of the same frequencies
+// and exchanging their partial sums of tau_hat n by shuffles; inverse step 2
+// writes back to global memory.
 template <int NZ, int T>
 __global__ void __launch_bounds__(PairZ<NZ, T>::TPB, PairZ<NZ, T>::MINB)
     k_pair_green(GridDev g, float4* __restrict__ spec, int mode, GammaArgs ga) {
@@ -1538,17 +1540,12 @@ cudaError_t launch_green_tile(const GridDev& g, float4* spec, int mode, const Ga
   }
 }
 
-#define RPM_PAIR_SIZES(X) \
-  X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128)
-#define RPM_PAIR_Z_SIZES(X) \
-  X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
-
 cudaError_t pass_fwd(const GridDev& g, const float* in, float4* spec, int mode, cudaStream_t st) {
   if (g.nx == 96 && few_planes(g))
     return launch_fwd<96, pair_threads(96, true)>(g, in, spec, mode, st);
   switch (g.nx) {
 #define RPM_CASE(N) case N: return launch_fwd<N, pair_threads(N, false)>(g, in, spec, mode, st);
-    RPM_PAIR_SIZES(RPM_CASE)
+    RPM_PLANE_SIZES(RPM_CASE)
 #undef RPM_CASE
     default: return cudaErrorInvalidValue;
   }
@@ -1560,7 +1557,7 @@ cudaError_t pass_inv(const GridDev& g, float* out, const float4* spec, const flo
     return launch_inv<96, pair_threads(96, true)>(g, out, spec, eps, post, st);
   switch (g.nx) {
 #define RPM_CASE(N) case N: return launch_inv<N, pair_threads(N, false)>(g, out, spec, eps, post, st);
-    RPM_PAIR_SIZES(RPM_CASE)
+    RPM_PLANE_SIZES(RPM_CASE)
 #undef RPM_CASE
     default: return cudaErrorInvalidValue;
   }
@@ -1572,13 +1569,11 @@ cudaError_t pass_green(const GridDev& g, float4* spec, int mode, const double E[
   for (float& v : ga.En) v *= 2.f;   // the spectrum holds 2 X
   switch (g.nz) {
 #define RPM_CASE(N) case N: return launch_green_tile<N>(g, spec, mode, ga, st);
-    RPM_PAIR_Z_SIZES(RPM_CASE)
+    RPM_Z_SIZES(RPM_CASE)
 #undef RPM_CASE
     default: return cudaErrorInvalidValue;
   }
 }
-
-#define RPM_XY_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
 
 cudaError_t pass_rows(const GridDev& g, const float* in, float* out, float4* spec, int mode,
                       bool inv, const float* add, cudaStream_t st) {
@@ -1606,7 +1601,7 @@ bool pair_plane_ok(const GridDev& g, const float2* spec) {
   if (g.nx != g.ny || ((uintptr_t)spec & 15) != 0) return false;   // 16-byte spectrum elements
   switch (g.nx) {
 #define RPM_CASE(N) case N:
-    RPM_PAIR_SIZES(RPM_CASE)
+    RPM_PLANE_SIZES(RPM_CASE)
 #undef RPM_CASE
     return true;
     default: return false;

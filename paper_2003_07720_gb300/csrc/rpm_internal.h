@@ -43,11 +43,18 @@ struct GridDev {
   float lam0, mu0;
   float inv_lx, inv_ly, inv_lz;   // 1 / L_j (frequency scaling)
   int nyquist;           // 0: zero mixed Nyquist frequencies, 1: signed
-  int plane_v;           // x/y passes: 0 paired where available, 1 whole-plane, 2 five-pass
-  int pencil_t;          // z pass: 0 fused where available, else the default tile;
-                         // 1 half, 2 twice the default pencils; 3 the default tile
+  int plane_v;           // x/y passes: 0 paired planes where they fit, 1 scalar whole-plane,
+                         // 2 paired in five passes
+  int pencil_t;          // z pass: 0 the default (of the scalar kernels the fused one where
+                         // available); 1 half, 2 twice the default pencils; 3 the default tile
   int* err;              // device flag set to 1 when a bounded wait of a kernel gave up
 };
+
+// Grid sides with kernels: x and y, z, and square planes that fit in shared memory.
+#define RPM_XY_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
+#define RPM_Z_SIZES(X) \
+  X(1) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(256)
+#define RPM_PLANE_SIZES(X) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128)
 
 struct GammaArgs {
   float En[6];       // E * n_vox (zero frequency of the strain in GM_FULL_MAP)

@@ -301,7 +301,7 @@ def rpm_pencil_tile(ctx) -> int:
 
 
 def rpm_plane_variant(ctx) -> int:
-    """Plane-pass kernels in use: 0 fused, 1 whole-plane, 2 five-pass."""
+    """Plane-pass kernels in use: 0 paired, 1 whole-plane, 2 five-pass."""
     return int(lib().rpm_plane_variant(ctx))
 
 
